@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "esdc_internal.h"
+#include "fix_f64.cuh"
 #include "kernels.h"
 
 namespace {
@@ -758,6 +759,21 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
             c->opsf.D2[i][j].x = c->opsf.D2[i][j].y = (float)hs.D[i * hs.N + j];
         }
     }
+    if (hs.N <= esdc::kMaxN) {
+        for (int i = 0; i < hs.N; ++i) {
+            for (int k = 1; k <= hs.N / 2; ++k)
+                c->ops.SF[k - 1][i] = esdc::fx_split(esdc::fx_from_double(c->ops.S[i][(i + k) % hs.N], 0));
+        }
+        double dmax = 0.0;
+        for (int i = 0; i < hs.N; ++i)
+            for (int j = 0; j < hs.N; ++j) dmax = std::fmax(dmax, std::fabs(c->ops.D[i][j]));
+        std::frexp(dmax, &c->ops.kD);
+        for (int i = 0; i < hs.N; ++i)
+            for (int j = 0; j < hs.N; ++j)
+                c->ops.DF[i][j] = esdc::fx_split(esdc::fx_from_double(c->ops.D[i][j], c->ops.kD));
+        c->ops.LF = esdc::fx_split(esdc::fx_from_double(0.5 * c->ops.winv[0], c->ops.kD));
+    }
+    c->ops.CG = esdc::fx_split(esdc::fx_from_double(std::frexp(1.0 / (s.gamma - 1.0), &c->ops.kg), 0));
     const double R = 1.0 / (s.gamma * s.Ma * s.Ma);
     const double mu = s.Re > 0.0 ? 1.0 / s.Re : 0.0;
     const double cp = s.gamma * R / (s.gamma - 1.0);
@@ -766,6 +782,8 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
     c->phys.mu = mu;
     c->phys.kappa = mu * cp / s.Pr;
     c->phys.inv_gm1 = 1.0 / (s.gamma - 1.0);
+    c->phys.gm1 = s.gamma - 1.0;
+    c->phys.kappa_R = c->phys.kappa / R;
     c->phys.dissipation = s.dissipation;
     c->phys.viscous = mu > 0.0;
     c->phys.ip_coef = mu > 0.0 ? s.ip_coef : 0.0;

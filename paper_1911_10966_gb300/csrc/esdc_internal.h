@@ -13,6 +13,11 @@ namespace esdc {
 constexpr int kMaxN = 8;     // p <= 7: one element per CTA (rhs_f64.cu, rhs_f32.cu, the adjoint)
 constexpr int kLargeN = 16;  // p = 15: the multi-pass float64 residual (rhs_large_f64.cu)
 
+// The two limbs of a fixed-point number (h 2^30 + l) 2^-60.
+struct alignas(8) FxPair {
+    int h, l;
+};
+
 // Per-degree operators passed by value to kernels (lands in the constant bank).
 struct Ops {
     int N;
@@ -21,6 +26,14 @@ struct Ops {
     double S[kMaxN][kMaxN];    // S itself (the pair coefficient of the forward kernels)
     double w[kLargeN];         // LGL weights (diagonal of P), every supported degree
     double winv[kLargeN];      // 1/w
+    // fixed-point forms (fix_f64.cuh): S[i][(i + k) % N] by cyclic distance k = 1..N/2,
+    // 1/(gamma - 1) = CG 2^kg
+    FxPair SF[kMaxN / 2][kMaxN];
+    FxPair CG;
+    int kg;
+    FxPair DF[kMaxN][kMaxN];   // D_ij 2^-kD
+    FxPair LF;                 // interface lift 1/(2 w_0) 2^-kD
+    int kD;
 };
 
 // The same operators for N = kLargeN (the p = 15 residual passes).
@@ -35,6 +48,7 @@ struct OpsL {
 struct Phys {
     double gamma, R, mu, kappa;
     double inv_gm1;            // 1/(gamma-1)
+    double gm1, kappa_R;       // gamma - 1, kappa/R
     double ip_coef;            // interior-penalty coefficient (0: off)
     int dissipation;           // 0 none, 1 local Lax-Friedrichs, 2 matrix
     int viscous;               // mu > 0

@@ -1,0 +1,413 @@
+// Block fixed-point arithmetic of the float64 element kernels.
+//
+// Why: this part issues one float64 instruction per 64 clocks and scheduler (2 lanes per clock and
+// SM), against 16 lanes per clock and scheduler for 32-bit integer adds, shifts and logic and 8 to 11
+// for 32 x 32 -> 64 multiply-adds.  A product of two 60-bit fixed-point numbers is three of those
+// multiply-adds and two shifts, an addition two integer adds, so a pair flux that keeps the float64
+// pipe busy for ~900 clocks per warp and SM takes ~120 on the integer pipes, with seven more bits in
+// every intermediate than a float64 significand has.
+//
+// Format: a value v with |v| < 2 is the pair (h, l), v = (h 2^30 + l) 2^-60 ("Q60"): h signed, l a
+// 30-bit limb, or the sum of two (so an addition needs no carry).  What a Q60 number stands for is
+// v 2^k with an exponent k that is the same for a whole element: the inputs are scaled by the largest
+// exponent of their kind in the element, and every intermediate's exponent follows from theirs.  An
+// element whose density or beta spans more than kMaxSpread binary exponents, or whose state is not
+// finite and positive, is evaluated in float64 instead (fix_range_ok).
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+#include <cuda_runtime.h>
+
+#include "esdc_internal.h"
+
+namespace esdc {
+
+#define ESDC_HD __host__ __device__ __forceinline__
+
+constexpr int kMaxSpread = 3;                  // exponent spread of density and of beta within an element
+
+using Fx = FxPair;
+
+ESDC_HD Fx fx_split(long long v) { return {(int)(v >> 30), (int)v & 0x3fffffff}; }
+
+ESDC_HD Fx fx_add(Fx a, Fx b) { return {a.h + b.h, a.l + b.l}; }
+ESDC_HD Fx fx_sub(Fx a, Fx b) { return {a.h - b.h, a.l - b.l}; }
+
+// 32 x 32 -> 64 signed products as single instructions: a limb is known not to be negative, and a
+// product of a signed and an unsigned 32-bit value is otherwise compiled as a general 64-bit one
+ESDC_HD long long mul_wide(int a, int b) {
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+#else
+    return (long long)a * b;
+#endif
+}
+ESDC_HD long long mad_wide(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+#else
+    return (long long)a * b + c;
+#endif
+}
+
+// Rounding of a product's limb sum before its alignment shift: half a unit, plus the mean of the low
+// limbs' product, which is left out: a quarter of a unit (2^28 here) per product of two normalised
+// operands, twice that for each operand that is a sum of two, nothing if one is a difference (LL, in
+// quarter units).  A constant bias of the fluxes would not cancel in the flux differences of an
+// element's end nodes.
+constexpr long long kFxHalf = 1 << 29, kFxLow = 1 << 28;
+
+ESDC_HD long long fx_join(Fx a) { return mad_wide(a.h, 1 << 30, (long long)a.l); }
+
+// a b in Q60 to within a unit
+template <int LL = 1>
+ESDC_HD long long fx_mul(Fx a, Fx b) {
+    const long long t = mad_wide(a.l, b.h, mad_wide(a.h, b.l, kFxHalf + LL * kFxLow));
+    return mad_wide(a.h, b.h, t >> 30);
+}
+// a b + c d with one shared alignment shift
+template <int LL = 2>
+ESDC_HD long long fx_mul2(Fx a, Fx b, Fx c, Fx d) {
+    long long t = mad_wide(a.l, b.h, mad_wide(a.h, b.l, kFxHalf + LL * kFxLow));
+    t = mad_wide(c.l, d.h, mad_wide(c.h, d.l, t));
+    return mad_wide(a.h, b.h, mad_wide(c.h, d.h, t >> 30));
+}
+// one more product added to the limb sums (hi, mid) of a dot product; fx_dot_end closes it
+ESDC_HD void fx_mac(long long& hi, long long& mid, Fx a, Fx b) {
+    hi = mad_wide(a.h, b.h, hi);
+    mid = mad_wide(a.l, b.h, mad_wide(a.h, b.l, mid));
+}
+
+// a b + c d + e f
+template <int LL = 3>
+ESDC_HD long long fx_dot(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f) {
+    long long mid = mad_wide(a.l, b.h, mad_wide(a.h, b.l, kFxHalf + LL * kFxLow));
+    mid = mad_wide(c.l, d.h, mad_wide(c.h, d.l, mid));
+    mid = mad_wide(e.l, f.h, mad_wide(e.h, f.l, mid));
+    return mad_wide(a.h, b.h, mad_wide(c.h, d.h, mad_wide(e.h, f.h, mid >> 30)));
+}
+
+ESDC_HD unsigned mul_hi_u32(unsigned a, unsigned b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (unsigned)(((unsigned long long)a * b) >> 32);
+#endif
+}
+
+ESDC_HD float rcp_seed(float x) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+ESDC_HD int double_hi(double x) {
+#ifdef __CUDA_ARCH__
+    return __double2hiint(x);
+#else
+    int64_t b;
+    memcpy(&b, &x, 8);
+    return (int)(b >> 32);
+#endif
+}
+ESDC_HD long long double_bits(double x) {
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(x);
+#else
+    long long b;
+    memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+ESDC_HD double bits_double(long long b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(b);
+#else
+    double x;
+    memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+// biased exponent of |x| (0 for zeros and subnormals, which the fixed-point form takes as zero)
+ESDC_HD int biased_exp(double x) { return (double_hi(x) >> 20) & 0x7ff; }
+
+// x 2^-k in Q60, truncated toward zero; |x| 2^-k < 2.  With E the largest biased exponent of a block,
+// k = E - 1021 makes every |value| of it < 1/2.
+ESDC_HD long long fx_from_double(double x, int k) {
+    const long long b = double_bits(x);
+    const int E = (int)(b >> 52) & 0x7ff;
+    unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+    // x = m 2^(E - 1075), value = m 2^(E - 1015 - k); m << 10 leaves 63 bits
+    int s = k + 1025 - E;                        // right shift of m << 10
+    s = s > 63 ? 63 : s;
+    long long v = E == 0 ? 0 : (long long)((m << 10) >> s);
+    return b < 0 ? -v : v;
+}
+
+// v 2^(k - 60) as a double, rounded to nearest; 0 below the normal range
+ESDC_HD double fx_to_double(long long v, int k) {
+#ifdef __CUDA_ARCH__
+    const double x = __ll2double_rn(v);
+    const int hi = __double2hiint(x);
+    const int e = ((hi >> 20) & 0x7ff) + k - 60;
+    return e < 1 || v == 0 ? 0.0 : __hiloint2double(hi + ((k - 60) << 20), __double2loint(x));
+#else
+    return __builtin_ldexp((double)v, k - 60);
+#endif
+}
+
+// 1/s 2^-ib in Q60 for 2^-ib <= s < 2 (seed: 2^(60 - ib) as a float).  The hardware's float32
+// approximation of the high limb gives r0 with e = 1 - s r0 ~ 2^-22; r0 (1 + e + e^2) is then exact
+// to the format, the next term being 2^-66.
+ESDC_HD int fx_rcp_seed(Fx s, float seed) {                               // r0 in units of 2^-30
+#ifdef __CUDA_ARCH__
+    return __float2int_rn(rcp_seed((float)s.h) * seed);
+#else
+    return (int)(rcp_seed((float)s.h) * seed + 0.5f);
+#endif
+}
+ESDC_HD long long fx_rcp(Fx s, float seed, int ib) {
+    const int r0 = fx_rcp_seed(s, seed);
+    const long long p = mad_wide(s.h, r0, mul_wide(s.l, r0) >> 30);      // s r0 2^-ib in Q60
+    const long long e = (1ll << 60) - (p << ib);
+    const int eh = (int)(e >> 16);                                       // units of 2^-44
+    const Fx y = fx_split(e + (mul_wide(eh, eh) >> 28));
+    return mad_wide(r0, 1 << 30, mad_wide(r0, y.h, mul_wide(r0, y.l) >> 30));
+}
+
+// Exponents of one element's fixed-point quantities (value = Q60 number * 2^k) and the alignment
+// shifts of the two-point flux; the same for all nodes of the element.
+struct FixScale {
+    int kr, ku, kb, kn, kq;  // half density, half velocity, beta, metric terms, |u|^2/4
+    int ir, ib;              // 1/(sum of half densities) <= 2^ir, 1/(sum of betas) <= 2^ib (in Q60)
+    int k0, km, k5;          // mass, momentum and energy flux
+    int kA;                  // inv_gm1 F / (sum of betas)
+    int sA, sB;              // f1 and p_t into the momentum flux
+    int sc, sq;              // the two parts of the energy coefficient
+    int sC, sD;              // its two products into the energy flux
+    long long hC, hD;        // half a unit of the last two
+    int ky, kz;              // mu RT/J and (kappa/R) RT^2/J
+    float fr, fb;            // 2^(60 - ir), 2^(60 - ib): the reciprocals' seeds
+};
+
+ESDC_HD float pow2f(int e) {      // 2^e, -126 <= e <= 127
+    const int b = (e + 127) << 23;
+#ifdef __CUDA_ARCH__
+    return __int_as_float(b);
+#else
+    float f;
+    memcpy(&f, &b, 4);
+    return f;
+#endif
+}
+ESDC_HD int fx_max(int a, int b) { return a > b ? a : b; }
+ESDC_HD int fx_clamp(int a) { return a > 62 ? 62 : a; }
+
+// Er, Eu, Eb, En: largest biased exponents of the half density, half velocity, beta and metric terms;
+// Er0, Eb0: smallest of half density and beta.  kg: exponent of inv_gm1 = c 2^kg, 1/2 <= c < 1.
+// Bounds in Q60: densities and betas < 1/2, velocities and metrics < 1/4 (so that the twelve limb
+// products of a three-term dot product stay inside 64 bits), |u|^2/4 < 3/8, ubar.n < 3/4 and kept doubled,
+// mass flux < 3/2, p_t <= 1, momentum flux < 5/4 (7/8 if the pressure part sets its exponent), energy
+// coefficient < 1.01, energy flux < 2.2.  All but p_t and the coefficient carry a factor S_ij (or 1 on a
+// face), |S_ij| with row sums below 3.41, so their sums over a line stay inside 63 bits.
+// Ey, Ez: largest exponents of mu RT/J and kappa/R RT^2/J.
+ESDC_HD FixScale fix_scale(int Er, int Er0, int Eu, int Eb, int Eb0, int En, int Ey, int Ez, int kg) {
+    FixScale s;
+    s.kr = Er - 1021;
+    s.ku = Eu - 1020;
+    s.kb = Eb - 1021;
+    s.kn = En - 1020;
+    s.kq = 2 * s.ku - 1;
+    s.ir = Er - Er0 + 1;
+    s.ib = Eb - Eb0 + 1;
+    s.fr = pow2f(60 - s.ir);
+    s.fb = pow2f(60 - s.ib);
+    s.k0 = s.kr + s.ku + s.kn - 1;
+    const int ka = s.k0 + s.ku, kb = s.kr + s.ib - s.kb + s.kn;
+    s.km = fx_max(ka, kb);
+    s.sA = fx_clamp(s.km - ka);
+    s.sB = fx_clamp(s.km - kb);
+    s.kA = kg + s.ib - s.kb;
+    const int kc = fx_max(s.kA, s.kq);
+    s.sc = fx_clamp(kc - s.kA);
+    s.sq = fx_clamp(kc - s.kq);
+    const int kC = s.k0 + kc, kM = s.ku + s.km;
+    s.k5 = kC - kM >= (kb > ka ? 1 : 2) ? kC : fx_max(kC, kM) + 1;
+    s.sC = fx_clamp(s.k5 - kC);
+    s.sD = fx_clamp(s.k5 - kM);
+    s.hC = (1ll << s.sC) >> 1;
+    s.hD = (1ll << s.sD) >> 1;
+    s.ky = Ey - 1021;
+    s.kz = Ez - 1021;
+    return s;
+}
+
+// The viscous chain's exponents, known once theta is: w2..w4 = 2 beta u < 1/2 in units 2^(kb + ku), w5 =
+// -2 beta as beta itself; operator entries D_ij 2^-kD with row sums below 1.7, so theta (with its lift)
+// < 1.25, or < 1 once shifted left by sw (w2..w4) and sb (w5).  Then the contraction with the metric
+// < 0.94, velocity gradients A < 1.2, a quarter of their symmetric combination < 1.2 in the stress,
+// stress < 0.6, energy flux < 0.92, contravariant fluxes < 0.7.
+struct ViscScale {
+    int ky, kz;              // mu RT/J and (kappa/R) RT^2/J
+    int sg, su;              // the two parts of the velocity gradients
+    int kf, kh;              // contravariant viscous fluxes: momentum, energy
+    int se, sz;              // stress work and heat flux into the energy part
+    long long he, hz;        // half a unit of the two
+};
+ESDC_HD ViscScale visc_scale(const FixScale& f, int sw, int sb, int kD) {
+    ViscScale s;
+    s.ky = f.ky;
+    s.kz = f.kz;
+    const int kg = f.kn + f.kb + f.ku + kD - sw, kb = f.kn + f.kb + 1 + kD - sb;     // contracted w2..w4, w5
+    const int ku = kb + f.ku + 1, ka = fx_max(kg, ku);
+    s.sg = fx_clamp(ka - kg);
+    s.su = fx_clamp(ka - ku);
+    const int kt = ka + 2 + s.ky;
+    const int ke = kt + f.ku + 1, kq = s.kz + kb;
+    const int kh = fx_max(ke, kq);
+    s.se = fx_clamp(kh - ke);
+    s.sz = fx_clamp(kh - kq);
+    s.he = (1ll << s.se) >> 1;
+    s.hz = (1ll << s.sz) >> 1;
+    s.kf = f.kn + kt;
+    s.kh = f.kn + kh;
+    return s;
+}
+
+// Whether an element is in range: positive, finite and normal density and beta within the spread,
+// finite velocities and metrics, and exponents that keep every derived one inside float64's.
+ESDC_HD bool fix_range_ok(int Er, int Er0, int Eu, int Eb, int Eb0, int En) {
+    return Er - Er0 <= kMaxSpread && Eb - Eb0 <= kMaxSpread && Er0 > 895 && Er < 1151 && Eb0 > 895 && Eb < 1151 &&
+           Eu < 1151 && En < 1151;
+}
+
+// Per-node inputs of the pair loop, Q60 limbs: half density, half velocity, beta, |u|^2/4.
+struct PrimFx {
+    Fx r, u0, u1, u2, b, q;
+};
+
+// Series of the logarithmic means in u = f^2, f = (a - b)/(a + b):
+//   artanh(f)/f = F(u) = sum u^k/(2k+1)      and      1/F(u) = G(u) = 1 - sum g_k u^k
+// (g_k by inverting the first series term by term: 1/3, 4/45, 44/945, 428/14175, ...).  Both are
+// 1 +- u P(u), and u P(u) in Q60 is what these return.  Terms are kept until their weight at the end of
+// the range is below 2^-58.
+
+// u < 2^-13 (neighbours within 2%): P = c1 + u c2 + u^2 c3, of which 32 bits beyond c1 reach 2^-58
+template <bool LOGF>
+ESDC_HD long long fx_series_near(long long u) {
+    constexpr Fx D1 = {357913941, 357913941};                        // 1/3
+    constexpr unsigned c2 = LOGF ? 858993459u : 381774871u;          // 1/5 or 4/45, units of 2^-32
+    constexpr unsigned c3 = LOGF ? 613566757u : 199977313u;          // 1/7 or 44/945
+    const unsigned us = (unsigned)(u >> 15);                         // units of 2^-45
+    const unsigned t = mul_hi_u32(us, c2 + (mul_hi_u32(us, c3) >> 13));
+    return fx_mul(fx_split(u), Fx{D1.h + (int)(t >> 15), D1.l + (int)((t & 0x7fffu) << 15)});
+}
+
+// u < 2^-6 (within 28%): Horner, the terms of weight u^4 and beyond in 32 bits; u' = 2^6 u
+template <bool LOGF>
+ESDC_HD long long fx_series_far(long long u) {
+    constexpr unsigned C4 = LOGF ? 477218588u : 129682258u;          // 1/9           428/14175
+    constexpr unsigned C5 = LOGF ? 390451572u : 93616560u;           // 1/11          10196/467775
+    constexpr unsigned C6 = LOGF ? 330382100u : 72101986u;           // 1/13          10719068/638512875
+    constexpr unsigned C7 = LOGF ? 286331153u : 57993934u;           // 1/15          25865068/1915538625
+    constexpr unsigned C8 = LOGF ? 252645135u : 48119721u;           // 1/17          5472607916/488462349375
+    constexpr unsigned C9 = LOGF ? 226050910u : 40871223u;           // 1/19          74185965772/7795859096025
+    constexpr Fx D1 = {357913941, 357913941};
+    constexpr Fx D2 = LOGF ? Fx{214748364, 858993459} : Fx{95443717, 739688812};
+    constexpr Fx D3 = LOGF ? Fx{153391689, 153391689} : Fx{49994328, 336325481};
+    const unsigned us = (unsigned)(u >> 22);                         // u' in units of 2^-32
+    unsigned t = C9;
+    t = C8 + (mul_hi_u32(us, t) >> 6);
+    t = C7 + (mul_hi_u32(us, t) >> 6);
+    t = C6 + (mul_hi_u32(us, t) >> 6);
+    t = C5 + (mul_hi_u32(us, t) >> 6);
+    t = mul_hi_u32(us, t);
+    const unsigned long long p4 = ((unsigned long long)C4 << 28) + ((unsigned long long)t << 22);
+    const Fx uf = fx_split(u << 6);
+    long long v = fx_mul(uf, fx_split((long long)p4)) >> 6;
+    v = fx_mul(uf, Fx{D3.h + (int)(v >> 30), D3.l + ((int)v & 0x3fffffff)}) >> 6;
+    v = fx_mul(uf, Fx{D2.h + (int)(v >> 30), D2.l + ((int)v & 0x3fffffff)}) >> 6;
+    return fx_mul(uf, Fx{D1.h + (int)(v >> 30), D1.l + ((int)v & 0x3fffffff)}) >> 6;
+}
+
+constexpr long long kFxSeriesEnd = 1ll << 54;     // u = 2^-6
+constexpr int kFxNear = 2965790;                  // high word of f = 2^-6.5 in Q60, less a part in 10^5
+
+// Logarithmic means of neighbours further apart than the near series: rl in Q60 2^kr, A in Q60 2^kA.
+// Rare in a resolved flow, so it starts over from the inputs.
+template <typename LogMean>
+ESDC_HD void log_means_far(Fx sh, Fx dh, Fx db, Fx rs, Fx g, const FixScale& s, const LogMean& lm, long long& rl,
+                           long long& A) {
+    const Fx fr = fx_split(fx_mul<0>(dh, fx_split(fx_rcp(sh, s.fr, s.ir))) << s.ir);
+    const long long ur = mad_wide(fr.h, fr.h, mul_wide(fr.h, fr.l) >> 29);
+    rl = ur < kFxSeriesEnd ? fx_join(sh) - fx_mul<2>(sh, fx_split(fx_series_far<false>(ur))) : lm.rho();
+    const Fx fb = fx_split(fx_mul<0>(db, rs) << s.ib);
+    const long long ub = mad_wide(fb.h, fb.h, mul_wide(fb.h, fb.l) >> 29);
+    A = ub < kFxSeriesEnd ? fx_join(g) + fx_mul(g, fx_split(fx_series_far<true>(ub))) : lm.inv_beta();
+}
+
+// The Chandrashekar flux of flux_f64.cuh (ec_flux) in block fixed point, contracted with n: f[0] in
+// units 2^k0, f[1..3] 2^km, f[4] 2^k5.  cg: inv_gm1 2^-kg.  LogMean supplies the logarithmic means where
+// u is beyond the series: rho_ln in Q60 2^kr and inv_gm1 / beta_ln in Q60 2^kA.  The near series is
+// evaluated without a branch, so that the two means, ubar.n and the reciprocals interleave.
+template <typename LogMean>
+ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, Fx cg, const FixScale& s,
+                        const LogMean& lm, long long f[5]) {
+    // log mean of the density: sh G(u), u = f^2.  f = d/sh from a 2^-22 reciprocal r0 and one correction:
+    // relative error 2^-44, which u P(u) < 2^-14 leaves below 2^-57
+    const Fx sh = fx_add(a.r, b.r), dh = fx_sub(a.r, b.r);
+    long long rl, fh;
+    {
+        const int r0 = fx_rcp_seed(sh, s.fr);
+        const long long p = mad_wide(sh.h, r0, mul_wide(sh.l, r0) >> 30);
+        const int e = (int)(((1ll << 60) - (p << s.ir)) >> 16);          // units of 2^-44
+        const long long f0 = mad_wide(dh.h, r0, mul_wide(dh.l, r0) >> 30) << s.ir;
+        fh = f0;
+        const Fx ff = fx_split(f0 + (mul_wide((int)(f0 >> 24), e) >> 20));
+        const long long u = mad_wide(ff.h, ff.h, mul_wide(ff.h, ff.l) >> 29);
+        rl = fx_join(sh) - fx_mul<2>(sh, fx_split(fx_series_near<false>(u)));
+    }
+    // 1/(sum of betas), and inv_gm1/beta_ln = inv_gm1 rsb F(u)
+    const Fx sb = fx_add(a.b, b.b), db = fx_sub(a.b, b.b);
+    const Fx rs = fx_split(fx_rcp(sb, s.fb, s.ib));
+    const Fx g = fx_split(fx_mul(rs, cg));
+    const long long fb = fx_mul<0>(db, rs) << s.ib;
+    long long A;
+    {
+        const Fx ff = fx_split(fb);
+        const long long u = mad_wide(ff.h, ff.h, mul_wide(ff.h, ff.l) >> 29);
+        A = fx_join(g) + fx_mul(g, fx_split(fx_series_near<true>(u)));
+    }
+    const int ir = (int)(fh >> 32), ib = (int)(fb >> 32);
+    if ((unsigned)(ir + kFxNear) >= 2u * kFxNear || (unsigned)(ib + kFxNear) >= 2u * kFxNear)
+        log_means_far(sh, dh, db, rs, g, s, lm, rl, A);
+    const Fx rlf = fx_split(rl);
+    const Fx v0 = fx_add(a.u0, b.u0), v1 = fx_add(a.u1, b.u1), v2 = fx_add(a.u2, b.u2);
+    long long mid = mad_wide(v0.l, n0.h, mad_wide(v0.h, n0.l, (kFxHalf >> 1) + 6 * kFxLow));
+    mid = mad_wide(v1.l, n1.h, mad_wide(v1.h, n1.l, mid));
+    mid = mad_wide(v2.l, n2.h, mad_wide(v2.h, n2.l, mid));
+    const long long hh = mad_wide(v0.h, n0.h, mad_wide(v1.h, n1.h, mul_wide(v2.h, n2.h)));
+    const Fx un = fx_split((hh << 1) + (mid >> 29));
+    const long long f1 = fx_mul(rlf, un);
+    const long long pt = fx_mul<2>(sh, rs);
+    const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(pt >> s.sB);
+    f[0] = f1;
+    f[1] = fx_mul2<3>(fa, v0, pa, n0);
+    f[2] = fx_mul2<3>(fa, v1, pa, n1);
+    f[3] = fx_mul2<3>(fa, v2, pa, n2);
+    const Fx c5 = fx_split((A >> s.sc) - (fx_join(fx_add(a.q, b.q)) >> s.sq));
+    const Fx m0 = fx_split(f[1]), m1 = fx_split(f[2]), m2 = fx_split(f[3]);
+    f[4] = ((fx_mul(fx_split(f1), c5) + s.hC) >> s.sC) + ((fx_dot<6>(v0, m0, v1, m1, v2, m2) + s.hD) >> s.sD);
+}
+
+}  // namespace esdc

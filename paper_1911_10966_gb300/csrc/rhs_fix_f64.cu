@@ -1,0 +1,655 @@
+// ES-C residual of the float64 form in block fixed point (fix_f64.cuh): flux differencing with the
+// Chandrashekar flux (eq. discEL), the entropy-stable interface SAT, BR1 entropy-variable gradients,
+// viscous fluxes and their divergence (eq. MacroForm, eq. NSL) for p <= 7.
+//
+// One element per group of N^3 threads (EPB elements per CTA).  Float64 is kept where it is needed or
+// cheap: primitives of own and neighbour states, the dissipation of the interface term, the sum of the
+// directions' results, the scaling by 1/J and everything in global memory.  Phases:
+//   0. primitives of the nodes and of the neighbours' face nodes; the element's largest and smallest
+//      exponents; everything scaled to Q60 limbs in shared memory.  An element out of the fixed-point
+//      range sends its CTA to the float64 form (element_f64.cuh).
+//   1. volume: one thread per (node, direction), whole lines side by side in a warp.  At cyclic distance
+//      k = 1..N/2 the thread of node i evaluates the pair (i, i + k mod N), so that each pair is
+//      evaluated once; S_ij f is summed in registers on one side and by a shuffle on the other.
+//   2. interface: one thread per face node; two-point flux in fixed point, dissipation in float64.
+//   3. viscous: lines of w for theta_a = D_a w + lift (one thread per line and variable, the operator
+//      from the constant bank), one thread per node for the fluxes, lines again for the divergence.
+//
+// Bound: multiply (8 lanes per clock and scheduler for a 32 x 32 -> 64 product) and shift/logic (16) pipes
+// in phases 1 and 3, the float64 pipe (half a lane) in 0 and 2.  Against the all-float64 kernel, which
+// kept the float64 pipe 87% busy, per viscous residual of the Taylor-Green flow: 8.59 -> 2.86 ms at p = 7
+// on 20^3 elements, 0.92 -> 0.31 ms at p = 4 on 16^3, 2.58 -> 1.02 ms at p = 2 on 41 x 37 x 39.  Its error
+// against extended precision is smaller in every variable and degree tried.
+#include <cuda_runtime.h>
+
+#include "element_f64.cuh"
+#include "esdc_internal.h"
+#include "fix_f64.cuh"
+#include "kernels.h"
+#include "visc_sat.cuh"
+
+namespace esdc {
+namespace {
+
+template <int N>
+struct FixCfg {
+    static constexpr int N2 = N * N, N3 = N * N * N;
+    static constexpr int EPB = Cfg<N>::EPB;
+    static constexpr int THREADS = (EPB * N3 + 31) / 32 * 32;    // whole warps (the pair loop's shuffles)
+    static constexpr int WARPS = THREADS / 32;
+    static constexpr int MINB = N >= 7 ? 1 : (N == 6 ? 2 : 4);
+    // pair loop: LPW whole lines per warp, TPD warp tasks per direction
+    static constexpr int LPW = 32 / N, TPD = (EPB * N2 + LPW - 1) / LPW;
+    // node slots of the limb arrays: rows of S2, layers of S3 (see slot)
+    static constexpr bool PAD = N == 4 || N == 6;
+    static constexpr int S2 = PAD ? N + 1 : N, S3 = N * S2 + (PAD ? 1 : 0), SL = N * S3;
+    // shared memory per element in 8-byte units
+    static constexpr int XN = 0;                 // [9][SL] metric rows; later the viscous fluxes' momentum part
+    static constexpr int XP = 9 * SL;            // [6][SL] half density, half velocity, beta, |u|^2/4; later
+                                                 //         [3][SL] the viscous fluxes' energy part
+    static constexpr int XW = 15 * SL;           // [3][SL] w2..w4 = 2 beta u
+    static constexpr int R = 18 * SL;            // [3][5][N3] results per direction (float64); then [12][SL] theta
+    static constexpr int P = 33 * SL;            // [4][N3] float64 half velocity and RT
+    static constexpr int F = P + 4 * N3;         // [7][6 N2] neighbour face nodes: six primitives, sound speed
+    static constexpr int SM = F + 42 * N2;
+};
+
+// Slot of node (i1, i2, i3) in the limb arrays.  A half-warp of 64-bit loads covers two lines of eight
+// nodes at N = 8: the XOR spreads every direction's over all banks without padding; N = 4 and 6 take
+// odd row strides; odd N needs nothing.
+template <int N>
+__device__ __forceinline__ int slot(int i1, int i2, int i3) {
+    if constexpr (N == 8) return (i1 ^ (2 * ((i2 >> 1) ^ (i3 >> 1)))) + 8 * (i2 ^ (i3 & 1)) + 64 * i3;
+    else return i1 + FixCfg<N>::S2 * i2 + FixCfg<N>::S3 * i3;
+}
+// node i of line (c1, c2) of direction l
+template <int N>
+__device__ __forceinline__ int line_slot(int l, int i, int c1, int c2) {
+    return l == 0 ? slot<N>(i, c1, c2) : (l == 1 ? slot<N>(c1, i, c2) : slot<N>(c1, c2, i));
+}
+
+// Element-wide maxima of NV non-negative integers into out (shared memory, zeroed), by the threads of
+// active elements; a warp (or an 8-lane group at N = 2) inside one element reduces first.
+template <int N, int NV>
+__device__ __forceinline__ void block_max(int* out, int (&v)[NV], int lane) {
+    constexpr bool warp_el = FixCfg<N>::EPB == 1 || FixCfg<N>::N3 % 32 == 0;
+    if constexpr (warp_el || N == 2) {
+        const unsigned mask = warp_el ? __activemask() : 0xffu << (lane & 24);
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = __reduce_max_sync(mask, v[i]);
+        if (lane == __ffs(mask) - 1)
+#pragma unroll
+            for (int i = 0; i < NV; ++i) atomicMax(out + i, v[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) atomicMax(out + i, v[i]);
+    }
+}
+
+// Logarithmic means beyond the series of ec_flux_fx, in float64 from the fixed-point inputs.
+__device__ __noinline__ long long log_mean_f64(long long a, long long b, int k, double num, int kout) {
+    const double x = fx_to_double(a, k), y = fx_to_double(b, k), lg = log(x / y);
+    return fx_from_double(num > 0.0 ? 0.5 * num * lg / (x - y) : 2.0 * (x - y) / lg, kout);
+}
+struct LogMeanF64 {
+    Fx ra, rb, ba, bb;
+    const FixScale& s;
+    double inv_gm1;
+    __device__ __forceinline__ long long rho() const { return log_mean_f64(fx_join(ra), fx_join(rb), s.kr, 0.0, s.kr); }
+    __device__ __forceinline__ long long inv_beta() const {
+        return log_mean_f64(fx_join(ba), fx_join(bb), s.kb, inv_gm1, s.kA);
+    }
+};
+
+// Primitives as in to_prim, with the float64 operations that can go to the integer pipe there: halving
+// is an exponent decrement (zeros, infinities and NaNs end up out of the fixed-point range), and the
+// reciprocals take r (1 + e + e^2), e = 1 - x r, from the 2^-23 approximation r.
+__device__ __forceinline__ double rcp_cubic(double x) {
+    const double r = rcp_approx(x), e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double half_of(double x) { return __hiloint2double(__double2hiint(x) - (1 << 20), __double2loint(x)); }
+__device__ __forceinline__ void to_prim_fx(const double* q, const Phys& ph, Prim& s, double& RT) {
+    const double ri = rcp_cubic(q[0]), rh = half_of(ri);
+    s.hu0 = q[1] * rh;
+    s.hu1 = q[2] * rh;
+    s.hu2 = q[3] * rh;
+    s.qq = fma(s.hu2, s.hu2, fma(s.hu1, s.hu1, s.hu0 * s.hu0));
+    const double p = ph.gm1 * fma(-2.0 * q[0], s.qq, q[4]);
+    s.hr = half_of(q[0]);
+    s.beta = s.hr * rcp_cubic(p);
+    RT = p * ri;
+}
+// sqrt of a positive normal x: Goldschmidt's iteration (one step to 2^-44) and a correction from the residual
+__device__ __forceinline__ double sqrt_newton(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = x * y, h = 0.5 * y;
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(h, fma(-g, g, x), g);
+}
+
+// the element of a CTA left to the float64 form; out of line, so that the kernel's registers are its own
+template <int N, bool XF>
+__device__ __noinline__ void out_of_range(double* smem, const double* q, double* dqdt, const double* geom,
+                                          const int32_t* nbr, double* trace, int64_t K, const Ops& ops, const Phys& ph,
+                                          const double* qext, const double* src, const double* nsurf,
+                                          const double* fnorm) {
+    element_f64<N, kFluxESC, XF>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+}
+
+// Derivatives along one line of N Q60 values: out_i = sum_j D_ij in_j 2^-kD, plus at the ends
+// lo, hi (the interface lift).
+template <int N>
+__device__ __forceinline__ void line_derivative(const Fx (&v)[N], const Ops& ops, long long lo, long long hi,
+                                                long long (&out)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        long long h = 0, m = kFxHalf + N * kFxLow;
+#pragma unroll
+        for (int j = 0; j < N; ++j) fx_mac(h, m, ops.DF[i][j], v[j]);
+        h += m >> 30;
+        if (i == 0) h += lo;
+        if (i == N - 1) h += hi;
+        out[i] = h;
+    }
+}
+
+// XF: the kernel also handles the matrix dissipation, the interior penalty, boundary faces with an
+// exterior state, a source term and surface metrics (compiled only into the instantiations of contexts
+// that use them)
+template <int N, bool XF>
+__global__ void __launch_bounds__(FixCfg<N>::THREADS, FixCfg<N>::MINB)
+rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
+            const double* __restrict__ jinv, const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K,
+            const __grid_constant__ Ops ops, const __grid_constant__ Phys ph, const double* __restrict__ qext,
+            const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
+    using C = FixCfg<N>;
+    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL;
+    extern __shared__ double smem[];
+    __shared__ int sE[EPB][8];                   // largest exponents (of 4096 - E for the smallest)
+    __shared__ FixScale sScale[EPB];
+    __shared__ unsigned sMag[EPB][2];            // magnitude bits of theta: w2..w4, w5
+    __shared__ Fx sS[(N / 2) * N];
+    __shared__ double sW[N];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int el_loc = t / N3;
+    const int node = t - el_loc * N3;
+    const int64_t el = (int64_t)blockIdx.x * EPB + el_loc;
+    const bool active = el_loc < EPB && el < K;
+    const int n_el = (int)(K - (int64_t)blockIdx.x * EPB < EPB ? K - (int64_t)blockIdx.x * EPB : EPB);
+    const int i1 = node % N, i2 = (node / N) % N, i3 = node / N2;
+    double* sm = smem + (size_t)el_loc * C::SM;
+    Fx* X = reinterpret_cast<Fx*>(sm);
+    const int own_slot = slot<N>(i1, i2, i3);
+    const int64_t eoff = el * 5 * N3;
+    for (int i = t; i < EPB * 8; i += C::THREADS) sE[i / 8][i % 8] = 0;
+    if (t < EPB) sMag[t][0] = sMag[t][1] = 0;
+    for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
+    for (int i = t; i < N; i += C::THREADS) sW[i] = ops.winv[i];
+    __syncthreads();
+
+    // ---- 0. primitives, exponents, scaling
+    double Jinv = 0.0, Y = 0.0, Z = 0.0;
+    if (active) {
+        double qv[5], RT;
+        Prim s;
+#pragma unroll
+        for (int v = 0; v < 5; ++v) qv[v] = q[eoff + v * N3 + node];
+        Jinv = jinv[el * N3 + node];
+        int E[8];
+        E[5] = 0;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            const double g = geom[(el * 10 + 1 + c) * N3 + node];
+            sm[C::XN + c * SL + own_slot] = g;
+            E[5] = max(E[5], biased_exp(g));
+        }
+        to_prim_fx(qv, ph, s, RT);
+        sm[C::XP + own_slot] = s.hr;
+        sm[C::XP + SL + own_slot] = s.hu0;
+        sm[C::XP + 2 * SL + own_slot] = s.hu1;
+        sm[C::XP + 3 * SL + own_slot] = s.hu2;
+        sm[C::XP + 4 * SL + own_slot] = s.beta;
+        sm[C::XP + 5 * SL + own_slot] = s.qq;
+        sm[C::P + node] = s.hu0;
+        sm[C::P + N3 + node] = s.hu1;
+        sm[C::P + 2 * N3 + node] = s.hu2;
+        sm[C::P + 3 * N3 + node] = RT;
+        // a sign bit counts as out of range (density and beta must be positive)
+        E[0] = (unsigned)double_hi(s.hr) >> 20;
+        E[1] = 4096 - E[0];
+        E[2] = max(biased_exp(s.hu0), max(biased_exp(s.hu1), biased_exp(s.hu2)));
+        E[3] = (unsigned)double_hi(s.beta) >> 20;
+        E[4] = 4096 - E[3];
+        Y = ph.mu * RT * Jinv;                   // velocity gradient to stress
+        Z = ph.kappa_R * RT * RT * Jinv;         // dw5 to heat flux
+        E[6] = biased_exp(Y);
+        E[7] = biased_exp(Z);
+        for (int fn = node; fn < 6 * N2; fn += N3) {
+            const int l = fn / (2 * N2);
+            const int rem = fn - l * 2 * N2;
+            const int side = rem / N2, fi = rem - side * N2;
+            const int st = dir_stride<N>(l);
+            const int base = line_base<N>(l, fi % N, fi / N);
+            const int64_t nb = nbr[el * 6 + 2 * l + side];
+            const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
+            // a boundary face (neighbour -1, bounded boxes only) sees the exterior state at its own nodes
+            if constexpr (XF) {
+                if (nb < 0) qn = qext + eoff + base + (side ? (N - 1) * st : 0);
+                if (nsurf) {
+                    const double* ns = nsurf + (el * 6 + 2 * l + side) * 3 * N2 + fi;
+                    E[5] = max(max(E[5], biased_exp(ns[0])), max(biased_exp(ns[N2]), biased_exp(ns[2 * N2])));
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
+            to_prim_fx(qv, ph, s, RT);
+            double* f = sm + C::F + fn;
+            f[0] = s.hr;
+            f[6 * N2] = s.hu0;
+            f[12 * N2] = s.hu1;
+            f[18 * N2] = s.hu2;
+            f[24 * N2] = s.beta;
+            f[30 * N2] = s.qq;
+            f[36 * N2] = sqrt_newton(ph.gamma * RT);
+            const int er = (unsigned)double_hi(s.hr) >> 20, eb = (unsigned)double_hi(s.beta) >> 20;
+            E[0] = max(E[0], er);
+            E[1] = max(E[1], 4096 - er);
+            E[2] = max(E[2], max(biased_exp(s.hu0), max(biased_exp(s.hu1), biased_exp(s.hu2))));
+            E[3] = max(E[3], eb);
+            E[4] = max(E[4], 4096 - eb);
+        }
+        block_max<N, 8>(sE[el_loc], E, lane);
+    }
+    __syncthreads();
+    bool ok = true;
+    for (int e = 0; e < n_el; ++e) {
+        const int* E = sE[e];
+        ok = ok && fix_range_ok(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5]) && E[6] < 1151 && E[7] < 1151;
+    }
+    if (!ok) {
+        __syncthreads();
+        out_of_range<N, XF>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+        return;
+    }
+    if (active) {
+        const int* E = sE[el_loc];
+        const FixScale s = fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], ops.kg);
+        if (node == 0) sScale[el_loc] = s;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            const int i = C::XN + c * SL + own_slot;
+            X[i] = fx_split(fx_from_double(sm[i], s.kn));
+        }
+        Fx* XP = X + C::XP + own_slot;
+        const double* sp = sm + C::XP + own_slot;
+        XP[0] = fx_split(fx_from_double(sp[0], s.kr));
+        const Fx b = fx_split(fx_from_double(sp[4 * SL], s.kb));
+        XP[4 * SL] = b;
+        XP[5 * SL] = fx_split(fx_from_double(sp[5 * SL], s.kq));
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const Fx u = fx_split(fx_from_double(sp[(1 + m) * SL], s.ku));
+            XP[(1 + m) * SL] = u;
+            X[C::XW + m * SL + own_slot] = fx_split(fx_mul(b, u) * 4);     // w = 2 beta u in units 2^(kb + ku)
+        }
+        for (int fn = node; fn < 6 * N2; fn += N3) {
+            const double* f = sm + C::F + fn;
+            Fx* g = X + C::F + fn;
+            g[0] = fx_split(fx_from_double(f[0], s.kr));
+#pragma unroll
+            for (int m = 0; m < 3; ++m) g[(1 + m) * 6 * N2] = fx_split(fx_from_double(f[(1 + m) * 6 * N2], s.ku));
+            g[24 * N2] = fx_split(fx_from_double(f[24 * N2], s.kb));
+            g[30 * N2] = fx_split(fx_from_double(f[30 * N2], s.kq));
+        }
+    }
+    __syncthreads();
+
+    // ---- 1. volume flux differencing
+    {
+        const int lw = lane / N, i = lane - lw * N;
+#pragma unroll 1
+        for (int task = warp; task < 3 * C::TPD; task += C::WARPS) {
+            const int l = task / C::TPD;
+            int line = (task - l * C::TPD) * C::LPW + lw;
+            const bool go = lw < C::LPW && line < n_el * N2;
+            line = go ? line : 0;
+            const int e = line / N2, li = line - e * N2;
+            const int c1 = li % N, c2 = li / N;
+            double* se = smem + (size_t)e * C::SM;
+            const Fx* XP = reinterpret_cast<const Fx*>(se) + C::XP;
+            const Fx* XN = reinterpret_cast<const Fx*>(se) + C::XN + 3 * l * SL;
+            const FixScale& s = sScale[e];
+            const int ii = line_slot<N>(l, i < N ? i : 0, c1, c2);
+            const PrimFx a = {XP[ii], XP[SL + ii], XP[2 * SL + ii], XP[3 * SL + ii], XP[4 * SL + ii], XP[5 * SL + ii]};
+            const Fx na0 = XN[ii], na1 = XN[SL + ii], na2 = XN[2 * SL + ii];
+            long long acc[5] = {0, 0, 0, 0, 0};
+#pragma unroll 1
+            for (int k = 1; k <= N / 2; ++k) {
+                const int j = i + k < N ? i + k : i + k - N;
+                long long Pv[5] = {0, 0, 0, 0, 0};
+                if (go && (2 * k < N || i < k)) {
+                    const int jj = line_slot<N>(l, j, c1, c2);
+                    const PrimFx b = {XP[jj], XP[SL + jj], XP[2 * SL + jj], XP[3 * SL + jj], XP[4 * SL + jj], XP[5 * SL + jj]};
+                    const LogMeanF64 lm = {a.r, b.r, a.b, b.b, s, ph.inv_gm1};
+                    // the flux is linear in n: contracted with S_ij (n_i + n_j), twice the averaged metric
+                    // times half the pair coefficient
+                    const Fx S = sS[(k - 1) * N + i];
+                    ec_flux_fx(a, b, fx_split(fx_mul<2>(S, fx_add(na0, XN[jj]))), fx_split(fx_mul<2>(S, fx_add(na1, XN[SL + jj]))),
+                               fx_split(fx_mul<2>(S, fx_add(na2, XN[2 * SL + jj]))), ops.CG, s, lm, Pv);
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) acc[v] -= Pv[v];
+                }
+                const int from = (lw * N + (i >= k ? i - k : i - k + N)) & 31;
+#pragma unroll
+                for (int v = 0; v < 5; ++v) acc[v] += __shfl_sync(0xffffffffu, Pv[v], from);
+            }
+            if (go) {
+                double* R = se + C::R + l * 5 * N3 + line_base<N>(l, c1, c2) + i * dir_stride<N>(l);
+                const double w = sW[i];
+#pragma unroll
+                for (int v = 0; v < 5; ++v)
+                    R[v * N3] = w * fx_to_double(acc[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km));
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---- 2. interface SAT: -(E_ii f_EC(own, nbr).n_J + lambda/2 (q_own - q_nbr)) / w_i, into the
+    // direction's result
+    if (active) {
+        const FixScale& s = sScale[el_loc];
+        for (int fn = node; fn < 6 * N2; fn += N3) {
+            const int l = fn / (2 * N2);
+            const int rem = fn - l * 2 * N2;
+            const int side = rem / N2, fi = rem - side * N2;
+            const int st = dir_stride<N>(l);
+            const int base = line_base<N>(l, fi % N, fi / N);
+            const int own = base + (side ? (N - 1) * st : 0);
+            const int os = line_slot<N>(l, side ? N - 1 : 0, fi % N, fi / N);
+            const int64_t nb = nbr[el * 6 + 2 * l + side];
+            const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
+            bool bnd = false;
+            if constexpr (XF) {
+                bnd = nb < 0;
+                if (bnd) qn = qext + eoff + own;
+            }
+            const Fx* XP = X + C::XP + os;
+            const Fx* g = X + C::F + fn;
+            const PrimFx a = {XP[0], XP[SL], XP[2 * SL], XP[3 * SL], XP[4 * SL], XP[5 * SL]};
+            const PrimFx b = {g[0], g[6 * N2], g[12 * N2], g[18 * N2], g[24 * N2], g[30 * N2]};
+            Fx n0 = X[C::XN + 3 * l * SL + os], n1 = X[C::XN + (3 * l + 1) * SL + os], n2 = X[C::XN + (3 * l + 2) * SL + os];
+            [[maybe_unused]] double nd[3];
+            if constexpr (XF) {
+                // optimized metrics: the interface terms take the analytic surface metrics (the own
+                // flux, cancelled against the volume term's boundary part, keeps the volume metrics)
+                const double* ns = nsurf ? nsurf + (el * 6 + 2 * l + side) * 3 * N2 + fi : geom + (el * 10 + 1 + 3 * l) * N3 + own;
+                const int sn = nsurf ? N2 : N3;
+                nd[0] = ns[0];
+                nd[1] = ns[sn];
+                nd[2] = ns[2 * sn];
+                if (nsurf) {
+                    n0 = fx_split(fx_from_double(nd[0], s.kn));
+                    n1 = fx_split(fx_from_double(nd[1], s.kn));
+                    n2 = fx_split(fx_from_double(nd[2], s.kn));
+                }
+            }
+            long long f[5];
+            const LogMeanF64 lm = {a.r, b.r, a.b, b.b, s, ph.inv_gm1};
+            ec_flux_fx(a, b, n0, n1, n2, ops.CG, s, lm, f);
+            double lam = 0.0;
+            double dm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};      // 1/2 D (w_own - w_nbr) + interior penalty
+            if constexpr (XF) {
+                double qv[5], jw[5], r[5], RTo, RTn, co, cn;
+                Prim so, sn;
+                FaceAvg fa;
+#pragma unroll
+                for (int v = 0; v < 5; ++v) qv[v] = q[eoff + v * N3 + own];
+                to_prim(qv, ph, so, RTo, co);
+#pragma unroll
+                for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
+                to_prim(qv, ph, sn, RTn, cn);
+                face_jump_avg(so, RTo, sn, RTn, ph, jw, r, fa);
+                if (ph.dissipation == 2) {
+                    matrix_dissipation(fa, jw, r, nd[0], nd[1], nd[2], ph, dm);
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) dm[v] *= 0.5;
+                }
+                if (ph.ip_coef > 0.0) {
+                    // sigma mu |n_J| / h with h = (J_own + J_nbr)/|n_J|
+                    const double nsq = nd[0] * nd[0] + nd[1] * nd[1] + nd[2] * nd[2];
+                    const double Jo = geom[el * 10 * N3 + own];
+                    const double Jn = bnd ? Jo : geom[nb * 10 * N3 + base + (side ? 0 : (N - 1) * st)];
+                    const double cip = ph.ip_coef * ph.mu * nsq / (Jo + Jn);
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) dm[v] = fma(cip, r[v], dm[v]);
+                }
+            }
+            if (ph.dissipation == 1) {
+                // |u.n| of both sides in Q60, c |n_J| in float64
+                const double nn = fnorm[(el * 6 + 2 * l + side) * N2 + fi];
+                const double co = sqrt_newton(ph.gamma * sm[C::P + 3 * N3 + own]), cn = sm[C::F + 36 * N2 + fn];
+                const double uo = fx_to_double(fx_dot(a.u0, n0, a.u1, n1, a.u2, n2), s.ku + s.kn + 1);
+                const double un = fx_to_double(fx_dot(b.u0, n0, b.u1, n1, b.u2, n2), s.ku + s.kn + 1);
+                lam = ops.winv[0] * (0.5 * fmax(fma(co, nn, fabs(uo)), fma(cn, nn, fabs(un))));
+            }
+            const double wi = side ? -ops.winv[N - 1] : ops.winv[0];
+            double* R = sm + C::R + l * 5 * N3 + own;
+#pragma unroll
+            for (int v = 0; v < 5; ++v) {
+                double r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * N3]);
+                if (ph.dissipation == 1) r = fma(-lam, q[eoff + v * N3 + own] - qn[v * N3], r);
+                if constexpr (XF) r = fma(-ops.winv[0], dm[v], r);
+                R[v * N3] = r;
+            }
+        }
+    }
+    __syncthreads();
+    double res[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    if (active) {
+        const double* R = sm + C::R + node;
+#pragma unroll
+        for (int v = 0; v < 5; ++v) res[v] = R[v * N3] + R[(5 + v) * N3] + R[(10 + v) * N3];
+    }
+
+    // ---- 3. viscous terms
+    if (ph.viscous) {
+        __syncthreads();                         // the results' space becomes theta's
+        // theta_a[k] = D_a w_k + lift: w2..w4 (k < 3), beta for w5 = -2 beta (k = 3)
+#pragma unroll 1
+        for (int id = t; id < n_el * 12 * N2; id += C::THREADS) {
+            const int e = id / (12 * N2), r = id - e * 12 * N2;
+            const int lk = r / N2, li = r - lk * N2;
+            const int l = lk >> 2, k = lk & 3;
+            const int c1 = li % N, c2 = li / N;
+            Fx* Xe = reinterpret_cast<Fx*>(smem + (size_t)e * C::SM);
+            const Fx* W = Xe + (k < 3 ? C::XW + k * SL : C::XP + 4 * SL);
+            Fx v[N];
+            long long out[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) v[j] = W[line_slot<N>(l, j, c1, c2)];
+            long long lift[2];
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const Fx* g = Xe + C::F + (2 * l + side) * N2 + li;
+                Fx wn = g[24 * N2];
+                if (k < 3) wn = fx_split(fx_mul(wn, g[(1 + k) * 6 * N2]) * 4);
+                const Fx wo = v[side ? N - 1 : 0];
+                lift[side] = fx_mul<0>(ops.LF, side ? fx_sub(wn, wo) : fx_sub(wo, wn));
+            }
+            line_derivative<N>(v, ops, lift[0], lift[1], out);
+            long long* T = reinterpret_cast<long long*>(Xe + C::R + lk * SL);
+            unsigned mag = 0;                    // bits of the magnitudes, units of 2^-31
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                T[line_slot<N>(l, j, c1, c2)] = out[j];
+                mag |= (unsigned)((out[j] ^ (out[j] >> 63)) >> 29);
+            }
+            if constexpr (N2 % 32 == 0) {        // one variable and element per warp
+                mag = __reduce_or_sync(0xffffffffu, mag);
+                if (lane == 0) atomicOr(&sMag[e][k == 3], mag);
+            } else {
+                atomicOr(&sMag[e][k == 3], mag);
+            }
+        }
+        __syncthreads();
+        if (active) {
+            // theta shifted up to the element's largest: its derivatives of nearly constant fields use few
+            // of their bits, and what follows would round them away
+            const int sw = max(__clz(sMag[el_loc][0]) - 1, 0), sb = max(__clz(sMag[el_loc][1]) - 1, 0);
+            const ViscScale s = visc_scale(sScale[el_loc], sw, sb, ops.kD);
+            const long long* T = reinterpret_cast<const long long*>(X + C::R + own_slot);
+            Fx* XN = X + C::XN + own_slot;
+            Fx* XP = X + C::XP + own_slot;
+            // A[k][m] = sum_a Ja_am theta_a[k] + u_k (the same of w5): du_k/dx_m without its factor J^-1 RT
+            long long A[3][3];
+            Fx Gb[3];
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+                Gb[m] = fx_split(fx_dot(XN[m * SL], fx_split(T[3 * SL] << sb), XN[(3 + m) * SL], fx_split(T[7 * SL] << sb),
+                                        XN[(6 + m) * SL], fx_split(T[11 * SL] << sb)));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const Fx t0 = fx_split(T[k * SL] << sw), t1 = fx_split(T[(4 + k) * SL] << sw), t2 = fx_split(T[(8 + k) * SL] << sw);
+                const Fx u = XP[(1 + k) * SL];
+#pragma unroll
+                for (int m = 0; m < 3; ++m)
+                    A[k][m] = (fx_dot(XN[m * SL], t0, XN[(3 + m) * SL], t1, XN[(6 + m) * SL], t2) >> s.sg) - (fx_mul(u, Gb[m]) >> s.su);
+            }
+            const Fx y = fx_split(fx_from_double(Y, s.ky)), z = fx_split(fx_from_double(Z, s.kz));
+            const long long tr = fx_mul(fx_split((A[0][0] + A[1][1] + A[2][2] + 2) >> 2), Fx{715827882, 715827883});
+            // stress mu (du_i/dx_m + du_m/dx_i - 2/3 div): xx, yy, zz, yz, xz, xy
+            Fx tau[6];
+#pragma unroll
+            for (int m = 0; m < 3; ++m) tau[m] = fx_split(fx_mul(y, fx_split(((A[m][m] + 1) >> 1) - tr)));
+            tau[3] = fx_split(fx_mul(y, fx_split((A[1][2] + A[2][1] + 2) >> 2)));
+            tau[4] = fx_split(fx_mul(y, fx_split((A[0][2] + A[2][0] + 2) >> 2)));
+            tau[5] = fx_split(fx_mul(y, fx_split((A[0][1] + A[1][0] + 2) >> 2)));
+            // energy flux tau u + heat flux
+            Fx en[3];
+            {
+                const Fx u0 = XP[SL], u1 = XP[2 * SL], u2 = XP[3 * SL];
+                const long long e0 = fx_dot(tau[0], u0, tau[5], u1, tau[4], u2);
+                const long long e1 = fx_dot(tau[5], u0, tau[1], u1, tau[3], u2);
+                const long long e2 = fx_dot(tau[4], u0, tau[3], u1, tau[2], u2);
+                en[0] = fx_split(((e0 + s.he) >> s.se) - ((fx_mul(z, Gb[0]) + s.hz) >> s.sz));
+                en[1] = fx_split(((e1 + s.he) >> s.se) - ((fx_mul(z, Gb[1]) + s.hz) >> s.sz));
+                en[2] = fx_split(((e2 + s.he) >> s.se) - ((fx_mul(z, Gb[2]) + s.hz) >> s.sz));
+            }
+            // contravariant fluxes Ftilde_l, each over the metric row it used and an unused primitive
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const Fx n0 = XN[3 * l * SL], n1 = XN[(3 * l + 1) * SL], n2 = XN[(3 * l + 2) * SL];
+                long long Ft[4];
+                Ft[0] = fx_dot(n0, tau[0], n1, tau[5], n2, tau[4]);
+                Ft[1] = fx_dot(n0, tau[5], n1, tau[1], n2, tau[3]);
+                Ft[2] = fx_dot(n0, tau[4], n1, tau[3], n2, tau[2]);
+                Ft[3] = fx_dot(n0, en[0], n1, en[1], n2, en[2]);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) XN[(3 * l + k) * SL] = fx_split(Ft[k]);
+                XP[l * SL] = fx_split(Ft[3]);
+                const int il = l == 0 ? i1 : (l == 1 ? i2 : i3);
+                if (il == 0 || il == N - 1) {
+                    const int side = il == N - 1;
+                    const int fi = l == 0 ? (i2 + N * i3) : (l == 1 ? (i1 + N * i3) : (i1 + N * i2));
+                    double* tr_out = trace + ((el * 6 + 2 * l + side) * 4) * N2 + fi;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) tr_out[k * N2] = fx_to_double(Ft[k], k < 3 ? s.kf : s.kh);
+                }
+            }
+        }
+        __syncthreads();
+        // the fluxes' derivatives along their own direction, in place
+#pragma unroll 1
+        for (int id = t; id < n_el * 12 * N2; id += C::THREADS) {
+            const int e = id / (12 * N2), r = id - e * 12 * N2;
+            const int lk = r / N2, li = r - lk * N2;
+            const int l = lk >> 2, k = lk & 3;
+            const int c1 = li % N, c2 = li / N;
+            Fx* W = reinterpret_cast<Fx*>(smem + (size_t)e * C::SM) + (k < 3 ? C::XN + (3 * l + k) * SL : C::XP + l * SL);
+            Fx v[N];
+            long long out[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) v[j] = W[line_slot<N>(l, j, c1, c2)];
+            line_derivative<N>(v, ops, 0, 0, out);
+            long long* D = reinterpret_cast<long long*>(W);
+#pragma unroll
+            for (int j = 0; j < N; ++j) D[line_slot<N>(l, j, c1, c2)] = out[j];
+        }
+        __syncthreads();
+        if (active) {
+            const int sw = max(__clz(sMag[el_loc][0]) - 1, 0), sb = max(__clz(sMag[el_loc][1]) - 1, 0);
+            const ViscScale s = visc_scale(sScale[el_loc], sw, sb, ops.kD);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const long long* D = reinterpret_cast<const long long*>(X + (k < 3 ? C::XN + k * SL : C::XP) + own_slot);
+                const int st = k < 3 ? 3 * SL : SL;
+                res[1 + k] += fx_to_double(D[0] + D[st] + D[2 * st], (k < 3 ? s.kf : s.kh) + ops.kD);
+            }
+        }
+    }
+    if (active) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+            double r = res[v] * Jinv;
+            if constexpr (XF) {
+                if (src) r = fma(res[v], Jinv, src[eoff + v * N3 + node]);
+            }
+            dqdt[eoff + v * N3 + node] = r;
+        }
+    }
+}
+
+template <int N>
+constexpr size_t fix_smem() { return (size_t)FixCfg<N>::EPB * FixCfg<N>::SM * sizeof(double); }
+
+template <int N, bool XF>
+cudaError_t launch_n(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    using C = FixCfg<N>;
+    static_assert(C::SM >= Cfg<N>::SM, "the float64 form runs in the same shared memory");
+    const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
+    rhs_fix_f64<N, XF><<<grid, C::THREADS, fix_smem<N>(), s>>>(q, dqdt, c->d_geom, c->d_jinv, c->d_nbr,
+                                                              (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext,
+                                                              c->d_src, c->d_nsurf, c->d_fnorm);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t prepare_n(bool xf) {
+    constexpr cudaFuncAttribute kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return xf ? cudaFuncSetAttribute(rhs_fix_f64<N, true>, kAttr, (int)fix_smem<N>())
+              : cudaFuncSetAttribute(rhs_fix_f64<N, false>, kAttr, (int)fix_smem<N>());
+}
+
+}  // namespace
+
+cudaError_t prepare_rhs_fix(const esdc_ctx* c, bool xf) {
+    switch (c->N) {
+        case 2: return prepare_n<2>(xf);
+        case 3: return prepare_n<3>(xf);
+        case 4: return prepare_n<4>(xf);
+        case 5: return prepare_n<5>(xf);
+        case 6: return prepare_n<6>(xf);
+        case 7: return prepare_n<7>(xf);
+        case 8: return prepare_n<8>(xf);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_rhs_fix(const esdc_ctx* c, bool xf, const double* q, double* dqdt, cudaStream_t s) {
+    switch (c->N) {
+        case 2: return xf ? launch_n<2, true>(c, q, dqdt, s) : launch_n<2, false>(c, q, dqdt, s);
+        case 3: return xf ? launch_n<3, true>(c, q, dqdt, s) : launch_n<3, false>(c, q, dqdt, s);
+        case 4: return xf ? launch_n<4, true>(c, q, dqdt, s) : launch_n<4, false>(c, q, dqdt, s);
+        case 5: return xf ? launch_n<5, true>(c, q, dqdt, s) : launch_n<5, false>(c, q, dqdt, s);
+        case 6: return xf ? launch_n<6, true>(c, q, dqdt, s) : launch_n<6, false>(c, q, dqdt, s);
+        case 7: return xf ? launch_n<7, true>(c, q, dqdt, s) : launch_n<7, false>(c, q, dqdt, s);
+        case 8: return xf ? launch_n<8, true>(c, q, dqdt, s) : launch_n<8, false>(c, q, dqdt, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace esdc
