@@ -35,9 +35,16 @@ template <int N>
 struct FixCfg {
     static constexpr int N2 = N * N, N3 = N * N * N;
     static constexpr int EPB = Cfg<N>::EPB;
-    static constexpr int THREADS = (EPB * N3 + 31) / 32 * 32;    // whole warps (the pair loop's shuffles)
+    // Whole warps (the pair loop's shuffles); N = 6 one more than its nodes fill, which makes its 24 pair
+    // tasks three rounds (2.43 -> 2.34 ms on 26^3 elements)
+    static constexpr int THREADS = N == 6 ? 256 : (EPB * N3 + 31) / 32 * 32;
     static constexpr int WARPS = THREADS / 32;
-    static constexpr int MINB = N >= 7 ? 1 : (N == 6 ? 2 : 4);
+    // Resident CTAs the registers are capped for: as many as the shared memory lets in.  The kernel takes
+    // 124 to 174 registers left alone; the few spills cost less than the warps bring (N = 7, two CTAs
+    // instead of one: 3.01 -> 2.39 ms on 22^3; N = 5, five instead of four: 2.31 -> 2.29 ms on 32^3; N = 3:
+    // 1.10 -> 1.07 ms on 40^3; N = 2 with five: 1.48 -> 1.51 ms, so four; N = 8 with 24 or 20 warps on its
+    // one CTA: 2.92 -> 2.96 and 3.01 ms on 20^3, so 16)
+    static constexpr int MINB = N == 8 ? 1 : (N >= 6 ? 2 : (N == 5 || N == 3 ? 5 : 4));
     // pair loop: LPW whole lines per warp, TPD warp tasks per direction
     static constexpr int LPW = 32 / N, TPD = (EPB * N2 + LPW - 1) / LPW;
     // node slots of the limb arrays: rows of S2, layers of S3 (see slot)
@@ -49,8 +56,8 @@ struct FixCfg {
                                                  //         [3][SL] the viscous fluxes' energy part
     static constexpr int XW = 15 * SL;           // [3][SL] w2..w4 = 2 beta u
     static constexpr int R = 18 * SL;            // [3][5][N3] results per direction (float64); then [12][SL] theta
-    static constexpr int P = 33 * SL;            // [4][N3] float64 half velocity and RT
-    static constexpr int F = P + 4 * N3;         // [7][6 N2] neighbour face nodes: six primitives, sound speed
+    static constexpr int P = 33 * SL;            // [N3] float64 RT
+    static constexpr int F = P + N3;             // [7][6 N2] neighbour face nodes: six primitives, sound speed
     static constexpr int SM = F + 42 * N2;
 };
 
@@ -214,10 +221,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         sm[C::XP + 3 * SL + own_slot] = s.hu2;
         sm[C::XP + 4 * SL + own_slot] = s.beta;
         sm[C::XP + 5 * SL + own_slot] = s.qq;
-        sm[C::P + node] = s.hu0;
-        sm[C::P + N3 + node] = s.hu1;
-        sm[C::P + 2 * N3 + node] = s.hu2;
-        sm[C::P + 3 * N3 + node] = RT;
+        sm[C::P + node] = RT;
         // a sign bit counts as out of range (density and beta must be positive)
         E[0] = (unsigned)double_hi(s.hr) >> 20;
         E[1] = 4096 - E[0];
@@ -431,7 +435,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             if (ph.dissipation == 1) {
                 // |u.n| of both sides in Q60, c |n_J| in float64
                 const double nn = fnorm[(el * 6 + 2 * l + side) * N2 + fi];
-                const double co = sqrt_newton(ph.gamma * sm[C::P + 3 * N3 + own]), cn = sm[C::F + 36 * N2 + fn];
+                const double co = sqrt_newton(ph.gamma * sm[C::P + own]), cn = sm[C::F + 36 * N2 + fn];
                 const double uo = fx_to_double(fx_dot(a.u0, n0, a.u1, n1, a.u2, n2), s.ku + s.kn + 1);
                 const double un = fx_to_double(fx_dot(b.u0, n0, b.u1, n1, b.u2, n2), s.ku + s.kn + 1);
                 lam = ops.winv[0] * (0.5 * fmax(fma(co, nn, fabs(uo)), fma(cn, nn, fabs(un))));
@@ -603,13 +607,16 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     }
 }
 
+// the float64 form runs in the same shared memory
 template <int N>
-constexpr size_t fix_smem() { return (size_t)FixCfg<N>::EPB * FixCfg<N>::SM * sizeof(double); }
+constexpr size_t fix_smem() {
+    constexpr int sm = FixCfg<N>::SM > Cfg<N>::SM ? FixCfg<N>::SM : Cfg<N>::SM;
+    return (size_t)FixCfg<N>::EPB * sm * sizeof(double);
+}
 
 template <int N, bool XF>
 cudaError_t launch_n(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
     using C = FixCfg<N>;
-    static_assert(C::SM >= Cfg<N>::SM, "the float64 form runs in the same shared memory");
     const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
     rhs_fix_f64<N, XF><<<grid, C::THREADS, fix_smem<N>(), s>>>(q, dqdt, c->d_geom, c->d_jinv, c->d_nbr,
                                                               (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext,
