@@ -2,7 +2,7 @@
 // fluxes and their divergence, every operation in float64.  rhs_f64.cu runs it for the volume fluxes
 // without a fixed-point form; rhs_fix_f64.cu for elements outside the fixed-point range.
 //
-// One element per group of N^3 threads (EPB elements per CTA).  The element's state is loaded once,
+// One element per group of N^3 threads (EPB elements per CTA, which has at least EPB N^3 threads).  The element's state is loaded once,
 // converted to primitive and entropy variables in shared memory, and then:
 //   1. volume: one thread per xi_l line of each direction evaluates the N(N-1)/2 distinct node pairs of
 //      its line once each, using the skew part S of Q = S + E/2: r_i -= 2 S_ij f_ij / w_i,
@@ -39,13 +39,13 @@ struct Cfg {
 // XF: the kernel also handles the matrix dissipation, the interior penalty, boundary faces with an
 // exterior state and a source term (compiled only into the instantiations of contexts that use
 // them, so the default kernel carries none of it)
-template <int N, int VF, bool XF>
+template <int N, int VF, bool XF, int EPB = Cfg<N>::EPB>
 __device__ __forceinline__ void
 element_f64(double* smem, const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
             const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K, const Ops& ops, const Phys& ph,
             const double* __restrict__ qext, const double* __restrict__ src, const double* __restrict__ nsurf,
             const double* __restrict__ fnorm) {
-    constexpr int N2 = Cfg<N>::N2, N3 = Cfg<N>::N3, EPB = Cfg<N>::EPB;
+    constexpr int N2 = Cfg<N>::N2, N3 = Cfg<N>::N3;
     const int t = threadIdx.x;
     const int el_loc = t / N3;
     const int node = t - el_loc * N3;

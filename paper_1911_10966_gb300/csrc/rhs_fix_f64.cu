@@ -31,20 +31,23 @@
 namespace esdc {
 namespace {
 
-template <int N>
+// WIDE: one element per CTA on as many warps as its pair loop has tasks (N = 7: half as many), for meshes
+// that leave SMs idle otherwise: what counts there is the length of one element's chain.
+template <int N, bool WIDE = false>
 struct FixCfg {
     static constexpr int N2 = N * N, N3 = N * N * N;
-    static constexpr int EPB = Cfg<N>::EPB;
+    static constexpr int EPB = WIDE ? 1 : Cfg<N>::EPB;
     // Whole warps (the pair loop's shuffles); N = 6 one more than its nodes fill, which makes its 24 pair
     // tasks three rounds (2.43 -> 2.34 ms on 26^3 elements)
-    static constexpr int THREADS = N == 6 ? 256 : (EPB * N3 + 31) / 32 * 32;
+    static constexpr int THREADS = WIDE ? (N == 2 ? 96 : (N == 3 ? 128 : (N == 4 ? 192 : (N == 5 ? 480 : 640))))
+                                        : (N == 6 ? 256 : (EPB * N3 + 31) / 32 * 32);
     static constexpr int WARPS = THREADS / 32;
     // Resident CTAs the registers are capped for: as many as the shared memory lets in.  The kernel takes
     // 124 to 174 registers left alone; the few spills cost less than the warps bring (N = 7, two CTAs
     // instead of one: 3.01 -> 2.39 ms on 22^3; N = 5, five instead of four: 2.31 -> 2.29 ms on 32^3; N = 3:
     // 1.10 -> 1.07 ms on 40^3; N = 2 with five: 1.48 -> 1.51 ms, so four; N = 8 with 24 or 20 warps on its
     // one CTA: 2.92 -> 2.96 and 3.01 ms on 20^3, so 16)
-    static constexpr int MINB = N == 8 ? 1 : (N >= 6 ? 2 : (N == 5 || N == 3 ? 5 : 4));
+    static constexpr int MINB = WIDE || N == 8 ? 1 : (N >= 6 ? 2 : (N == 5 || N == 3 ? 5 : 4));
     // pair loop: LPW whole lines per warp, TPD warp tasks per direction
     static constexpr int LPW = 32 / N, TPD = (EPB * N2 + LPW - 1) / LPW;
     // node slots of the limb arrays: rows of S2, layers of S3 (see slot)
@@ -75,22 +78,17 @@ __device__ __forceinline__ int line_slot(int l, int i, int c1, int c2) {
     return l == 0 ? slot<N>(i, c1, c2) : (l == 1 ? slot<N>(c1, i, c2) : slot<N>(c1, c2, i));
 }
 
-// Element-wide maxima of NV non-negative integers into out (shared memory, zeroed), by the threads of
-// active elements; a warp (or an 8-lane group at N = 2) inside one element reduces first.
-template <int N, int NV>
-__device__ __forceinline__ void block_max(int* out, int (&v)[NV], int lane) {
-    constexpr bool warp_el = FixCfg<N>::EPB == 1 || FixCfg<N>::N3 % 32 == 0;
-    if constexpr (warp_el || N == 2) {
-        const unsigned mask = warp_el ? __activemask() : 0xffu << (lane & 24);
+// Element-wide maxima of NV non-negative integers into out (element e's, shared memory, zeroed).  Called by
+// the active threads of a warp; UNIFORM: of one element.  The lanes of an element reduce first.
+template <bool UNIFORM, int NV>
+__device__ __forceinline__ void block_max(int* out, int e, int (&v)[NV], int lane) {
+    unsigned mask = __activemask();
+    if constexpr (!UNIFORM) mask = __match_any_sync(mask, e);
 #pragma unroll
-        for (int i = 0; i < NV; ++i) v[i] = __reduce_max_sync(mask, v[i]);
-        if (lane == __ffs(mask) - 1)
-#pragma unroll
-            for (int i = 0; i < NV; ++i) atomicMax(out + i, v[i]);
-    } else {
+    for (int i = 0; i < NV; ++i) v[i] = __reduce_max_sync(mask, v[i]);
+    if (lane == __ffs(mask) - 1)
 #pragma unroll
         for (int i = 0; i < NV; ++i) atomicMax(out + i, v[i]);
-    }
 }
 
 // Logarithmic means beyond the series of ec_flux_fx, in float64 from the fixed-point inputs.
@@ -139,12 +137,12 @@ __device__ __forceinline__ double sqrt_newton(double x) {
 }
 
 // the element of a CTA left to the float64 form; out of line, so that the kernel's registers are its own
-template <int N, bool XF>
+template <int N, bool XF, int EPB>
 __device__ __noinline__ void out_of_range(double* smem, const double* q, double* dqdt, const double* geom,
                                           const int32_t* nbr, double* trace, int64_t K, const Ops& ops, const Phys& ph,
                                           const double* qext, const double* src, const double* nsurf,
                                           const double* fnorm) {
-    element_f64<N, kFluxESC, XF>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+    element_f64<N, kFluxESC, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
 }
 
 // Derivatives along one line of N Q60 values: out_i = sum_j D_ij in_j 2^-kD, plus at the ends
@@ -167,13 +165,13 @@ __device__ __forceinline__ void line_derivative(const Fx (&v)[N], const Ops& ops
 // XF: the kernel also handles the matrix dissipation, the interior penalty, boundary faces with an
 // exterior state, a source term and surface metrics (compiled only into the instantiations of contexts
 // that use them)
-template <int N, bool XF>
-__global__ void __launch_bounds__(FixCfg<N>::THREADS, FixCfg<N>::MINB)
+template <int N, bool XF, bool WIDE>
+__global__ void __launch_bounds__(FixCfg<N, WIDE>::THREADS, FixCfg<N, WIDE>::MINB)
 rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
             const double* __restrict__ jinv, const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K,
             const __grid_constant__ Ops ops, const __grid_constant__ Phys ph, const double* __restrict__ qext,
             const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
-    using C = FixCfg<N>;
+    using C = FixCfg<N, WIDE>;
     constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL;
     extern __shared__ double smem[];
     __shared__ int sE[EPB][8];                   // largest exponents (of 4096 - E for the smallest)
@@ -232,41 +230,47 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         Z = ph.kappa_R * RT * RT * Jinv;         // dw5 to heat flux
         E[6] = biased_exp(Y);
         E[7] = biased_exp(Z);
-        for (int fn = node; fn < 6 * N2; fn += N3) {
-            const int l = fn / (2 * N2);
-            const int rem = fn - l * 2 * N2;
-            const int side = rem / N2, fi = rem - side * N2;
-            const int st = dir_stride<N>(l);
-            const int base = line_base<N>(l, fi % N, fi / N);
-            const int64_t nb = nbr[el * 6 + 2 * l + side];
-            const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
-            // a boundary face (neighbour -1, bounded boxes only) sees the exterior state at its own nodes
-            if constexpr (XF) {
-                if (nb < 0) qn = qext + eoff + base + (side ? (N - 1) * st : 0);
-                if (nsurf) {
-                    const double* ns = nsurf + (el * 6 + 2 * l + side) * 3 * N2 + fi;
-                    E[5] = max(max(E[5], biased_exp(ns[0])), max(biased_exp(ns[N2]), biased_exp(ns[2 * N2])));
-                }
+        block_max<EPB == 1 || N3 % 32 == 0>(sE[el_loc], el_loc, E, lane);
+    }
+#pragma unroll 1
+    for (int id = t; id < n_el * 6 * N2; id += C::THREADS) {
+        const int e = id / (6 * N2), fn = id - e * 6 * N2;
+        const int64_t ee = (int64_t)blockIdx.x * EPB + e;
+        const int l = fn / (2 * N2);
+        const int rem = fn - l * 2 * N2;
+        const int side = rem / N2, fi = rem - side * N2;
+        const int st = dir_stride<N>(l);
+        const int base = line_base<N>(l, fi % N, fi / N);
+        const int64_t nb = nbr[ee * 6 + 2 * l + side];
+        const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
+        int E[6] = {0, 0, 0, 0, 0, 0};
+        // a boundary face (neighbour -1, bounded boxes only) sees the exterior state at its own nodes
+        if constexpr (XF) {
+            if (nb < 0) qn = qext + ee * 5 * N3 + base + (side ? (N - 1) * st : 0);
+            if (nsurf) {
+                const double* ns = nsurf + (ee * 6 + 2 * l + side) * 3 * N2 + fi;
+                E[5] = max(biased_exp(ns[0]), max(biased_exp(ns[N2]), biased_exp(ns[2 * N2])));
             }
-#pragma unroll
-            for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
-            to_prim_fx(qv, ph, s, RT);
-            double* f = sm + C::F + fn;
-            f[0] = s.hr;
-            f[6 * N2] = s.hu0;
-            f[12 * N2] = s.hu1;
-            f[18 * N2] = s.hu2;
-            f[24 * N2] = s.beta;
-            f[30 * N2] = s.qq;
-            f[36 * N2] = sqrt_newton(ph.gamma * RT);
-            const int er = (unsigned)double_hi(s.hr) >> 20, eb = (unsigned)double_hi(s.beta) >> 20;
-            E[0] = max(E[0], er);
-            E[1] = max(E[1], 4096 - er);
-            E[2] = max(E[2], max(biased_exp(s.hu0), max(biased_exp(s.hu1), biased_exp(s.hu2))));
-            E[3] = max(E[3], eb);
-            E[4] = max(E[4], 4096 - eb);
         }
-        block_max<N, 8>(sE[el_loc], E, lane);
+        double qv[5], RT;
+        Prim s;
+#pragma unroll
+        for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
+        to_prim_fx(qv, ph, s, RT);
+        double* f = smem + (size_t)e * C::SM + C::F + fn;
+        f[0] = s.hr;
+        f[6 * N2] = s.hu0;
+        f[12 * N2] = s.hu1;
+        f[18 * N2] = s.hu2;
+        f[24 * N2] = s.beta;
+        f[30 * N2] = s.qq;
+        f[36 * N2] = sqrt_newton(ph.gamma * RT);
+        E[0] = (unsigned)double_hi(s.hr) >> 20;
+        E[1] = 4096 - E[0];
+        E[2] = max(biased_exp(s.hu0), max(biased_exp(s.hu1), biased_exp(s.hu2)));
+        E[3] = (unsigned)double_hi(s.beta) >> 20;
+        E[4] = 4096 - E[3];
+        block_max<EPB == 1 || (6 * N2) % 32 == 0>(sE[e], e, E, lane);
     }
     __syncthreads();
     bool ok = true;
@@ -276,7 +280,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     }
     if (!ok) {
         __syncthreads();
-        out_of_range<N, XF>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+        out_of_range<N, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
         return;
     }
     if (active) {
@@ -300,15 +304,19 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             XP[(1 + m) * SL] = u;
             X[C::XW + m * SL + own_slot] = fx_split(fx_mul(b, u) * 4);     // w = 2 beta u in units 2^(kb + ku)
         }
-        for (int fn = node; fn < 6 * N2; fn += N3) {
-            const double* f = sm + C::F + fn;
-            Fx* g = X + C::F + fn;
-            g[0] = fx_split(fx_from_double(f[0], s.kr));
+    }
+#pragma unroll 1
+    for (int id = t; id < n_el * 6 * N2; id += C::THREADS) {
+        const int e = id / (6 * N2), fn = id - e * 6 * N2;
+        const int* E = sE[e];
+        const FixScale s = fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], ops.kg);
+        const double* f = smem + (size_t)e * C::SM + C::F + fn;
+        Fx* g = reinterpret_cast<Fx*>(smem + (size_t)e * C::SM) + C::F + fn;
+        g[0] = fx_split(fx_from_double(f[0], s.kr));
 #pragma unroll
-            for (int m = 0; m < 3; ++m) g[(1 + m) * 6 * N2] = fx_split(fx_from_double(f[(1 + m) * 6 * N2], s.ku));
-            g[24 * N2] = fx_split(fx_from_double(f[24 * N2], s.kb));
-            g[30 * N2] = fx_split(fx_from_double(f[30 * N2], s.kq));
-        }
+        for (int m = 0; m < 3; ++m) g[(1 + m) * 6 * N2] = fx_split(fx_from_double(f[(1 + m) * 6 * N2], s.ku));
+        g[24 * N2] = fx_split(fx_from_double(f[24 * N2], s.kb));
+        g[30 * N2] = fx_split(fx_from_double(f[30 * N2], s.kq));
     }
     __syncthreads();
 
@@ -364,91 +372,94 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
 
     // ---- 2. interface SAT: -(E_ii f_EC(own, nbr).n_J + lambda/2 (q_own - q_nbr)) / w_i, into the
     // direction's result
-    if (active) {
-        const FixScale& s = sScale[el_loc];
-        for (int fn = node; fn < 6 * N2; fn += N3) {
-            const int l = fn / (2 * N2);
-            const int rem = fn - l * 2 * N2;
-            const int side = rem / N2, fi = rem - side * N2;
-            const int st = dir_stride<N>(l);
-            const int base = line_base<N>(l, fi % N, fi / N);
-            const int own = base + (side ? (N - 1) * st : 0);
-            const int os = line_slot<N>(l, side ? N - 1 : 0, fi % N, fi / N);
-            const int64_t nb = nbr[el * 6 + 2 * l + side];
-            const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
-            bool bnd = false;
-            if constexpr (XF) {
-                bnd = nb < 0;
-                if (bnd) qn = qext + eoff + own;
+#pragma unroll 1
+    for (int id = t; id < n_el * 6 * N2; id += C::THREADS) {
+        const int e = id / (6 * N2), fn = id - e * 6 * N2;
+        const int64_t ee = (int64_t)blockIdx.x * EPB + e;
+        double* se = smem + (size_t)e * C::SM;
+        const Fx* Xe = reinterpret_cast<const Fx*>(se);
+        const FixScale& s = sScale[e];
+        const int l = fn / (2 * N2);
+        const int rem = fn - l * 2 * N2;
+        const int side = rem / N2, fi = rem - side * N2;
+        const int st = dir_stride<N>(l);
+        const int base = line_base<N>(l, fi % N, fi / N);
+        const int own = base + (side ? (N - 1) * st : 0);
+        const int os = line_slot<N>(l, side ? N - 1 : 0, fi % N, fi / N);
+        const int64_t nb = nbr[ee * 6 + 2 * l + side];
+        const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
+        bool bnd = false;
+        if constexpr (XF) {
+            bnd = nb < 0;
+            if (bnd) qn = qext + ee * 5 * N3 + own;
+        }
+        const Fx* XP = Xe + C::XP + os;
+        const Fx* g = Xe + C::F + fn;
+        const PrimFx a = {XP[0], XP[SL], XP[2 * SL], XP[3 * SL], XP[4 * SL], XP[5 * SL]};
+        const PrimFx b = {g[0], g[6 * N2], g[12 * N2], g[18 * N2], g[24 * N2], g[30 * N2]};
+        Fx n0 = Xe[C::XN + 3 * l * SL + os], n1 = Xe[C::XN + (3 * l + 1) * SL + os], n2 = Xe[C::XN + (3 * l + 2) * SL + os];
+        [[maybe_unused]] double nd[3];
+        if constexpr (XF) {
+            // optimized metrics: the interface terms take the analytic surface metrics (the own
+            // flux, cancelled against the volume term's boundary part, keeps the volume metrics)
+            const double* ns = nsurf ? nsurf + (ee * 6 + 2 * l + side) * 3 * N2 + fi : geom + (ee * 10 + 1 + 3 * l) * N3 + own;
+            const int sn = nsurf ? N2 : N3;
+            nd[0] = ns[0];
+            nd[1] = ns[sn];
+            nd[2] = ns[2 * sn];
+            if (nsurf) {
+                n0 = fx_split(fx_from_double(nd[0], s.kn));
+                n1 = fx_split(fx_from_double(nd[1], s.kn));
+                n2 = fx_split(fx_from_double(nd[2], s.kn));
             }
-            const Fx* XP = X + C::XP + os;
-            const Fx* g = X + C::F + fn;
-            const PrimFx a = {XP[0], XP[SL], XP[2 * SL], XP[3 * SL], XP[4 * SL], XP[5 * SL]};
-            const PrimFx b = {g[0], g[6 * N2], g[12 * N2], g[18 * N2], g[24 * N2], g[30 * N2]};
-            Fx n0 = X[C::XN + 3 * l * SL + os], n1 = X[C::XN + (3 * l + 1) * SL + os], n2 = X[C::XN + (3 * l + 2) * SL + os];
-            [[maybe_unused]] double nd[3];
-            if constexpr (XF) {
-                // optimized metrics: the interface terms take the analytic surface metrics (the own
-                // flux, cancelled against the volume term's boundary part, keeps the volume metrics)
-                const double* ns = nsurf ? nsurf + (el * 6 + 2 * l + side) * 3 * N2 + fi : geom + (el * 10 + 1 + 3 * l) * N3 + own;
-                const int sn = nsurf ? N2 : N3;
-                nd[0] = ns[0];
-                nd[1] = ns[sn];
-                nd[2] = ns[2 * sn];
-                if (nsurf) {
-                    n0 = fx_split(fx_from_double(nd[0], s.kn));
-                    n1 = fx_split(fx_from_double(nd[1], s.kn));
-                    n2 = fx_split(fx_from_double(nd[2], s.kn));
-                }
+        }
+        long long f[5];
+        const LogMeanF64 lm = {a.r, b.r, a.b, b.b, s, ph.inv_gm1};
+        ec_flux_fx(a, b, n0, n1, n2, ops.CG, s, lm, f);
+        double lam = 0.0;
+        double dm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};      // 1/2 D (w_own - w_nbr) + interior penalty
+        if (XF && (ph.dissipation == 2 || ph.ip_coef > 0.0)) {
+            double qv[5], jw[5], r[5], RTo, RTn, co, cn;
+            Prim so, sn;
+            FaceAvg fa;
+#pragma unroll
+            for (int v = 0; v < 5; ++v) qv[v] = q[ee * 5 * N3 + v * N3 + own];
+            to_prim(qv, ph, so, RTo, co);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
+            to_prim(qv, ph, sn, RTn, cn);
+            face_jump_avg(so, RTo, sn, RTn, ph, jw, r, fa);
+            if (ph.dissipation == 2) {
+                matrix_dissipation(fa, jw, r, nd[0], nd[1], nd[2], ph, dm);
+#pragma unroll
+                for (int v = 0; v < 5; ++v) dm[v] *= 0.5;
             }
-            long long f[5];
-            const LogMeanF64 lm = {a.r, b.r, a.b, b.b, s, ph.inv_gm1};
-            ec_flux_fx(a, b, n0, n1, n2, ops.CG, s, lm, f);
-            double lam = 0.0;
-            double dm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};      // 1/2 D (w_own - w_nbr) + interior penalty
-            if constexpr (XF) {
-                double qv[5], jw[5], r[5], RTo, RTn, co, cn;
-                Prim so, sn;
-                FaceAvg fa;
+            if (ph.ip_coef > 0.0) {
+                // sigma mu |n_J| / h with h = (J_own + J_nbr)/|n_J|
+                const double nsq = nd[0] * nd[0] + nd[1] * nd[1] + nd[2] * nd[2];
+                const double Jo = geom[ee * 10 * N3 + own];
+                const double Jn = bnd ? Jo : geom[nb * 10 * N3 + base + (side ? 0 : (N - 1) * st)];
+                const double cip = ph.ip_coef * ph.mu * nsq / (Jo + Jn);
 #pragma unroll
-                for (int v = 0; v < 5; ++v) qv[v] = q[eoff + v * N3 + own];
-                to_prim(qv, ph, so, RTo, co);
-#pragma unroll
-                for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
-                to_prim(qv, ph, sn, RTn, cn);
-                face_jump_avg(so, RTo, sn, RTn, ph, jw, r, fa);
-                if (ph.dissipation == 2) {
-                    matrix_dissipation(fa, jw, r, nd[0], nd[1], nd[2], ph, dm);
-#pragma unroll
-                    for (int v = 0; v < 5; ++v) dm[v] *= 0.5;
-                }
-                if (ph.ip_coef > 0.0) {
-                    // sigma mu |n_J| / h with h = (J_own + J_nbr)/|n_J|
-                    const double nsq = nd[0] * nd[0] + nd[1] * nd[1] + nd[2] * nd[2];
-                    const double Jo = geom[el * 10 * N3 + own];
-                    const double Jn = bnd ? Jo : geom[nb * 10 * N3 + base + (side ? 0 : (N - 1) * st)];
-                    const double cip = ph.ip_coef * ph.mu * nsq / (Jo + Jn);
-#pragma unroll
-                    for (int v = 0; v < 5; ++v) dm[v] = fma(cip, r[v], dm[v]);
-                }
+                for (int v = 0; v < 5; ++v) dm[v] = fma(cip, r[v], dm[v]);
             }
-            if (ph.dissipation == 1) {
-                // |u.n| of both sides in Q60, c |n_J| in float64
-                const double nn = fnorm[(el * 6 + 2 * l + side) * N2 + fi];
-                const double co = sqrt_newton(ph.gamma * sm[C::P + own]), cn = sm[C::F + 36 * N2 + fn];
-                const double uo = fx_to_double(fx_dot(a.u0, n0, a.u1, n1, a.u2, n2), s.ku + s.kn + 1);
-                const double un = fx_to_double(fx_dot(b.u0, n0, b.u1, n1, b.u2, n2), s.ku + s.kn + 1);
-                lam = ops.winv[0] * (0.5 * fmax(fma(co, nn, fabs(uo)), fma(cn, nn, fabs(un))));
-            }
-            const double wi = side ? -ops.winv[N - 1] : ops.winv[0];
-            double* R = sm + C::R + l * 5 * N3 + own;
+        }
+        if (ph.dissipation == 1) {
+            // |u.n| of both sides in Q60, c |n_J| in float64
+            const double nn = fnorm[(ee * 6 + 2 * l + side) * N2 + fi];
+            const double co = sqrt_newton(ph.gamma * se[C::P + own]), cn = se[C::F + 36 * N2 + fn];
+            const double uo = fx_to_double(fx_dot(a.u0, n0, a.u1, n1, a.u2, n2), s.ku + s.kn + 1);
+            const double un = fx_to_double(fx_dot(b.u0, n0, b.u1, n1, b.u2, n2), s.ku + s.kn + 1);
+            lam = ops.winv[0] * (0.5 * fmax(fma(co, nn, fabs(uo)), fma(cn, nn, fabs(un))));
+        }
+        const double wi = side ? -ops.winv[N - 1] : ops.winv[0];
+        double* R = se + C::R + l * 5 * N3 + own;
 #pragma unroll
-            for (int v = 0; v < 5; ++v) {
-                double r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * N3]);
-                if (ph.dissipation == 1) r = fma(-lam, q[eoff + v * N3 + own] - qn[v * N3], r);
-                if constexpr (XF) r = fma(-ops.winv[0], dm[v], r);
-                R[v * N3] = r;
-            }
+        for (int v = 0; v < 5; ++v) {
+            double r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * N3]);
+            if (ph.dissipation == 1) r = fma(-lam, q[ee * 5 * N3 + v * N3 + own] - qn[v * N3], r);
+            if constexpr (XF) r = fma(-ops.winv[0], dm[v], r);
+            R[v * N3] = r;
         }
     }
     __syncthreads();
@@ -608,28 +619,49 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
 }
 
 // the float64 form runs in the same shared memory
-template <int N>
+template <int N, bool WIDE>
 constexpr size_t fix_smem() {
-    constexpr int sm = FixCfg<N>::SM > Cfg<N>::SM ? FixCfg<N>::SM : Cfg<N>::SM;
-    return (size_t)FixCfg<N>::EPB * sm * sizeof(double);
+    constexpr int sm = FixCfg<N, WIDE>::SM > Cfg<N>::SM ? FixCfg<N, WIDE>::SM : Cfg<N>::SM;
+    return (size_t)FixCfg<N, WIDE>::EPB * sm * sizeof(double);
 }
 
-template <int N, bool XF>
-cudaError_t launch_n(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
-    using C = FixCfg<N>;
+template <int N, bool XF, bool WIDE>
+cudaError_t launch_w(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    using C = FixCfg<N, WIDE>;
     const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
-    rhs_fix_f64<N, XF><<<grid, C::THREADS, fix_smem<N>(), s>>>(q, dqdt, c->d_geom, c->d_jinv, c->d_nbr,
-                                                              (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext,
-                                                              c->d_src, c->d_nsurf, c->d_fnorm);
+    rhs_fix_f64<N, XF, WIDE><<<grid, C::THREADS, fix_smem<N, WIDE>(), s>>>(q, dqdt, c->d_geom, c->d_jinv, c->d_nbr,
+                                                                         (double*)c->d_trace, c->K, c->ops, c->phys,
+                                                                         c->d_qext, c->d_src, c->d_nsurf, c->d_fnorm);
     return cudaGetLastError();
 }
 
-template <int N>
-cudaError_t prepare_n(bool xf) {
-    constexpr cudaFuncAttribute kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    return xf ? cudaFuncSetAttribute(rhs_fix_f64<N, true>, kAttr, (int)fix_smem<N>())
-              : cudaFuncSetAttribute(rhs_fix_f64<N, false>, kAttr, (int)fix_smem<N>());
+// Elements per SM up to which the wide form is taken (0: never), per residual with its face kernel, normal
+// against wide form: N = 2 512 elements 36.0 -> 20.7 us, N = 3 512 32.9 -> 24.7, N = 4 64 30 -> 20, 216
+// 30.9 -> 24.7, 343 37.0 -> 35.0, 512 37.1 -> 39.1, N = 5 125 35.0 -> 26.8, 216 41.1 -> 41.8, N = 7 125
+// 53.4 -> 47.3, 343 121.5 -> 125.1; N = 6 and 8 gain nothing (37.0 and 63.6 us for up to one element per SM).
+constexpr int wide_upto(int n) { return n == 2 ? 6 : (n == 3 ? 4 : (n == 4 ? 2 : (n == 5 || n == 7 ? 1 : 0))); }
+
+template <int N, bool XF>
+cudaError_t launch_x(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    if constexpr (wide_upto(N) > 0)
+        if (c->K <= (int64_t)wide_upto(N) * sm_count()) return launch_w<N, XF, true>(c, q, dqdt, s);
+    return launch_w<N, XF, false>(c, q, dqdt, s);
 }
+template <int N>
+cudaError_t launch_n(const esdc_ctx* c, bool xf, const double* q, double* dqdt, cudaStream_t s) {
+    return xf ? launch_x<N, true>(c, q, dqdt, s) : launch_x<N, false>(c, q, dqdt, s);
+}
+
+template <int N, bool XF>
+cudaError_t prepare_x() {
+    constexpr cudaFuncAttribute kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(rhs_fix_f64<N, XF, false>, kAttr, (int)fix_smem<N, false>());
+    if constexpr (wide_upto(N) > 0)
+        if (e == cudaSuccess) return cudaFuncSetAttribute(rhs_fix_f64<N, XF, true>, kAttr, (int)fix_smem<N, true>());
+    return e;
+}
+template <int N>
+cudaError_t prepare_n(bool xf) { return xf ? prepare_x<N, true>() : prepare_x<N, false>(); }
 
 }  // namespace
 
@@ -648,13 +680,13 @@ cudaError_t prepare_rhs_fix(const esdc_ctx* c, bool xf) {
 
 cudaError_t launch_rhs_fix(const esdc_ctx* c, bool xf, const double* q, double* dqdt, cudaStream_t s) {
     switch (c->N) {
-        case 2: return xf ? launch_n<2, true>(c, q, dqdt, s) : launch_n<2, false>(c, q, dqdt, s);
-        case 3: return xf ? launch_n<3, true>(c, q, dqdt, s) : launch_n<3, false>(c, q, dqdt, s);
-        case 4: return xf ? launch_n<4, true>(c, q, dqdt, s) : launch_n<4, false>(c, q, dqdt, s);
-        case 5: return xf ? launch_n<5, true>(c, q, dqdt, s) : launch_n<5, false>(c, q, dqdt, s);
-        case 6: return xf ? launch_n<6, true>(c, q, dqdt, s) : launch_n<6, false>(c, q, dqdt, s);
-        case 7: return xf ? launch_n<7, true>(c, q, dqdt, s) : launch_n<7, false>(c, q, dqdt, s);
-        case 8: return xf ? launch_n<8, true>(c, q, dqdt, s) : launch_n<8, false>(c, q, dqdt, s);
+        case 2: return launch_n<2>(c, xf, q, dqdt, s);
+        case 3: return launch_n<3>(c, xf, q, dqdt, s);
+        case 4: return launch_n<4>(c, xf, q, dqdt, s);
+        case 5: return launch_n<5>(c, xf, q, dqdt, s);
+        case 6: return launch_n<6>(c, xf, q, dqdt, s);
+        case 7: return launch_n<7>(c, xf, q, dqdt, s);
+        case 8: return launch_n<8>(c, xf, q, dqdt, s);
         default: return cudaErrorInvalidValue;
     }
 }

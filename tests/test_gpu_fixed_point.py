@@ -12,8 +12,8 @@ from tests.gpu_common import assert_parity, make_pair
 pytestmark = pytest.mark.gpu
 
 
-def _case(p, kind):
-    solver, q, mesh, gas, qo = make_pair(p, (3, 3, 3), warp=0.1, seed=2, Re=400.0, Ma=0.4)
+def _case(p, kind, k=(3, 3, 3)):
+    solver, q, mesh, gas, qo = make_pair(p, k, warp=0.1, seed=2, Re=400.0, Ma=0.4)
     rng = np.random.default_rng(7 * p)
     x = qo.numpy().copy()
     rho, mom = x[:, 0], x[:, 1:4]
@@ -41,6 +41,14 @@ def _case(p, kind):
 @pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6, 7])
 def test_residual_parity_across_the_rules(p, kind):
     solver, q, mesh, gas, qo = _case(p, kind)
+    assert_parity(solver.rhs(q), O.rhs(qo, mesh, gas), qo, mesh, gas)
+
+
+@pytest.mark.parametrize("kind", ["far", "range"])
+@pytest.mark.parametrize("p,k", [(1, (11, 10, 9)), (2, (9, 8, 9)), (3, (7, 7, 7)), (4, (5, 6, 6)), (6, (5, 6, 6))])
+def test_residual_parity_beyond_the_wide_form(p, k, kind):
+    """Up to 1 to 6 elements per SM (by degree) run one element per CTA on more warps; these do not."""
+    solver, q, mesh, gas, qo = _case(p, kind, k)
     assert_parity(solver.rhs(q), O.rhs(qo, mesh, gas), qo, mesh, gas)
 
 
