@@ -31,6 +31,7 @@ struct Ops {
     FxPair SF[kMaxN / 2][kMaxN];
     FxPair CG;
     int kg;
+    FxPair MF[kMaxN][kMaxN];   // S_ij / 2, on the diagonal half the row's sum 1/2, 0, .., -1/2 (DC)
     FxPair DF[kMaxN][kMaxN];   // D_ij 2^-kD
     FxPair LF;                 // interface lift 1/(2 w_0) 2^-kD
     int kD;

@@ -93,6 +93,16 @@ ESDC_HD long long fx_dot(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f) {
     return mad_wide(a.h, b.h, mad_wide(c.h, d.h, mad_wide(e.h, f.h, mid >> 30)));
 }
 
+// the same times 2^SH
+template <int LL, int SH>
+ESDC_HD long long fx_dot_shl(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f) {
+    long long mid = mad_wide(a.l, b.h, mad_wide(a.h, b.l, (kFxHalf >> SH) + LL * kFxLow));
+    mid = mad_wide(c.l, d.h, mad_wide(c.h, d.l, mid));
+    mid = mad_wide(e.l, f.h, mad_wide(e.h, f.l, mid));
+    const long long hh = mad_wide(a.h, b.h, mad_wide(c.h, d.h, mul_wide(e.h, f.h)));
+    return (hh << SH) + (mid >> (30 - SH));
+}
+
 ESDC_HD unsigned mul_hi_u32(unsigned a, unsigned b) {
 #ifdef __CUDA_ARCH__
     return __umulhi(a, b);
@@ -188,7 +198,8 @@ ESDC_HD long long fx_rcp(Fx s, float seed, int ib) {
 // Exponents of one element's fixed-point quantities (value = Q60 number * 2^k) and the alignment
 // shifts of the two-point flux; the same for all nodes of the element.
 struct FixScale {
-    int kr, ku, kb, kn, kq;  // half density, half velocity, beta, metric terms, |u|^2/4
+    int kr, ku, kb, kn;      // half density, half velocity, beta, metric terms
+    int kq, kp;              // PrimFx::q and p
     int ir, ib;              // 1/(sum of half densities) <= 2^ir, 1/(sum of betas) <= 2^ib (in Q60)
     int k0, km, k5;          // mass, momentum and energy flux
     int kA;                  // inv_gm1 F / (sum of betas)
@@ -252,6 +263,49 @@ ESDC_HD FixScale fix_scale(int Er, int Er0, int Eu, int Eb, int Eb0, int En, int
     return s;
 }
 
+// The same for the Kennedy-Gruber flux; Eq, Ep: largest exponents of PrimFx::q and p.  Bounds: q and p < 1/2,
+// mass flux < 3/2, momentum flux < 5/4, energy flux < 3/2 (each with its factor S_ij).
+ESDC_HD FixScale fix_scale_kg(int Er, int Eu, int Eb, int En, int Ey, int Ez, int Eq, int Ep) {
+    FixScale s = {};
+    s.kr = Er - 1021;
+    s.ku = Eu - 1020;
+    s.kb = Eb - 1021;
+    s.kn = En - 1020;
+    s.kq = Eq - 1021;
+    s.kp = Ep - 1021;
+    s.k0 = s.kr + s.ku + s.kn - 1;
+    const int ka = s.k0 + s.ku, kb = s.kp + s.kn;
+    s.km = fx_max(ka, kb);
+    s.sA = fx_clamp(s.km - ka);
+    s.sB = fx_clamp(s.km - kb);
+    const int kC = s.k0 + s.kq, kM = s.kp + s.ku + s.kn - 1;
+    s.k5 = fx_max(kC, kM) + 1;
+    s.sC = fx_clamp(s.k5 - kC);
+    s.sD = fx_clamp(s.k5 - kM);
+    s.hC = (1ll << s.sC) >> 1;
+    s.hD = (1ll << s.sD) >> 1;
+    s.ky = Ey - 1021;
+    s.kz = Ez - 1021;
+    return s;
+}
+
+// The same for nodal fluxes contracted with n < 1/4, whose densities and enthalpies are not summed: both < 1,
+// u.n < 3/16 and kept quadrupled, mass and energy flux < 3/4, momentum flux < 5/16.  Their products with half
+// of S: absolute row sums < 2.4 with the diagonal, at most seven limbs besides the head's, so the limb sums
+// stay below 7.6 2^60.
+ESDC_HD FixScale fix_scale_dc(int Er, int Eu, int Eb, int En, int Ey, int Ez, int Eq, int Ep) {
+    FixScale s = fix_scale_kg(Er, Eu, Eb, En, Ey, Ez, Eq, Ep);
+    --s.kr;
+    --s.kq;
+    s.k0 = s.kr + s.ku + s.kn;
+    const int ka = s.k0 + s.ku + 1, kb = s.kp + 1 + s.kn;
+    s.km = fx_max(ka, kb);
+    s.sA = fx_clamp(s.km - ka);
+    s.sB = fx_clamp(s.km - kb);
+    s.k5 = s.k0 + s.kq;
+    return s;
+}
+
 // The viscous chain's exponents, known once theta is: w2..w4 = 2 beta u < 1/2 in units 2^(kb + ku), w5 =
 // -2 beta as beta itself; operator entries D_ij 2^-kD with row sums below 1.7, so theta (with its lift)
 // < 1.25, or < 1 once shifted left by sw (w2..w4) and sb (w5).  Then the contraction with the metric
@@ -291,9 +345,11 @@ ESDC_HD bool fix_range_ok(int Er, int Er0, int Eu, int Eb, int Eb0, int En) {
            Eu < 1151 && En < 1151;
 }
 
-// Per-node inputs of the pair loop, Q60 limbs: half density, half velocity, beta, |u|^2/4.
+// Per-node inputs of the pair loop, Q60 limbs: half density, half velocity, beta, and
+//   ES-C: q = |u|^2/4;   SF-KG: q = RT/(2(gamma - 1)) + |u|^2/4, p = half the pressure;
+//   DC: q = the specific enthalpy, p = half the pressure.
 struct PrimFx {
-    Fx r, u0, u1, u2, b, q;
+    Fx r, u0, u1, u2, b, q, p;
 };
 
 // Series of the logarithmic means in u = f^2, f = (a - b)/(a + b):
@@ -393,11 +449,7 @@ ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, F
         log_means_far(sh, dh, db, rs, g, s, lm, rl, A);
     const Fx rlf = fx_split(rl);
     const Fx v0 = fx_add(a.u0, b.u0), v1 = fx_add(a.u1, b.u1), v2 = fx_add(a.u2, b.u2);
-    long long mid = mad_wide(v0.l, n0.h, mad_wide(v0.h, n0.l, (kFxHalf >> 1) + 6 * kFxLow));
-    mid = mad_wide(v1.l, n1.h, mad_wide(v1.h, n1.l, mid));
-    mid = mad_wide(v2.l, n2.h, mad_wide(v2.h, n2.l, mid));
-    const long long hh = mad_wide(v0.h, n0.h, mad_wide(v1.h, n1.h, mul_wide(v2.h, n2.h)));
-    const Fx un = fx_split((hh << 1) + (mid >> 29));
+    const Fx un = fx_split(fx_dot_shl<6, 1>(v0, n0, v1, n1, v2, n2));
     const long long f1 = fx_mul(rlf, un);
     const long long pt = fx_mul<2>(sh, rs);
     const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(pt >> s.sB);
@@ -408,6 +460,32 @@ ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, F
     const Fx c5 = fx_split((A >> s.sc) - (fx_join(fx_add(a.q, b.q)) >> s.sq));
     const Fx m0 = fx_split(f[1]), m1 = fx_split(f[2]), m2 = fx_split(f[3]);
     f[4] = ((fx_mul(fx_split(f1), c5) + s.hC) >> s.sC) + ((fx_dot<6>(v0, m0, v1, m1, v2, m2) + s.hD) >> s.sD);
+}
+
+// The Kennedy-Gruber flux of flux_f64.cuh (kg_flux), units as above
+ESDC_HD void kg_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, const FixScale& s, long long f[5]) {
+    const Fx sh = fx_add(a.r, b.r), pt = fx_add(a.p, b.p);
+    const Fx v0 = fx_add(a.u0, b.u0), v1 = fx_add(a.u1, b.u1), v2 = fx_add(a.u2, b.u2);
+    const Fx un = fx_split(fx_dot_shl<6, 1>(v0, n0, v1, n1, v2, n2));
+    const long long f1 = fx_mul<2>(sh, un);
+    const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(fx_join(pt) >> s.sB);
+    f[0] = f1;
+    f[1] = fx_mul2<3>(fa, v0, pa, n0);
+    f[2] = fx_mul2<3>(fa, v1, pa, n1);
+    f[3] = fx_mul2<3>(fa, v2, pa, n2);
+    f[4] = ((fx_mul<2>(fx_split(f1), fx_add(a.q, b.q)) + s.hC) >> s.sC) + ((fx_mul<2>(pt, un) + s.hD) >> s.sD);
+}
+
+// The Euler flux of one node contracted with n (euler_flux_prim), units as above
+ESDC_HD void euler_flux_fx(const PrimFx& a, Fx n0, Fx n1, Fx n2, const FixScale& s, long long f[5]) {
+    const Fx un = fx_split(fx_dot_shl<3, 2>(a.u0, n0, a.u1, n1, a.u2, n2));
+    const long long f1 = fx_mul(a.r, un);
+    const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(fx_join(a.p) >> s.sB);
+    f[0] = f1;
+    f[1] = fx_mul2(fa, a.u0, pa, n0);
+    f[2] = fx_mul2(fa, a.u1, pa, n1);
+    f[3] = fx_mul2(fa, a.u2, pa, n2);
+    f[4] = fx_mul(fx_split(f1), a.q);
 }
 
 }  // namespace esdc

@@ -20,10 +20,17 @@ struct DivU64 {
 cudaError_t prepare_rhs_f64(const esdc_ctx* c);
 // ev: NULL, or four events recorded around the element kernel and the face kernel
 cudaError_t launch_rhs_f64(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s, cudaEvent_t* ev);
-// the ES-C element kernel in block fixed point (rhs_fix_f64.cu), called by the two above; xf: with the
-// optional interface terms
-cudaError_t prepare_rhs_fix(const esdc_ctx* c, bool xf);
-cudaError_t launch_rhs_fix(const esdc_ctx* c, bool xf, const double* q, double* dqdt, cudaStream_t s);
+// the element kernel in block fixed point (rhs_fix.cuh) by volume flux; _xf: with the optional interface terms
+#define ESDC_FIX_DECL(name)                          \
+    cudaError_t prepare_fix_##name(const esdc_ctx* c); \
+    cudaError_t launch_fix_##name(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s);
+ESDC_FIX_DECL(esc)
+ESDC_FIX_DECL(esc_xf)
+ESDC_FIX_DECL(kg)
+ESDC_FIX_DECL(kg_xf)
+ESDC_FIX_DECL(dc)
+ESDC_FIX_DECL(dc_xf)
+#undef ESDC_FIX_DECL
 // the p = 15 float64 residual (N = kLargeN), called by the two above
 cudaError_t prepare_rhs_large(const esdc_ctx* c);
 cudaError_t launch_rhs_large(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s, cudaEvent_t* ev);

@@ -1,6 +1,7 @@
-// ES-C residual of the float64 form in block fixed point (fix_f64.cuh): flux differencing with the
-// Chandrashekar flux (eq. discEL), the entropy-stable interface SAT, BR1 entropy-variable gradients,
-// viscous fluxes and their divergence (eq. MacroForm, eq. NSL) for p <= 7.
+// Residual of the float64 form in block fixed point (fix_f64.cuh): flux differencing with the
+// Chandrashekar flux (ES-C, eq. discEL), the Kennedy-Gruber flux (SF-KG) or the nodal fluxes (DC), the
+// interface SAT, BR1 entropy-variable gradients, viscous fluxes and their divergence (eq. MacroForm,
+// eq. NSL) for p <= 7.  rhs_fix_*.cu instantiate it.
 //
 // One element per group of N^3 threads (EPB elements per CTA).  Float64 is kept where it is needed or
 // cheap: primitives of own and neighbour states, the dissipation of the interface term, the sum of the
@@ -10,7 +11,8 @@
 //      range sends its CTA to the float64 form (element_f64.cuh).
 //   1. volume: one thread per (node, direction), whole lines side by side in a warp.  At cyclic distance
 //      k = 1..N/2 the thread of node i evaluates the pair (i, i + k mod N), so that each pair is
-//      evaluated once; S_ij f is summed in registers on one side and by a shuffle on the other.
+//      evaluated once; S_ij f is summed in registers on one side and by a shuffle on the other.  DC: the
+//      nodal contravariant fluxes per node, then one thread per line and variable.
 //   2. interface: one thread per face node; two-point flux in fixed point, dissipation in float64.
 //   3. viscous: lines of w for theta_a = D_a w + lift (one thread per line and variable, the operator
 //      from the constant bank), one thread per node for the fluxes, lines again for the divergence.
@@ -20,6 +22,8 @@
 // kept the float64 pipe 87% busy, per viscous residual of the Taylor-Green flow: 8.59 -> 2.86 ms at p = 7
 // on 20^3 elements, 0.92 -> 0.31 ms at p = 4 on 16^3, 2.58 -> 1.02 ms at p = 2 on 41 x 37 x 39.  Its error
 // against extended precision is smaller in every variable and degree tried.
+#pragma once
+
 #include <cuda_runtime.h>
 
 #include "element_f64.cuh"
@@ -31,9 +35,16 @@
 namespace esdc {
 namespace {
 
+// Node slots of the limb arrays: rows of S2, layers of S3 (see slot).
+template <int N>
+struct FixSlot {
+    static constexpr bool PAD = N == 4 || N == 6;
+    static constexpr int S2 = PAD ? N + 1 : N, S3 = N * S2 + (PAD ? 1 : 0), SL = N * S3;
+};
+
 // WIDE: one element per CTA on as many warps as its pair loop has tasks (N = 7: half as many), for meshes
 // that leave SMs idle otherwise: what counts there is the length of one element's chain.
-template <int N, bool WIDE = false>
+template <int N, int VF, bool WIDE = false>
 struct FixCfg {
     static constexpr int N2 = N * N, N3 = N * N * N;
     static constexpr int EPB = WIDE ? 1 : Cfg<N>::EPB;
@@ -50,18 +61,18 @@ struct FixCfg {
     static constexpr int MINB = WIDE || N == 8 ? 1 : (N >= 6 ? 2 : (N == 5 || N == 3 ? 5 : 4));
     // pair loop: LPW whole lines per warp, TPD warp tasks per direction
     static constexpr int LPW = 32 / N, TPD = (EPB * N2 + LPW - 1) / LPW;
-    // node slots of the limb arrays: rows of S2, layers of S3 (see slot)
-    static constexpr bool PAD = N == 4 || N == 6;
-    static constexpr int S2 = PAD ? N + 1 : N, S3 = N * S2 + (PAD ? 1 : 0), SL = N * S3;
+    static constexpr int SL = FixSlot<N>::SL;
     // shared memory per element in 8-byte units
     static constexpr int XN = 0;                 // [9][SL] metric rows; later the viscous fluxes' momentum part
-    static constexpr int XP = 9 * SL;            // [6][SL] half density, half velocity, beta, |u|^2/4; later
-                                                 //         [3][SL] the viscous fluxes' energy part
-    static constexpr int XW = 15 * SL;           // [3][SL] w2..w4 = 2 beta u
-    static constexpr int R = 18 * SL;            // [3][5][N3] results per direction (float64); then [12][SL] theta
-    static constexpr int P = 33 * SL;            // [N3] float64 RT
-    static constexpr int F = P + N3;             // [7][6 N2] neighbour face nodes: six primitives, sound speed
-    static constexpr int SM = F + 42 * N2;
+    static constexpr int NP = VF == kFluxESC ? 6 : 7;
+    static constexpr int XP = 9 * SL;            // [NP][SL] pair inputs (PrimFx); later [3][SL] the viscous
+                                                 //          fluxes' energy part
+    static constexpr int XW = XP + NP * SL;      // [3][SL] w2..w4 = 2 beta u
+    static constexpr int R = XW + 3 * SL;        // [3][5][SL] results per direction (float64; DC: the nodal
+                                                 //            fluxes before); then [12][SL] theta
+    static constexpr int P = R + 15 * SL;        // [N3] float64 RT
+    static constexpr int F = P + N3;             // [NP + 1][6 N2] neighbour face nodes: pair inputs, sound speed
+    static constexpr int SM = F + (NP + 1) * 6 * N2;
 };
 
 // Slot of node (i1, i2, i3) in the limb arrays.  A half-warp of 64-bit loads covers two lines of eight
@@ -70,7 +81,7 @@ struct FixCfg {
 template <int N>
 __device__ __forceinline__ int slot(int i1, int i2, int i3) {
     if constexpr (N == 8) return (i1 ^ (2 * ((i2 >> 1) ^ (i3 >> 1)))) + 8 * (i2 ^ (i3 & 1)) + 64 * i3;
-    else return i1 + FixCfg<N>::S2 * i2 + FixCfg<N>::S3 * i3;
+    else return i1 + FixSlot<N>::S2 * i2 + FixSlot<N>::S3 * i3;
 }
 // node i of line (c1, c2) of direction l
 template <int N>
@@ -125,6 +136,62 @@ __device__ __forceinline__ void to_prim_fx(const double* q, const Phys& ph, Prim
     s.beta = s.hr * rcp_cubic(p);
     RT = p * ri;
 }
+// The pair loop's inputs of a node, in PrimFx's order: half density, half velocity, beta, then |u|^2/4
+// (ES-C); or the node's part of the mean specific energy and half the pressure (SF-KG); or the specific
+// enthalpy and half the pressure (DC).
+template <int VF, int NP>
+__device__ __forceinline__ void pair_inputs(const double* q, const Phys& ph, double (&pi)[NP], double& RT) {
+    Prim s;
+    to_prim_fx(q, ph, s, RT);
+    pi[0] = s.hr;
+    pi[1] = s.hu0;
+    pi[2] = s.hu1;
+    pi[3] = s.hu2;
+    pi[4] = s.beta;
+    if constexpr (VF == kFluxESC) pi[5] = s.qq;
+    else {
+        pi[5] = VF == kFluxKG ? fma(0.5 * ph.inv_gm1, RT, s.qq) : fma(ph.gamma * ph.inv_gm1, RT, 2.0 * s.qq);
+        pi[6] = s.hr * RT;
+    }
+}
+// Exponents of a node's pair inputs for the element-wide maxima; a sign bit counts as out of range (density
+// and beta must be positive).
+template <int NP, int NE>
+__device__ __forceinline__ void pair_exponents(const double (&pi)[NP], int (&E)[NE]) {
+    E[0] = (unsigned)double_hi(pi[0]) >> 20;
+    E[1] = 4096 - E[0];
+    E[2] = max(biased_exp(pi[1]), max(biased_exp(pi[2]), biased_exp(pi[3])));
+    E[3] = (unsigned)double_hi(pi[4]) >> 20;
+    E[4] = 4096 - E[3];
+    if constexpr (NP == 7) {
+        E[8] = biased_exp(pi[5]);
+        E[9] = biased_exp(pi[6]);
+    }
+}
+// the element's scales from its maxima
+template <int VF, int NE>
+__device__ __forceinline__ FixScale element_scale(const int (&E)[NE], const Ops& ops) {
+    if constexpr (VF == kFluxESC) return fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], ops.kg);
+    else if constexpr (VF == kFluxKG) return fix_scale_kg(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
+    else return fix_scale_dc(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
+}
+// a node's (or neighbour's) pair inputs from float64 to limbs, arrays `stride` apart
+template <int VF>
+__device__ __forceinline__ void scale_inputs(const double* p, Fx* x, int stride, const FixScale& s) {
+    x[0] = fx_split(fx_from_double(p[0], s.kr));
+#pragma unroll
+    for (int m = 1; m < 4; ++m) x[m * stride] = fx_split(fx_from_double(p[m * stride], s.ku));
+    x[4 * stride] = fx_split(fx_from_double(p[4 * stride], s.kb));
+    x[5 * stride] = fx_split(fx_from_double(p[5 * stride], s.kq));
+    if constexpr (VF != kFluxESC) x[6 * stride] = fx_split(fx_from_double(p[6 * stride], s.kp));
+}
+template <int VF>
+__device__ __forceinline__ PrimFx load_inputs(const Fx* x, int stride) {
+    PrimFx a = {x[0], x[stride], x[2 * stride], x[3 * stride], x[4 * stride], x[5 * stride], Fx{0, 0}};
+    if constexpr (VF != kFluxESC) a.p = x[6 * stride];
+    return a;
+}
+
 // sqrt of a positive normal x: Goldschmidt's iteration (one step to 2^-44) and a correction from the residual
 __device__ __forceinline__ double sqrt_newton(double x) {
     double y;
@@ -137,44 +204,56 @@ __device__ __forceinline__ double sqrt_newton(double x) {
 }
 
 // the element of a CTA left to the float64 form; out of line, so that the kernel's registers are its own
-template <int N, bool XF, int EPB>
+template <int N, int VF, bool XF, int EPB>
 __device__ __noinline__ void out_of_range(double* smem, const double* q, double* dqdt, const double* geom,
                                           const int32_t* nbr, double* trace, int64_t K, const Ops& ops, const Phys& ph,
                                           const double* qext, const double* src, const double* nsurf,
                                           const double* fnorm) {
-    element_f64<N, kFluxESC, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+    element_f64<N, VF, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
 }
 
-// Derivatives along one line of N Q60 values: out_i = sum_j D_ij in_j 2^-kD, plus at the ends
-// lo, hi (the interface lift).
+// The two-point flux in fixed point (units 2^k0, 2^km, 2^k5), contracted with n.
+template <int VF>
+__device__ __forceinline__ void two_point(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, Fx cg, double inv_gm1,
+                                          const FixScale& s, long long (&f)[5]) {
+    if constexpr (VF == kFluxESC) {
+        ec_flux_fx(a, b, n0, n1, n2, cg, s, LogMeanF64{a.r, b.r, a.b, b.b, s, inv_gm1}, f);
+    } else if constexpr (VF == kFluxKG) {
+        kg_flux_fx(a, b, n0, n1, n2, s, f);
+    } else {
+        long long g[5];                          // the mean of the two nodal fluxes
+        euler_flux_fx(a, n0, n1, n2, s, f);
+        euler_flux_fx(b, n0, n1, n2, s, g);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) f[v] = (f[v] + g[v] + 1) >> 1;
+    }
+}
+
+// out_i = sum_j M_ij in_j along one line of N Q60 values
 template <int N>
-__device__ __forceinline__ void line_derivative(const Fx (&v)[N], const Ops& ops, long long lo, long long hi,
-                                                long long (&out)[N]) {
+__device__ __forceinline__ void line_product(const Fx (&v)[N], const Fx (&M)[kMaxN][kMaxN], long long (&out)[N]) {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         long long h = 0, m = kFxHalf + N * kFxLow;
 #pragma unroll
-        for (int j = 0; j < N; ++j) fx_mac(h, m, ops.DF[i][j], v[j]);
-        h += m >> 30;
-        if (i == 0) h += lo;
-        if (i == N - 1) h += hi;
-        out[i] = h;
+        for (int j = 0; j < N; ++j) fx_mac(h, m, M[i][j], v[j]);
+        out[i] = h + (m >> 30);
     }
 }
 
 // XF: the kernel also handles the matrix dissipation, the interior penalty, boundary faces with an
 // exterior state, a source term and surface metrics (compiled only into the instantiations of contexts
 // that use them)
-template <int N, bool XF, bool WIDE>
-__global__ void __launch_bounds__(FixCfg<N, WIDE>::THREADS, FixCfg<N, WIDE>::MINB)
+template <int N, int VF, bool XF, bool WIDE>
+__global__ void __launch_bounds__(FixCfg<N, VF, WIDE>::THREADS, FixCfg<N, VF, WIDE>::MINB)
 rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
             const double* __restrict__ jinv, const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K,
             const __grid_constant__ Ops ops, const __grid_constant__ Phys ph, const double* __restrict__ qext,
             const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
-    using C = FixCfg<N, WIDE>;
-    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL;
+    using C = FixCfg<N, VF, WIDE>;
+    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxESC ? 8 : 10;
     extern __shared__ double smem[];
-    __shared__ int sE[EPB][8];                   // largest exponents (of 4096 - E for the smallest)
+    __shared__ int sE[EPB][NE];                  // largest exponents (of 4096 - E for the smallest)
     __shared__ FixScale sScale[EPB];
     __shared__ unsigned sMag[EPB][2];            // magnitude bits of theta: w2..w4, w5
     __shared__ Fx sS[(N / 2) * N];
@@ -190,7 +269,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     Fx* X = reinterpret_cast<Fx*>(sm);
     const int own_slot = slot<N>(i1, i2, i3);
     const int64_t eoff = el * 5 * N3;
-    for (int i = t; i < EPB * 8; i += C::THREADS) sE[i / 8][i % 8] = 0;
+    for (int i = t; i < EPB * NE; i += C::THREADS) sE[i / NE][i % NE] = 0;
     if (t < EPB) sMag[t][0] = sMag[t][1] = 0;
     for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
     for (int i = t; i < N; i += C::THREADS) sW[i] = ops.winv[i];
@@ -199,12 +278,11 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     // ---- 0. primitives, exponents, scaling
     double Jinv = 0.0, Y = 0.0, Z = 0.0;
     if (active) {
-        double qv[5], RT;
-        Prim s;
+        double qv[5], RT, pi[NP];
 #pragma unroll
         for (int v = 0; v < 5; ++v) qv[v] = q[eoff + v * N3 + node];
         Jinv = jinv[el * N3 + node];
-        int E[8];
+        int E[NE];
         E[5] = 0;
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
@@ -212,20 +290,11 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             sm[C::XN + c * SL + own_slot] = g;
             E[5] = max(E[5], biased_exp(g));
         }
-        to_prim_fx(qv, ph, s, RT);
-        sm[C::XP + own_slot] = s.hr;
-        sm[C::XP + SL + own_slot] = s.hu0;
-        sm[C::XP + 2 * SL + own_slot] = s.hu1;
-        sm[C::XP + 3 * SL + own_slot] = s.hu2;
-        sm[C::XP + 4 * SL + own_slot] = s.beta;
-        sm[C::XP + 5 * SL + own_slot] = s.qq;
+        pair_inputs<VF>(qv, ph, pi, RT);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) sm[C::XP + i * SL + own_slot] = pi[i];
         sm[C::P + node] = RT;
-        // a sign bit counts as out of range (density and beta must be positive)
-        E[0] = (unsigned)double_hi(s.hr) >> 20;
-        E[1] = 4096 - E[0];
-        E[2] = max(biased_exp(s.hu0), max(biased_exp(s.hu1), biased_exp(s.hu2)));
-        E[3] = (unsigned)double_hi(s.beta) >> 20;
-        E[4] = 4096 - E[3];
+        pair_exponents<NP>(pi, E);
         Y = ph.mu * RT * Jinv;                   // velocity gradient to stress
         Z = ph.kappa_R * RT * RT * Jinv;         // dw5 to heat flux
         E[6] = biased_exp(Y);
@@ -243,7 +312,8 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         const int base = line_base<N>(l, fi % N, fi / N);
         const int64_t nb = nbr[ee * 6 + 2 * l + side];
         const double* qn = q + nb * 5 * N3 + base + (side ? 0 : (N - 1) * st);
-        int E[6] = {0, 0, 0, 0, 0, 0};
+        int E[NE];
+        E[5] = E[6] = E[7] = 0;
         // a boundary face (neighbour -1, bounded boxes only) sees the exterior state at its own nodes
         if constexpr (XF) {
             if (nb < 0) qn = qext + ee * 5 * N3 + base + (side ? (N - 1) * st : 0);
@@ -252,24 +322,15 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                 E[5] = max(biased_exp(ns[0]), max(biased_exp(ns[N2]), biased_exp(ns[2 * N2])));
             }
         }
-        double qv[5], RT;
-        Prim s;
+        double qv[5], RT, pi[NP];
 #pragma unroll
         for (int v = 0; v < 5; ++v) qv[v] = qn[v * N3];
-        to_prim_fx(qv, ph, s, RT);
+        pair_inputs<VF>(qv, ph, pi, RT);
         double* f = smem + (size_t)e * C::SM + C::F + fn;
-        f[0] = s.hr;
-        f[6 * N2] = s.hu0;
-        f[12 * N2] = s.hu1;
-        f[18 * N2] = s.hu2;
-        f[24 * N2] = s.beta;
-        f[30 * N2] = s.qq;
-        f[36 * N2] = sqrt_newton(ph.gamma * RT);
-        E[0] = (unsigned)double_hi(s.hr) >> 20;
-        E[1] = 4096 - E[0];
-        E[2] = max(biased_exp(s.hu0), max(biased_exp(s.hu1), biased_exp(s.hu2)));
-        E[3] = (unsigned)double_hi(s.beta) >> 20;
-        E[4] = 4096 - E[3];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) f[i * 6 * N2] = pi[i];
+        f[NP * 6 * N2] = sqrt_newton(ph.gamma * RT);
+        pair_exponents<NP>(pi, E);
         block_max<EPB == 1 || (6 * N2) % 32 == 0>(sE[e], e, E, lane);
     }
     __syncthreads();
@@ -280,12 +341,11 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     }
     if (!ok) {
         __syncthreads();
-        out_of_range<N, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+        out_of_range<N, VF, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
         return;
     }
     if (active) {
-        const int* E = sE[el_loc];
-        const FixScale s = fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], ops.kg);
+        const FixScale s = element_scale<VF>(sE[el_loc], ops);
         if (node == 0) sScale[el_loc] = s;
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
@@ -293,35 +353,54 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             X[i] = fx_split(fx_from_double(sm[i], s.kn));
         }
         Fx* XP = X + C::XP + own_slot;
-        const double* sp = sm + C::XP + own_slot;
-        XP[0] = fx_split(fx_from_double(sp[0], s.kr));
-        const Fx b = fx_split(fx_from_double(sp[4 * SL], s.kb));
-        XP[4 * SL] = b;
-        XP[5 * SL] = fx_split(fx_from_double(sp[5 * SL], s.kq));
+        scale_inputs<VF>(sm + C::XP + own_slot, XP, SL, s);
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const Fx u = fx_split(fx_from_double(sp[(1 + m) * SL], s.ku));
-            XP[(1 + m) * SL] = u;
-            X[C::XW + m * SL + own_slot] = fx_split(fx_mul(b, u) * 4);     // w = 2 beta u in units 2^(kb + ku)
-        }
+        for (int m = 0; m < 3; ++m)              // w = 2 beta u in units 2^(kb + ku)
+            X[C::XW + m * SL + own_slot] = fx_split(fx_mul(XP[4 * SL], XP[(1 + m) * SL]) * 4);
     }
 #pragma unroll 1
     for (int id = t; id < n_el * 6 * N2; id += C::THREADS) {
         const int e = id / (6 * N2), fn = id - e * 6 * N2;
-        const int* E = sE[e];
-        const FixScale s = fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], ops.kg);
-        const double* f = smem + (size_t)e * C::SM + C::F + fn;
-        Fx* g = reinterpret_cast<Fx*>(smem + (size_t)e * C::SM) + C::F + fn;
-        g[0] = fx_split(fx_from_double(f[0], s.kr));
-#pragma unroll
-        for (int m = 0; m < 3; ++m) g[(1 + m) * 6 * N2] = fx_split(fx_from_double(f[(1 + m) * 6 * N2], s.ku));
-        g[24 * N2] = fx_split(fx_from_double(f[24 * N2], s.kb));
-        g[30 * N2] = fx_split(fx_from_double(f[30 * N2], s.kq));
+        double* f = smem + (size_t)e * C::SM + C::F + fn;
+        scale_inputs<VF>(f, reinterpret_cast<Fx*>(f), 6 * N2, element_scale<VF>(sE[e], ops));
     }
     __syncthreads();
 
     // ---- 1. volume flux differencing
-    {
+    if constexpr (VF == kFluxDC) {
+        // nodal contravariant fluxes Ftilde_l, then twice their central fluxes' differences along the lines,
+        // acc_i = sum_j S_ij (F_i + F_j) = sum_j M_ij F_j, in place
+        if (active) {
+            const FixScale& s = sScale[el_loc];
+            const PrimFx a = load_inputs<VF>(X + C::XP + own_slot, SL);
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const Fx* n = X + C::XN + 3 * l * SL + own_slot;
+                long long f[5];
+                euler_flux_fx(a, n[0], n[SL], n[2 * SL], s, f);
+#pragma unroll
+                for (int v = 0; v < 5; ++v) X[C::R + (5 * l + v) * SL + own_slot] = fx_split(f[v]);
+            }
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int id = t; id < n_el * 15 * N2; id += C::THREADS) {
+            const int e = id / (15 * N2), r = id - e * 15 * N2;
+            const int lv = r / N2, li = r - lv * N2;
+            const int l = lv / 5, v = lv - 5 * l;
+            const int c1 = li % N, c2 = li / N;
+            double* R = smem + (size_t)e * C::SM + C::R + lv * SL;
+            const FixScale& s = sScale[e];
+            const int k = (v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)) + 1;
+            Fx x[N];
+            long long out[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) x[j] = reinterpret_cast<const Fx*>(R)[line_slot<N>(l, j, c1, c2)];
+            line_product<N>(x, ops.MF, out);
+#pragma unroll
+            for (int j = 0; j < N; ++j) R[line_slot<N>(l, j, c1, c2)] = -ops.winv[j] * fx_to_double(out[j], k);
+        }
+    } else {
         const int lw = lane / N, i = lane - lw * N;
 #pragma unroll 1
         for (int task = warp; task < 3 * C::TPD; task += C::WARPS) {
@@ -336,7 +415,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             const Fx* XN = reinterpret_cast<const Fx*>(se) + C::XN + 3 * l * SL;
             const FixScale& s = sScale[e];
             const int ii = line_slot<N>(l, i < N ? i : 0, c1, c2);
-            const PrimFx a = {XP[ii], XP[SL + ii], XP[2 * SL + ii], XP[3 * SL + ii], XP[4 * SL + ii], XP[5 * SL + ii]};
+            const PrimFx a = load_inputs<VF>(XP + ii, SL);
             const Fx na0 = XN[ii], na1 = XN[SL + ii], na2 = XN[2 * SL + ii];
             long long acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll 1
@@ -345,13 +424,13 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                 long long Pv[5] = {0, 0, 0, 0, 0};
                 if (go && (2 * k < N || i < k)) {
                     const int jj = line_slot<N>(l, j, c1, c2);
-                    const PrimFx b = {XP[jj], XP[SL + jj], XP[2 * SL + jj], XP[3 * SL + jj], XP[4 * SL + jj], XP[5 * SL + jj]};
-                    const LogMeanF64 lm = {a.r, b.r, a.b, b.b, s, ph.inv_gm1};
+                    const PrimFx b = load_inputs<VF>(XP + jj, SL);
                     // the flux is linear in n: contracted with S_ij (n_i + n_j), twice the averaged metric
                     // times half the pair coefficient
                     const Fx S = sS[(k - 1) * N + i];
-                    ec_flux_fx(a, b, fx_split(fx_mul<2>(S, fx_add(na0, XN[jj]))), fx_split(fx_mul<2>(S, fx_add(na1, XN[SL + jj]))),
-                               fx_split(fx_mul<2>(S, fx_add(na2, XN[2 * SL + jj]))), ops.CG, s, lm, Pv);
+                    const Fx n0 = fx_split(fx_mul<2>(S, fx_add(na0, XN[jj]))), n1 = fx_split(fx_mul<2>(S, fx_add(na1, XN[SL + jj]))),
+                             n2 = fx_split(fx_mul<2>(S, fx_add(na2, XN[2 * SL + jj])));
+                    two_point<VF>(a, b, n0, n1, n2, ops.CG, ph.inv_gm1, s, Pv);
 #pragma unroll
                     for (int v = 0; v < 5; ++v) acc[v] -= Pv[v];
                 }
@@ -360,11 +439,11 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                 for (int v = 0; v < 5; ++v) acc[v] += __shfl_sync(0xffffffffu, Pv[v], from);
             }
             if (go) {
-                double* R = se + C::R + l * 5 * N3 + line_base<N>(l, c1, c2) + i * dir_stride<N>(l);
+                double* R = se + C::R + l * 5 * SL + ii;
                 const double w = sW[i];
 #pragma unroll
                 for (int v = 0; v < 5; ++v)
-                    R[v * N3] = w * fx_to_double(acc[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km));
+                    R[v * SL] = w * fx_to_double(acc[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km));
             }
         }
     }
@@ -395,8 +474,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         }
         const Fx* XP = Xe + C::XP + os;
         const Fx* g = Xe + C::F + fn;
-        const PrimFx a = {XP[0], XP[SL], XP[2 * SL], XP[3 * SL], XP[4 * SL], XP[5 * SL]};
-        const PrimFx b = {g[0], g[6 * N2], g[12 * N2], g[18 * N2], g[24 * N2], g[30 * N2]};
+        const PrimFx a = load_inputs<VF>(XP, SL), b = load_inputs<VF>(g, 6 * N2);
         Fx n0 = Xe[C::XN + 3 * l * SL + os], n1 = Xe[C::XN + (3 * l + 1) * SL + os], n2 = Xe[C::XN + (3 * l + 2) * SL + os];
         [[maybe_unused]] double nd[3];
         if constexpr (XF) {
@@ -414,8 +492,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             }
         }
         long long f[5];
-        const LogMeanF64 lm = {a.r, b.r, a.b, b.b, s, ph.inv_gm1};
-        ec_flux_fx(a, b, n0, n1, n2, ops.CG, s, lm, f);
+        two_point<VF>(a, b, n0, n1, n2, ops.CG, ph.inv_gm1, s, f);
         double lam = 0.0;
         double dm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};      // 1/2 D (w_own - w_nbr) + interior penalty
         if (XF && (ph.dissipation == 2 || ph.ip_coef > 0.0)) {
@@ -447,27 +524,27 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         if (ph.dissipation == 1) {
             // |u.n| of both sides in Q60, c |n_J| in float64
             const double nn = fnorm[(ee * 6 + 2 * l + side) * N2 + fi];
-            const double co = sqrt_newton(ph.gamma * se[C::P + own]), cn = se[C::F + 36 * N2 + fn];
+            const double co = sqrt_newton(ph.gamma * se[C::P + own]), cn = se[C::F + NP * 6 * N2 + fn];
             const double uo = fx_to_double(fx_dot(a.u0, n0, a.u1, n1, a.u2, n2), s.ku + s.kn + 1);
             const double un = fx_to_double(fx_dot(b.u0, n0, b.u1, n1, b.u2, n2), s.ku + s.kn + 1);
             lam = ops.winv[0] * (0.5 * fmax(fma(co, nn, fabs(uo)), fma(cn, nn, fabs(un))));
         }
         const double wi = side ? -ops.winv[N - 1] : ops.winv[0];
-        double* R = se + C::R + l * 5 * N3 + own;
+        double* R = se + C::R + l * 5 * SL + os;
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            double r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * N3]);
+            double r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * SL]);
             if (ph.dissipation == 1) r = fma(-lam, q[ee * 5 * N3 + v * N3 + own] - qn[v * N3], r);
             if constexpr (XF) r = fma(-ops.winv[0], dm[v], r);
-            R[v * N3] = r;
+            R[v * SL] = r;
         }
     }
     __syncthreads();
     double res[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     if (active) {
-        const double* R = sm + C::R + node;
+        const double* R = sm + C::R + own_slot;
 #pragma unroll
-        for (int v = 0; v < 5; ++v) res[v] = R[v * N3] + R[(5 + v) * N3] + R[(10 + v) * N3];
+        for (int v = 0; v < 5; ++v) res[v] = R[v * SL] + R[(5 + v) * SL] + R[(10 + v) * SL];
     }
 
     // ---- 3. viscous terms
@@ -495,7 +572,9 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                 const Fx wo = v[side ? N - 1 : 0];
                 lift[side] = fx_mul<0>(ops.LF, side ? fx_sub(wn, wo) : fx_sub(wo, wn));
             }
-            line_derivative<N>(v, ops, lift[0], lift[1], out);
+            line_product<N>(v, ops.DF, out);     // in units 2^kD
+            out[0] += lift[0];
+            out[N - 1] += lift[1];
             long long* T = reinterpret_cast<long long*>(Xe + C::R + lk * SL);
             unsigned mag = 0;                    // bits of the magnitudes, units of 2^-31
 #pragma unroll
@@ -589,7 +668,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             long long out[N];
 #pragma unroll
             for (int j = 0; j < N; ++j) v[j] = W[line_slot<N>(l, j, c1, c2)];
-            line_derivative<N>(v, ops, 0, 0, out);
+            line_product<N>(v, ops.DF, out);
             long long* D = reinterpret_cast<long long*>(W);
 #pragma unroll
             for (int j = 0; j < N; ++j) D[line_slot<N>(l, j, c1, c2)] = out[j];
@@ -619,19 +698,19 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
 }
 
 // the float64 form runs in the same shared memory
-template <int N, bool WIDE>
+template <int N, int VF, bool WIDE>
 constexpr size_t fix_smem() {
-    constexpr int sm = FixCfg<N, WIDE>::SM > Cfg<N>::SM ? FixCfg<N, WIDE>::SM : Cfg<N>::SM;
-    return (size_t)FixCfg<N, WIDE>::EPB * sm * sizeof(double);
+    constexpr int sm = FixCfg<N, VF, WIDE>::SM > Cfg<N>::SM ? FixCfg<N, VF, WIDE>::SM : Cfg<N>::SM;
+    return (size_t)FixCfg<N, VF, WIDE>::EPB * sm * sizeof(double);
 }
 
-template <int N, bool XF, bool WIDE>
+template <int N, int VF, bool XF, bool WIDE>
 cudaError_t launch_w(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
-    using C = FixCfg<N, WIDE>;
+    using C = FixCfg<N, VF, WIDE>;
     const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
-    rhs_fix_f64<N, XF, WIDE><<<grid, C::THREADS, fix_smem<N, WIDE>(), s>>>(q, dqdt, c->d_geom, c->d_jinv, c->d_nbr,
-                                                                         (double*)c->d_trace, c->K, c->ops, c->phys,
-                                                                         c->d_qext, c->d_src, c->d_nsurf, c->d_fnorm);
+    rhs_fix_f64<N, VF, XF, WIDE><<<grid, C::THREADS, fix_smem<N, VF, WIDE>(), s>>>(
+        q, dqdt, c->d_geom, c->d_jinv, c->d_nbr, (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext, c->d_src,
+        c->d_nsurf, c->d_fnorm);
     return cudaGetLastError();
 }
 
@@ -641,54 +720,49 @@ cudaError_t launch_w(const esdc_ctx* c, const double* q, double* dqdt, cudaStrea
 // 53.4 -> 47.3, 343 121.5 -> 125.1; N = 6 and 8 gain nothing (37.0 and 63.6 us for up to one element per SM).
 constexpr int wide_upto(int n) { return n == 2 ? 6 : (n == 3 ? 4 : (n == 4 ? 2 : (n == 5 || n == 7 ? 1 : 0))); }
 
-template <int N, bool XF>
-cudaError_t launch_x(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+template <int N, int VF, bool XF>
+cudaError_t launch_n(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
     if constexpr (wide_upto(N) > 0)
-        if (c->K <= (int64_t)wide_upto(N) * sm_count()) return launch_w<N, XF, true>(c, q, dqdt, s);
-    return launch_w<N, XF, false>(c, q, dqdt, s);
-}
-template <int N>
-cudaError_t launch_n(const esdc_ctx* c, bool xf, const double* q, double* dqdt, cudaStream_t s) {
-    return xf ? launch_x<N, true>(c, q, dqdt, s) : launch_x<N, false>(c, q, dqdt, s);
+        if (c->K <= (int64_t)wide_upto(N) * sm_count()) return launch_w<N, VF, XF, true>(c, q, dqdt, s);
+    return launch_w<N, VF, XF, false>(c, q, dqdt, s);
 }
 
-template <int N, bool XF>
-cudaError_t prepare_x() {
+template <int N, int VF, bool XF>
+cudaError_t prepare_n() {
     constexpr cudaFuncAttribute kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const cudaError_t e = cudaFuncSetAttribute(rhs_fix_f64<N, XF, false>, kAttr, (int)fix_smem<N, false>());
+    const cudaError_t e = cudaFuncSetAttribute(rhs_fix_f64<N, VF, XF, false>, kAttr, (int)fix_smem<N, VF, false>());
     if constexpr (wide_upto(N) > 0)
-        if (e == cudaSuccess) return cudaFuncSetAttribute(rhs_fix_f64<N, XF, true>, kAttr, (int)fix_smem<N, true>());
+        if (e == cudaSuccess) return cudaFuncSetAttribute(rhs_fix_f64<N, VF, XF, true>, kAttr, (int)fix_smem<N, VF, true>());
     return e;
 }
-template <int N>
-cudaError_t prepare_n(bool xf) { return xf ? prepare_x<N, true>() : prepare_x<N, false>(); }
+
+template <int VF, bool XF>
+cudaError_t prepare_vf(const esdc_ctx* c) {
+    switch (c->N) {
+        case 2: return prepare_n<2, VF, XF>();
+        case 3: return prepare_n<3, VF, XF>();
+        case 4: return prepare_n<4, VF, XF>();
+        case 5: return prepare_n<5, VF, XF>();
+        case 6: return prepare_n<6, VF, XF>();
+        case 7: return prepare_n<7, VF, XF>();
+        case 8: return prepare_n<8, VF, XF>();
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <int VF, bool XF>
+cudaError_t launch_vf(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    switch (c->N) {
+        case 2: return launch_n<2, VF, XF>(c, q, dqdt, s);
+        case 3: return launch_n<3, VF, XF>(c, q, dqdt, s);
+        case 4: return launch_n<4, VF, XF>(c, q, dqdt, s);
+        case 5: return launch_n<5, VF, XF>(c, q, dqdt, s);
+        case 6: return launch_n<6, VF, XF>(c, q, dqdt, s);
+        case 7: return launch_n<7, VF, XF>(c, q, dqdt, s);
+        case 8: return launch_n<8, VF, XF>(c, q, dqdt, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
 
 }  // namespace
-
-cudaError_t prepare_rhs_fix(const esdc_ctx* c, bool xf) {
-    switch (c->N) {
-        case 2: return prepare_n<2>(xf);
-        case 3: return prepare_n<3>(xf);
-        case 4: return prepare_n<4>(xf);
-        case 5: return prepare_n<5>(xf);
-        case 6: return prepare_n<6>(xf);
-        case 7: return prepare_n<7>(xf);
-        case 8: return prepare_n<8>(xf);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-cudaError_t launch_rhs_fix(const esdc_ctx* c, bool xf, const double* q, double* dqdt, cudaStream_t s) {
-    switch (c->N) {
-        case 2: return launch_n<2>(c, xf, q, dqdt, s);
-        case 3: return launch_n<3>(c, xf, q, dqdt, s);
-        case 4: return launch_n<4>(c, xf, q, dqdt, s);
-        case 5: return launch_n<5>(c, xf, q, dqdt, s);
-        case 6: return launch_n<6>(c, xf, q, dqdt, s);
-        case 7: return launch_n<7>(c, xf, q, dqdt, s);
-        case 8: return launch_n<8>(c, xf, q, dqdt, s);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
 }  // namespace esdc

@@ -1,0 +1,11 @@
+// Fixed-point residual kernels: ES-C flux, with the optional interface terms.
+#include "rhs_fix.cuh"
+
+namespace esdc {
+
+cudaError_t prepare_fix_esc_xf(const esdc_ctx* c) { return prepare_vf<kFluxESC, true>(c); }
+cudaError_t launch_fix_esc_xf(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    return launch_vf<kFluxESC, true>(c, q, dqdt, s);
+}
+
+}  // namespace esdc

@@ -1,4 +1,4 @@
-"""The block fixed-point form of the ES-C residual (rhs_fix_f64.cu) where its rules change: elements
+"""The block fixed-point form of the float64 residual (csrc/rhs_fix.cuh) where its rules change: elements
 inside and outside the fixed-point range side by side, neighbours beyond the near and the far series of
 the logarithmic means, vanishing velocities, and partly filled CTAs at every degree (p = 1 to 3 put
 16, 4 and 2 elements in a CTA).  Bound: the float64 rounding bound of the other parity tests."""
@@ -12,8 +12,8 @@ from tests.gpu_common import assert_parity, make_pair
 pytestmark = pytest.mark.gpu
 
 
-def _case(p, kind, k=(3, 3, 3)):
-    solver, q, mesh, gas, qo = make_pair(p, k, warp=0.1, seed=2, Re=400.0, Ma=0.4)
+def _case(p, kind, k=(3, 3, 3), flux="esc"):
+    solver, q, mesh, gas, qo = make_pair(p, k, warp=0.1, seed=2, Re=400.0, Ma=0.4, volume_flux=flux)
     rng = np.random.default_rng(7 * p)
     x = qo.numpy().copy()
     rho, mom = x[:, 0], x[:, 1:4]
@@ -42,6 +42,14 @@ def _case(p, kind, k=(3, 3, 3)):
 def test_residual_parity_across_the_rules(p, kind):
     solver, q, mesh, gas, qo = _case(p, kind)
     assert_parity(solver.rhs(q), O.rhs(qo, mesh, gas), qo, mesh, gas)
+
+
+@pytest.mark.parametrize("kind", ["log", "range", "still"])
+@pytest.mark.parametrize("flux", ["kg", "dc"])
+@pytest.mark.parametrize("p", [1, 2, 4, 5, 6, 7])
+def test_variant_parity_across_the_rules(p, flux, kind):
+    solver, q, mesh, gas, qo = _case(p, kind, flux=flux)
+    assert_parity(solver.rhs(q), O.rhs(qo, mesh, gas, scheme=flux), qo, mesh, gas)
 
 
 @pytest.mark.parametrize("kind", ["far", "range"])
