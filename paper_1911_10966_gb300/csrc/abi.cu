@@ -487,6 +487,8 @@ int ensure_adjoint(esdc_ctx* c) {
     const size_t N2 = (size_t)c->N * c->N;
     CUDA_TRY(cudaMalloc(&c->d_adj_g, (size_t)c->K * 6 * 5 * N2 * sizeof(double)));
     CUDA_TRY(cudaMalloc(&c->d_adj_t, (size_t)c->K * 6 * 4 * N2 * sizeof(double)));
+    if (c->setup.volume_flux == ESDC_FLUX_ESC)
+        CUDA_TRY(cudaMalloc(&c->d_adj_pb, (size_t)c->K * 5 * c->N3 * sizeof(double)));
     CUDA_TRY(cudaMalloc(&c->d_adj_mu, esdc::adjoint_mu_blocks(c) * sizeof(double)));
     CUDA_TRY(cudaMalloc(&c->d_adj_acc, 8 * sizeof(double)));
     CUDA_TRY(esdc::prepare_adjoint(c));
@@ -536,6 +538,7 @@ void free_ctx(esdc_ctx* c) {
     cudaFree(c->d_stage_q);
     cudaFree(c->d_adj_g);
     cudaFree(c->d_adj_t);
+    cudaFree(c->d_adj_pb);
     cudaFree(c->d_adj_mu);
     cudaFree(c->d_adj_acc);
     cudaFree(c->d_stage_r);
@@ -768,6 +771,11 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
             for (int j = 0; j < hs.N; ++j)       // the rows of S sum to -E_ii/2
                 c->ops.MF[i][j] = esdc::fx_split(esdc::fx_from_double(
                     i != j ? c->ops.S[i][j] : (i == 0 ? 0.5 : (i == hs.N - 1 ? -0.5 : 0.0)), 1));
+        std::frexp(c->ops.winv[0], &c->ops.kW);          // the end weights are the smallest
+        for (int i = 0; i < hs.N; ++i) {
+            std::frexp(c->ops.winv[i], &c->ops.WE[i]);
+            c->ops.WB[i] = esdc::fx_split(esdc::fx_from_double(c->ops.winv[i], c->ops.kW));
+        }
         double dmax = 0.0;
         for (int i = 0; i < hs.N; ++i)
             for (int j = 0; j < hs.N; ++j) dmax = std::fmax(dmax, std::fabs(c->ops.D[i][j]));

@@ -31,6 +31,9 @@ struct Ops {
     FxPair SF[kMaxN / 2][kMaxN];
     FxPair CG;
     int kg;
+    FxPair WB[kMaxN];          // 1/w_i 2^-kW < 1
+    int WE[kMaxN];             // 1/w_i < 2^WE[i]
+    int kW;
     FxPair MF[kMaxN][kMaxN];   // S_ij / 2, on the diagonal half the row's sum 1/2, 0, .., -1/2 (DC)
     FxPair DF[kMaxN][kMaxN];   // D_ij 2^-kD
     FxPair LF;                 // interface lift 1/(2 w_0) 2^-kD
@@ -142,6 +145,7 @@ struct esdc_ctx {
     // adjoint buffers, allocated on the first vector-Jacobian product
     double* d_adj_g = nullptr;       // [K][6][5][N2] interface cotangents for the neighbour
     double* d_adj_t = nullptr;       // [K][6][4][N2] lifted-gradient cotangents for the neighbour
+    double* d_adj_pb = nullptr;      // [K][5][N3] cotangents of the volume term (ES-C)
     double* d_adj_mu = nullptr;      // per-block partial sums of lambda . R_visc
     double* d_adj_acc = nullptr;     // accumulated d/dmu
     // one DP5 step captured as a CUDA graph, replayed by multi-step esdc_rk_step calls; valid for

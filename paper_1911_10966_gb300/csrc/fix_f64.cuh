@@ -71,6 +71,14 @@ ESDC_HD long long fx_mul(Fx a, Fx b) {
     const long long t = mad_wide(a.l, b.h, mad_wide(a.h, b.l, kFxHalf + LL * kFxLow));
     return mad_wide(a.h, b.h, t >> 30);
 }
+// the same times 2^SH
+template <int LL, int SH>
+ESDC_HD long long fx_mul_shl(Fx a, Fx b) {
+    const long long t = mad_wide(a.l, b.h, mad_wide(a.h, b.l, (kFxHalf >> SH) + LL * kFxLow));
+    return (mul_wide(a.h, b.h) << SH) + (t >> (30 - SH));
+}
+// v 2^-s rounded to nearest, h half a unit
+ESDC_HD long long fx_shr(long long v, int s, long long h) { return (v + h) >> s; }
 // a b + c d with one shared alignment shift
 template <int LL = 2>
 ESDC_HD long long fx_mul2(Fx a, Fx b, Fx c, Fx d) {
@@ -355,46 +363,62 @@ struct PrimFx {
 // Series of the logarithmic means in u = f^2, f = (a - b)/(a + b):
 //   artanh(f)/f = F(u) = sum u^k/(2k+1)      and      1/F(u) = G(u) = 1 - sum g_k u^k
 // (g_k by inverting the first series term by term: 1/3, 4/45, 44/945, 428/14175, ...).  Both are
-// 1 +- u P(u), and u P(u) in Q60 is what these return.  Terms are kept until their weight at the end of
-// the range is below 2^-58.
-
-// u < 2^-13 (neighbours within 2%): P = c1 + u c2 + u^2 c3, of which 32 bits beyond c1 reach 2^-58
-template <bool LOGF>
-ESDC_HD long long fx_series_near(long long u) {
-    constexpr Fx D1 = {357913941, 357913941};                        // 1/3
-    constexpr unsigned c2 = LOGF ? 858993459u : 381774871u;          // 1/5 or 4/45, units of 2^-32
-    constexpr unsigned c3 = LOGF ? 613566757u : 199977313u;          // 1/7 or 44/945
-    const unsigned us = (unsigned)(u >> 15);                         // units of 2^-45
-    const unsigned t = mul_hi_u32(us, c2 + (mul_hi_u32(us, c3) >> 13));
-    return fx_mul(fx_split(u), Fx{D1.h + (int)(t >> 15), D1.l + (int)((t & 0x7fffu) << 15)});
+// 1 +- u P(u); their derivatives are +- series of the same kind with coefficients k/(2k+1) and k g_k.  All four
+// P start with 1/3.  Terms are kept until their weight at the end of the range is below 2^-58.
+enum : int { kSerG = 0, kSerF = 1, kSerDG = 2, kSerDF = 3 };
+struct SeriesFx {
+    Fx d[3];                 // c_1 .. c_3 in Q60
+    unsigned c[8];           // c_2 .. c_9 in units of 2^-32
+};
+template <int SET>
+ESDC_HD constexpr SeriesFx series_fx() {
+    constexpr SeriesFx t[4] = {
+        {{{357913941, 357913941}, {95443717, 739688812}, {49994328, 336325481}}, {381774871u, 199977313u, 129682258u, 93616560u, 72101986u, 57993934u, 48119721u, 40871223u}},
+        {{{357913941, 357913941}, {214748364, 858993459}, {153391689, 153391689}}, {858993459u, 613566757u, 477218588u, 390451572u, 330382100u, 286331153u, 252645135u, 226050910u}},
+        {{{357913941, 357913941}, {190887435, 405635800}, {149982984, 1008976444}}, {763549742u, 599931940u, 518729031u, 468082802u, 432611917u, 405957540u, 384957769u, 367841008u}},
+        {{{357913941, 357913941}, {429496729, 644245094}, {460175067, 460175067}}, {1717986918u, 1840700270u, 1908874354u, 1952257862u, 1982292598u, 2004318071u, 2021161080u, 2034458193u}}};
+    return t[SET];
 }
 
-// u < 2^-6 (within 28%): Horner, the terms of weight u^4 and beyond in 32 bits; u' = 2^6 u
-template <bool LOGF>
-ESDC_HD long long fx_series_far(long long u) {
-    constexpr unsigned C4 = LOGF ? 477218588u : 129682258u;          // 1/9           428/14175
-    constexpr unsigned C5 = LOGF ? 390451572u : 93616560u;           // 1/11          10196/467775
-    constexpr unsigned C6 = LOGF ? 330382100u : 72101986u;           // 1/13          10719068/638512875
-    constexpr unsigned C7 = LOGF ? 286331153u : 57993934u;           // 1/15          25865068/1915538625
-    constexpr unsigned C8 = LOGF ? 252645135u : 48119721u;           // 1/17          5472607916/488462349375
-    constexpr unsigned C9 = LOGF ? 226050910u : 40871223u;           // 1/19          74185965772/7795859096025
-    constexpr Fx D1 = {357913941, 357913941};
-    constexpr Fx D2 = LOGF ? Fx{214748364, 858993459} : Fx{95443717, 739688812};
-    constexpr Fx D3 = LOGF ? Fx{153391689, 153391689} : Fx{49994328, 336325481};
+// P for u < 2^-13 (neighbours within 2%): c1 + u c2 + u^2 c3, of which 32 bits beyond c1 reach 2^-58 in u P
+template <int SET>
+ESDC_HD Fx fx_poly_near(long long u) {
+    constexpr SeriesFx S = series_fx<SET>();
+    const unsigned us = (unsigned)(u >> 15);                         // units of 2^-45
+    const unsigned t = mul_hi_u32(us, S.c[0] + (mul_hi_u32(us, S.c[1]) >> 13));
+    return Fx{S.d[0].h + (int)(t >> 15), S.d[0].l + (int)((t & 0x7fffu) << 15)};
+}
+
+// The same with one more term and a full product, where P itself counts (the derivatives take f P, f < 2^-6.5)
+template <int SET>
+ESDC_HD Fx fx_poly_near_full(long long u) {
+    constexpr SeriesFx S = series_fx<SET>();
+    const unsigned us = (unsigned)(u >> 15);                         // units of 2^-45
+    const unsigned t = mul_hi_u32(us, S.c[1] + (mul_hi_u32(us, S.c[2]) >> 13));
+    const long long v = fx_mul(fx_split(u), Fx{S.d[1].h + (int)(t >> 15), S.d[1].l + (int)((t & 0x7fffu) << 15)});
+    return Fx{S.d[0].h + (int)(v >> 30), S.d[0].l + ((int)v & 0x3fffffff)};
+}
+
+// P for u < 2^-6 (within 28%): Horner, the terms of weight u^4 and beyond in 32 bits; u' = 2^6 u
+template <int SET>
+ESDC_HD Fx fx_poly_far(long long u) {
+    constexpr SeriesFx S = series_fx<SET>();
     const unsigned us = (unsigned)(u >> 22);                         // u' in units of 2^-32
-    unsigned t = C9;
-    t = C8 + (mul_hi_u32(us, t) >> 6);
-    t = C7 + (mul_hi_u32(us, t) >> 6);
-    t = C6 + (mul_hi_u32(us, t) >> 6);
-    t = C5 + (mul_hi_u32(us, t) >> 6);
+    unsigned t = S.c[7];
+#pragma unroll
+    for (int k = 6; k >= 3; --k) t = S.c[k] + (mul_hi_u32(us, t) >> 6);
     t = mul_hi_u32(us, t);
-    const unsigned long long p4 = ((unsigned long long)C4 << 28) + ((unsigned long long)t << 22);
+    const unsigned long long p4 = ((unsigned long long)S.c[2] << 28) + ((unsigned long long)t << 22);
     const Fx uf = fx_split(u << 6);
     long long v = fx_mul(uf, fx_split((long long)p4)) >> 6;
-    v = fx_mul(uf, Fx{D3.h + (int)(v >> 30), D3.l + ((int)v & 0x3fffffff)}) >> 6;
-    v = fx_mul(uf, Fx{D2.h + (int)(v >> 30), D2.l + ((int)v & 0x3fffffff)}) >> 6;
-    return fx_mul(uf, Fx{D1.h + (int)(v >> 30), D1.l + ((int)v & 0x3fffffff)}) >> 6;
+    v = fx_mul(uf, Fx{S.d[2].h + (int)(v >> 30), S.d[2].l + ((int)v & 0x3fffffff)}) >> 6;
+    v = fx_mul(uf, Fx{S.d[1].h + (int)(v >> 30), S.d[1].l + ((int)v & 0x3fffffff)}) >> 6;
+    return Fx{S.d[0].h + (int)(v >> 30), S.d[0].l + ((int)v & 0x3fffffff)};
 }
+template <int SET>
+ESDC_HD long long fx_series_near(long long u) { return fx_mul(fx_split(u), fx_poly_near<SET>(u)); }     // u P
+template <int SET>
+ESDC_HD long long fx_series_far(long long u) { return fx_mul(fx_split(u), fx_poly_far<SET>(u)); }
 
 constexpr long long kFxSeriesEnd = 1ll << 54;     // u = 2^-6
 constexpr int kFxNear = 2965790;                  // high word of f = 2^-6.5 in Q60, less a part in 10^5
@@ -406,10 +430,10 @@ ESDC_HD void log_means_far(Fx sh, Fx dh, Fx db, Fx rs, Fx g, const FixScale& s, 
                            long long& A) {
     const Fx fr = fx_split(fx_mul<0>(dh, fx_split(fx_rcp(sh, s.fr, s.ir))) << s.ir);
     const long long ur = mad_wide(fr.h, fr.h, mul_wide(fr.h, fr.l) >> 29);
-    rl = ur < kFxSeriesEnd ? fx_join(sh) - fx_mul<2>(sh, fx_split(fx_series_far<false>(ur))) : lm.rho();
+    rl = ur < kFxSeriesEnd ? fx_join(sh) - fx_mul<2>(sh, fx_split(fx_series_far<kSerG>(ur))) : lm.rho();
     const Fx fb = fx_split(fx_mul<0>(db, rs) << s.ib);
     const long long ub = mad_wide(fb.h, fb.h, mul_wide(fb.h, fb.l) >> 29);
-    A = ub < kFxSeriesEnd ? fx_join(g) + fx_mul(g, fx_split(fx_series_far<true>(ub))) : lm.inv_beta();
+    A = ub < kFxSeriesEnd ? fx_join(g) + fx_mul(g, fx_split(fx_series_far<kSerF>(ub))) : lm.inv_beta();
 }
 
 // The Chandrashekar flux of flux_f64.cuh (ec_flux) in block fixed point, contracted with n: f[0] in
@@ -431,7 +455,7 @@ ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, F
         fh = f0;
         const Fx ff = fx_split(f0 + (mul_wide((int)(f0 >> 24), e) >> 20));
         const long long u = mad_wide(ff.h, ff.h, mul_wide(ff.h, ff.l) >> 29);
-        rl = fx_join(sh) - fx_mul<2>(sh, fx_split(fx_series_near<false>(u)));
+        rl = fx_join(sh) - fx_mul<2>(sh, fx_split(fx_series_near<kSerG>(u)));
     }
     // 1/(sum of betas), and inv_gm1/beta_ln = inv_gm1 rsb F(u)
     const Fx sb = fx_add(a.b, b.b), db = fx_sub(a.b, b.b);
@@ -442,7 +466,7 @@ ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, F
     {
         const Fx ff = fx_split(fb);
         const long long u = mad_wide(ff.h, ff.h, mul_wide(ff.h, ff.l) >> 29);
-        A = fx_join(g) + fx_mul(g, fx_split(fx_series_near<true>(u)));
+        A = fx_join(g) + fx_mul(g, fx_split(fx_series_near<kSerF>(u)));
     }
     const int ir = (int)(fh >> 32), ib = (int)(fb >> 32);
     if ((unsigned)(ir + kFxNear) >= 2u * kFxNear || (unsigned)(ib + kFxNear) >= 2u * kFxNear)
@@ -486,6 +510,180 @@ ESDC_HD void euler_flux_fx(const PrimFx& a, Fx n0, Fx n1, Fx n2, const FixScale&
     f[2] = fx_mul2(fa, a.u1, pa, n1);
     f[3] = fx_mul2(fa, a.u2, pa, n2);
     f[4] = fx_mul(fx_split(f1), a.q);
+}
+
+// ---- reverse of the Chandrashekar flux
+
+// Exponents and alignment shifts of an element's pair reverse.  Cotangents mu (differences of the nodes'
+// lambda/(J w), |mu| < 1/4): l0, l1, l4 of the mass, momentum and energy components.  A smooth lambda's
+// differences, and what cancels in mu0 + fmb.ubar for a kinetic-energy functional, leave results far below any
+// bound known beforehand: each pair shifts its mu up to the largest, products keep their own exponents, and the
+// results are summed in float64, whose pipe is idle otherwise.  Bounds with n' = S_ij (n_i + n_j): fmb < 3/8,
+// f1b < 1.1, ptb < 1.13 (doubled), An < 1.4, the other operands as in the flux.
+struct AdjScale {
+    int l0, l1, l4;
+    int t4;                      // energy component into fmb
+    int s4, sF;                  // its product with the energy coefficient, that of fmb with ubar, into f1b
+    int a1, a2;                  // mu4 p_t and f1b rho_ln into An
+    int m4;                      // smallest shift of the energy component
+    int dp;                      // relative pressure jumps < 2^-dp
+    int kx, kz;                  // x: f1b un's part, the pressure jump's
+    int kf, ka;                  // velocity: f1 (mu5 ubar + fmb) and An n
+    int kb, kp;                  // beta: c5b's and p_t's part
+    int kc;                      // energy coefficient
+    int kd;                      // d(inv_gm1/(2 beta_ln))/d beta in Q60
+    int kA;                      // inv_gm1/(2 beta_ln)
+    long long hF, h4;            // half a unit of sF, s4
+};
+// E0, E1, E4: biased exponents that bound lambda/(J w)'s components; pmin, pmax: high words of the smallest and
+// largest pressure, whose difference bounds the relative pressure jump by 2^-dp (a step of the high word is at
+// most 2^-19 of the value below it)
+ESDC_HD AdjScale adj_scale(const FixScale& s, int E0, int E1, int E4, int pmin, int pmax) {
+    AdjScale t;
+    t.dp = 0;
+    for (int d = pmax - pmin + 1; t.dp < 19 && (d >> (18 - t.dp)) == 0;) ++t.dp;
+    t.l0 = E0 - 1019;
+    t.l1 = E1 - 1019;
+    t.l4 = E4 - 1019;
+    const int kc = fx_max(s.kA, s.kq), kp = s.kr + s.ib - s.kb;
+    const int ef = fx_max(t.l1, t.l4 + s.ku);
+    t.t4 = fx_clamp(ef - (t.l4 + s.ku));
+    t.l1 = ef;                                       // converted at fmb's exponent
+    const int eb = fx_max(t.l0, fx_max(t.l4 + kc, ef + s.ku));
+    t.l0 = eb;                                       // converted at f1b's
+    t.s4 = fx_clamp(eb - (t.l4 + kc));
+    t.sF = fx_clamp(eb - (ef + s.ku));
+    const int ea = fx_max(t.l4 + kp, eb + s.kr);
+    t.a1 = fx_clamp(ea - (t.l4 + kp));
+    t.a2 = fx_clamp(ea - (eb + s.kr));
+    t.m4 = -fx_max(-t.t4, fx_max(-t.s4, -t.a1));
+    const int ep = ef + s.kn - 1 + s.ib - s.kb;      // p_t's cotangent / (sum of betas)
+    t.kc = t.l4 + s.k0;
+    t.kd = s.kA + s.ib - s.kb;
+    t.kA = s.kA;
+    t.kx = eb + s.ku + s.kn - 1 + s.kr;
+    t.kz = ep + s.kr + s.ib - t.dp;
+    t.kf = s.k0 + ef;
+    t.ka = ea + s.kn;
+    t.kb = t.kc + t.kd;
+    t.kp = kp + ep;
+    t.hF = (1ll << t.sF) >> 1;
+    t.h4 = (1ll << t.s4) >> 1;
+    return t;
+}
+
+// The logarithmic means of a pair with their derivatives: rl and A as in ec_flux_fx, La, Lb = d rho_ln / d rho_a,
+// d rho_b, DA, DB = d (inv_gm1/(2 beta_ln)) / d beta_a, d beta_b in units 2^kd
+struct LogMeansFx {
+    long long rl, La, Lb, A, DA, DB;
+};
+// FAR: the far series.  With f, u = f^2: rho_ln = (a + b) G/2, d/da = G/2 - W + W f, d/db = G/2 + W + W f,
+// W = -f G'(u); 1/beta_ln = 2 F/(a + b), d/da = 2 (w - w f - F)/(a + b)^2, d/db = -2 (w + w f + F)/(a + b)^2,
+// w = 2 f F'(u).
+template <bool FAR>
+ESDC_HD void rho_mean_fx(Fx sh, long long fr, LogMeansFx& m) {
+    const Fx f = fx_split(fr);
+    const long long u = mad_wide(f.h, f.h, mul_wide(f.h, f.l) >> 29);
+    const Fx P = FAR ? fx_poly_far<kSerG>(u) : fx_poly_near<kSerG>(u), V = FAR ? fx_poly_far<kSerDG>(u) : fx_poly_near_full<kSerDG>(u);
+    const long long uP = fx_mul(fx_split(u), P);
+    m.rl = fx_join(sh) - fx_mul<2>(sh, fx_split(uP));
+    const long long W = fx_mul(f, V), Y = (((1ll << 60) - uP + 1) >> 1) + fx_mul(f, fx_split(W));
+    m.La = Y - W;
+    m.Lb = Y + W;
+}
+template <bool FAR>
+ESDC_HD void beta_mean_fx(Fx rs, Fx g, long long fb, LogMeansFx& m) {
+    const Fx f = fx_split(fb);
+    const long long u = mad_wide(f.h, f.h, mul_wide(f.h, f.l) >> 29);
+    const Fx P = FAR ? fx_poly_far<kSerF>(u) : fx_poly_near<kSerF>(u), V = FAR ? fx_poly_far<kSerDF>(u) : fx_poly_near_full<kSerDF>(u);
+    const long long uP = fx_mul(fx_split(u), P);
+    m.A = fx_join(g) + fx_mul(g, fx_split(uP));
+    const long long w = fx_mul(f, V) << 1, X = fx_mul(f, fx_split(w)) + (1ll << 60) + uP;
+    const Fx T = fx_split(fx_mul(g, rs));
+    m.DA = fx_mul(T, fx_split(w - X));
+    m.DB = -fx_mul(T, fx_split(w + X));
+}
+template <typename LogMean>
+ESDC_HD void adj_means_far(long long fr, long long fb, Fx sh, Fx rs, Fx g, const LogMean& lm, LogMeansFx& m) {
+    const int ir = (int)(fr >> 32), ib = (int)(fb >> 32), end = 1 << 25;      // f = 2^-3
+    if ((unsigned)(ir + end) < 2u * end) rho_mean_fx<true>(sh, fr, m);
+    else lm.rho(m);
+    if ((unsigned)(ib + end) < 2u * end) beta_mean_fx<true>(rs, g, fb, m);
+    else lm.beta(m);
+}
+
+struct PairBarFx {
+    double xa, xb, ba, bb, u[3], c;
+};
+
+// v 2^-r for r of either sign
+ESDC_HD long long fx_shift(long long v, int r) { return r >= 0 ? v >> r : v << -r; }
+// left shift that brings a magnitude (top bit `a`) to just below 2^top
+ESDC_HD int fx_norm(unsigned long long a, int top) {
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((long long)(a | 1));
+#else
+    const int z = __builtin_clzll(a | 1);
+#endif
+    return fx_max(z - (64 - top), 0);
+}
+ESDC_HD unsigned long long fx_mag(long long v) { return (unsigned long long)(v ^ (v >> 63)); }
+
+// Reverse of f(a, b; n) for the cotangent mu (mu[0] in units 2^l0, mu[1..3] 2^l1, mu[4] 2^l4): the two nodes' x =
+// rho rho-bar + beta beta-bar (the density cotangent at constant pressure, times rho) and beta cotangents, their
+// common doubled velocity cotangent and that of the energy coefficient, as ec_pair_vjp gives them.  p_t's parts of
+// rho-bar and beta-bar cancel in x up to the pressure jump, which is formed directly.
+template <typename LogMean>
+ESDC_HD void ec_pair_vjp_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, const long long (&mu)[5], Fx cg,
+                            const FixScale& s, const AdjScale& t, const LogMean& lm, PairBarFx& o) {
+    const Fx sh = fx_add(a.r, b.r), sb = fx_add(a.b, b.b);
+    const Fx rs = fx_split(fx_rcp(sb, s.fb, s.ib));
+    const Fx g = fx_split(fx_mul(rs, cg));
+    const long long fr = fx_mul<0>(fx_sub(a.r, b.r), fx_split(fx_rcp(sh, s.fr, s.ir))) << s.ir;
+    const long long fb = fx_mul<0>(fx_sub(a.b, b.b), rs) << s.ib;
+    LogMeansFx m;
+    rho_mean_fx<false>(sh, fr, m);
+    beta_mean_fx<false>(rs, g, fb, m);
+    const int ir = (int)(fr >> 32), ib = (int)(fb >> 32);
+    if ((unsigned)(ir + kFxNear) >= 2u * kFxNear || (unsigned)(ib + kFxNear) >= 2u * kFxNear)
+        adj_means_far(fr, fb, sh, rs, g, lm, m);
+    const Fx rl = fx_split(m.rl);
+    const Fx v0 = fx_add(a.u0, b.u0), v1 = fx_add(a.u1, b.u1), v2 = fx_add(a.u2, b.u2);
+    // ubar.n' and the mass flux, shifted up by nu
+    const long long unl = fx_dot_shl<6, 1>(v0, n0, v1, n1, v2, n2);
+    const int nu = fx_norm(fx_mag(unl), 60);
+    const Fx un = fx_split(unl << nu), f1 = fx_split(fx_mul(rl, un));
+    const Fx pt = fx_split(fx_mul<2>(sh, rs));
+    const Fx c5 = fx_split((m.A >> s.sc) - (fx_join(fx_add(a.q, b.q)) >> s.sq));
+    // cotangents of the momentum flux, fmb = mu5 ubar + mu, and mu5 ubar + fmb, shifted up by ns
+    const int ns = fx_norm(fx_mag(mu[0]) | fx_mag(mu[1]) | fx_mag(mu[2]) | fx_mag(mu[3]) | (fx_mag(mu[4]) >> t.m4), 58);
+    const Fx mu4 = fx_split(mu[4]), m4 = fx_split(fx_shift(mu[4], t.t4 - ns));
+    const long long w0 = fx_mul<2>(m4, v0), w1 = fx_mul<2>(m4, v1), w2 = fx_mul<2>(m4, v2);
+    const long long g0 = w0 + (mu[1] << ns), g1 = w1 + (mu[2] << ns), g2 = w2 + (mu[3] << ns);
+    const Fx q0 = fx_split(g0), q1 = fx_split(g1), q2 = fx_split(g2);
+    const long long f1bl = (mu[0] << ns) + fx_shift(fx_mul(mu4, c5), t.s4 - ns)
+                         + fx_shr(fx_dot<6>(v0, q0, v1, q1, v2, q2), t.sF, t.hF);
+    const Fx c5b = fx_split(fx_mul(mu4, f1));
+    const Fx ptr = fx_split(fx_mul(fx_split(fx_dot_shl<3, 1>(q0, n0, q1, n1, q2, n2)), rs));
+    o.c = fx_to_double(fx_join(c5b), t.kc - nu);
+    // x: f1b un rho d rho_ln + c5b beta d A + ptr (rho_a beta_b - rho_b beta_a)/(2 (sum of betas)); the means are
+    // homogeneous, rho_a La + rho_b Lb = rho_ln and beta_a DA + beta_b DB = -A
+    const int nf = fx_norm(fx_mag(f1bl), 60);
+    const Fx Lb = fx_split(fx_mul(fx_split(f1bl << nf), un));
+    const long long X = fx_mul_shl<1, 1>(a.r, fx_split(m.La)), Y = fx_mul(a.b, fx_split(m.DA)) << s.ib;
+    const long long cr = fx_mul2<2>(a.r, b.b, Fx{-b.r.h, -b.r.l}, a.b);
+    const double z = fx_to_double(fx_mul(ptr, fx_split(fx_mul(fx_split(cr << t.dp), rs))), t.kz - ns);
+    const int kx = t.kx - nf - nu - ns, kA = t.kc - nu + t.kA;
+    o.xa = fx_to_double(fx_mul(Lb, fx_split(X)), kx) + (fx_to_double(fx_mul(c5b, fx_split(Y)), kA) + z);
+    o.xb = fx_to_double(fx_mul(Lb, fx_split(m.rl - X)), kx) - (fx_to_double(fx_mul(c5b, fx_split(m.A + Y)), kA) + z);
+    const double bp = fx_to_double(fx_mul(pt, ptr), t.kp - ns);
+    o.ba = fx_to_double(fx_mul(c5b, fx_split(m.DA)), t.kb - nu) - bp;
+    o.bb = fx_to_double(fx_mul(c5b, fx_split(m.DB)), t.kb - nu) - bp;
+    const Fx An = fx_split(fx_shift(fx_mul(mu4, pt), t.a1 - ns) + (fx_mul(fx_split(f1bl), rl) >> t.a2));
+    const int kf = t.kf - nu - ns, ka = t.ka - ns;
+    o.u[0] = fx_to_double(fx_mul(f1, fx_split(g0 + w0)), kf) + fx_to_double(fx_mul(An, n0), ka);
+    o.u[1] = fx_to_double(fx_mul(f1, fx_split(g1 + w1)), kf) + fx_to_double(fx_mul(An, n1), ka);
+    o.u[2] = fx_to_double(fx_mul(f1, fx_split(g2 + w2)), kf) + fx_to_double(fx_mul(An, n2), ka);
 }
 
 }  // namespace esdc

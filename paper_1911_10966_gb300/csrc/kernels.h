@@ -31,6 +31,9 @@ ESDC_FIX_DECL(kg_xf)
 ESDC_FIX_DECL(dc)
 ESDC_FIX_DECL(dc_xf)
 #undef ESDC_FIX_DECL
+// volume part of the ES-C adjoint (adj_pairs_fix.cu) into c->d_adj_pb
+cudaError_t prepare_adj_pairs(const esdc_ctx* c);
+cudaError_t launch_adj_pairs(const esdc_ctx* c, const double* q, const double* lam, cudaStream_t s);
 // the p = 15 float64 residual (N = kLargeN), called by the two above
 cudaError_t prepare_rhs_large(const esdc_ctx* c);
 cudaError_t launch_rhs_large(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s, cudaEvent_t* ev);
