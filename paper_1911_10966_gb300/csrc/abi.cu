@@ -795,6 +795,7 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
     c->phys.kappa = mu * cp / s.Pr;
     c->phys.inv_gm1 = 1.0 / (s.gamma - 1.0);
     c->phys.gm1 = s.gamma - 1.0;
+    c->phys.inv_gamma = 1.0 / s.gamma;
     c->phys.kappa_R = c->phys.kappa / R;
     c->phys.dissipation = s.dissipation;
     c->phys.viscous = mu > 0.0;

@@ -35,7 +35,7 @@ struct PRaw {
 __device__ __forceinline__ void ec_pair_vjp(const PrimH& a, const PrimH& b, double n0, double n1, double n2,
                                             const double mu[5], const Phys& ph, PRaw& ab, PRaw& bb) {
     const double sr = a.rho + b.rho, sb = a.beta + b.beta;
-    const double rsb = rcp_newton2(sb);
+    const double rsb = rcp_cubic(sb);
     // rho log mean and its partial derivatives
     double Lr, Lra, Lrb;
     {
@@ -51,8 +51,8 @@ __device__ __forceinline__ void ec_pair_vjp(const PrimH& a, const PrimH& b, doub
             Lra = hG - W + Y;
             Lrb = hG + W + Y;
         } else {
-            const double ra = rcp_newton2(a.rho), rb = rcp_newton2(b.rho);
-            const double rl = rcp_newton2(log(a.rho * rb));
+            const double ra = rcp_cubic(a.rho), rb = rcp_cubic(b.rho);
+            const double rl = rcp_cubic(log(a.rho * rb));
             Lr = d * rl;
             Lra = fma(-Lr, ra, 1.0) * rl;
             Lrb = fma(Lr, rb, -1.0) * rl;
@@ -74,8 +74,8 @@ __device__ __forceinline__ void ec_pair_vjp(const PrimH& a, const PrimH& b, doub
             Ab = w - X - F;
             Bb = -(w + X + F);
         } else {
-            const double ra = rcp_newton2(a.beta), rb = rcp_newton2(b.beta);
-            sc = rcp_newton2(d);
+            const double ra = rcp_cubic(a.beta), rb = rcp_cubic(b.beta);
+            sc = rcp_cubic(d);
             IB = log(a.beta * rb) * sc;
             Ab = ra - IB;
             Bb = IB - rb;

@@ -65,21 +65,21 @@ struct PBar {   // cotangents of (rho, u0, u1, u2, beta, usq)
 };
 
 __device__ __forceinline__ void to_prim(const double* q, const Phys& ph, Prim& s) {
-    const double ri = rcp_newton2(q[0]);
+    const double ri = rcp_cubic(q[0]);
     s.rho = q[0];
     s.u0 = q[1] * ri;
     s.u1 = q[2] * ri;
     s.u2 = q[3] * ri;
     s.usq = s.u0 * s.u0 + s.u1 * s.u1 + s.u2 * s.u2;
-    const double p = (ph.gamma - 1.0) * (q[4] - 0.5 * q[0] * s.usq);
-    s.beta = 0.5 * q[0] * rcp_newton2(p);
+    const double p = ph.gm1 * (q[4] - 0.5 * q[0] * s.usq);
+    s.beta = 0.5 * q[0] * rcp_cubic(p);
 }
 
 // pull a primitive cotangent back to the conserved variables at state s
 __device__ __forceinline__ void pbar_to_q(const Prim& s, const PBar& b, const Phys& ph, double qb[5]) {
-    const double gm1 = ph.gamma - 1.0;
+    const double gm1 = ph.gm1;
     const double ut0 = b.u0 + 2.0 * s.u0 * b.usq, ut1 = b.u1 + 2.0 * s.u1 * b.usq, ut2 = b.u2 + 2.0 * s.u2 * b.usq;
-    const double ri = rcp_newton2(s.rho);
+    const double ri = rcp_cubic(s.rho);
     // beta = rho/(2p): d beta = beta/rho d rho - beta/p d p, and beta/p = 2 beta^2/rho
     const double pb = -b.beta * 2.0 * s.beta * s.beta * ri;
     qb[0] = b.rho + b.beta * s.beta * ri + pb * gm1 * 0.5 * s.usq - (ut0 * s.u0 + ut1 * s.u1 + ut2 * s.u2) * ri;
@@ -145,7 +145,7 @@ __device__ __forceinline__ void ec_flux_vjp(const Prim& a, const Prim& b, double
 // f5 = f1 e_bar + p_bar u_bar.n.  Adds the primitive cotangents of both states to ab, bb.
 __device__ __forceinline__ void kg_flux_vjp(const Prim& a, const Prim& b, double n0, double n1, double n2,
                                             const double mu[5], const Phys& ph, PBar& ab, PBar& bb) {
-    const double RTa = 0.5 * rcp_newton2(a.beta), RTb = 0.5 * rcp_newton2(b.beta);
+    const double RTa = 0.5 * rcp_cubic(a.beta), RTb = 0.5 * rcp_cubic(b.beta);
     const double rb = 0.5 * (a.rho + b.rho);
     const double ub0 = 0.5 * (a.u0 + b.u0), ub1 = 0.5 * (a.u1 + b.u1), ub2 = 0.5 * (a.u2 + b.u2);
     const double pb = 0.5 * (a.rho * RTa + b.rho * RTb);
@@ -180,7 +180,7 @@ __device__ __forceinline__ void kg_flux_vjp(const Prim& a, const Prim& b, double
 // and H = gamma/(gamma-1) RT + |u|^2/2.  Adds the primitive cotangents of the state to sb.
 __device__ __forceinline__ void euler_flux_vjp(const Prim& s, double n0, double n1, double n2, const double mu[5],
                                                const Phys& ph, PBar& sb) {
-    const double RT = 0.5 * rcp_newton2(s.beta);
+    const double RT = 0.5 * rcp_cubic(s.beta);
     const double un = s.u0 * n0 + s.u1 * n1 + s.u2 * n2;
     const double H = ph.gamma * ph.inv_gm1 * RT + 0.5 * s.usq;
     const double A = s.rho * un;                                   // mass flux
@@ -419,7 +419,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
          const int32_t* __restrict__ nbr, double* __restrict__ grad, double* __restrict__ gbuf,
          double* __restrict__ tbuf, double* __restrict__ mupart, int64_t K, const Ops ops, const Phys ph,
          const double* __restrict__ nsurf, const double* __restrict__ qext, const double* __restrict__ fnorm,
-         const double* __restrict__ pbar) {
+         const double* __restrict__ pbar, const double* __restrict__ jinv) {
     constexpr int N2 = CfgA<N>::N2, N3 = CfgA<N>::N3, EPB = CfgA<N>::EPB;
     extern __shared__ double smem[];
     __shared__ double red[CfgA<N>::THREADS];
@@ -456,7 +456,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
         sP[9 * N3 + node] = -2.0 * s.beta;
 #pragma unroll
         for (int c = 0; c < 10; ++c) sG[c * N3 + node] = geom[(el * 10 + c) * N3 + node];
-        const double Jinv = rcp_newton2(sG[node]);
+        const double Jinv = jinv[el * N3 + node];
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
             sL[v * N3 + node] = lam[eoff + v * N3 + node] * Jinv;
@@ -555,7 +555,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
     // face buffer (sT, free until the viscous part), gathered per node below; the neighbour's
     // cotangents to gbuf
     double* sFo = sT;                                   // [5][6 N2]
-    const double igam = rcp_newton2(ph.gamma);
+    const double igam = ph.inv_gamma;
     if (active) {
 #pragma unroll 1
         for (int fn = node; fn < 6 * N2; fn += N3) {
@@ -694,7 +694,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
                     for (int k = 0; k < 4; ++k) th[a][k] += E * (wf[k * N2] - wown[k]) * ops.winv[ia];
                 }
             }
-            const double Jinv = rcp_newton2(sG[node]);
+            const double Jinv = jinv[el * N3 + node];
             double g[3][4];
 #pragma unroll
             for (int m = 0; m < 3; ++m)
@@ -703,7 +703,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
                     g[m][k] = Jinv * (sG[(1 + m) * N3 + node] * th[0][k] + sG[(4 + m) * N3 + node] * th[1][k] +
                                       sG[(7 + m) * N3 + node] * th[2][k]);
             const double beta = sP[4 * N3 + node];
-            const double RT = 0.5 * rcp_newton2(beta);
+            const double RT = 0.5 * rcp_cubic(beta);
             const double u[3] = {sP[N3 + node], sP[2 * N3 + node], sP[3 * N3 + node]};
             double du[3][3];
 #pragma unroll
@@ -711,7 +711,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
 #pragma unroll
                 for (int m = 0; m < 3; ++m) du[k][m] = RT * (g[m][k] + u[k] * g[m][3]);
             const double div = du[0][0] + du[1][1] + du[2][2];
-            const double hc = ph.kappa / ph.R * RT * RT;
+            const double hc = ph.kappa_R * RT * RT;
             double FV[3][4];
 #pragma unroll
             for (int m = 0; m < 3; ++m) {
@@ -739,7 +739,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
                     const int side = il == N - 1;
                     const int st2 = dir_stride<N>(l);
                     const int nbn = node + (side ? -(N - 1) * st2 : (N - 1) * st2);   // matching node in nb
-                    const double Jn = rcp_newton2(geom[nb * 10 * N3 + nbn]);
+                    const double Jn = jinv[nb * N3 + nbn];
                     const double E = side ? 0.5 : -0.5;
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
@@ -794,7 +794,7 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
                 for (int m = 0; m < 3; ++m) sdE = fma(du[k][m], E[k][m], sdE);
             }
             // hc = kappa/R RT^2: its cotangent reaches beta as hcb (kappa/R) 2 RT (-2 RT^2)
-            bb -= fma(4.0 * ph.kappa / ph.R * RT * RT * RT, hcb, 2.0 * sdE);
+            bb -= fma(4.0 * ph.kappa_R * RT * RT * RT, hcb, 2.0 * sdE);
             // g = J^-1 sum_a Ja_am theta_a  ->  theta-bar
 #pragma unroll
             for (int a = 0; a < 3; ++a)
@@ -858,13 +858,16 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
 #pragma unroll
         for (int v = 0; v < 5; ++v) grad[eoff + v * N3 + node] = qb[v] + sQ[v * N3 + node];
     }
-    // deterministic block sum of the mu cotangent (lambda . R_visc)
+    // block sum of the mu cotangent (lambda . R_visc) in a fixed order: one warp, its lanes over strides of 32,
+    // then halving (a single thread adding all of them took a tenth of a p = 7 element's time)
     red[t] = mu_acc;
     __syncthreads();
-    if (t == 0) {
+    if (t < 32) {
         double s = 0.0;
-        for (int i = 0; i < CfgA<N>::THREADS; ++i) s += red[i];
-        mupart[blockIdx.x] = s;
+        for (int i = t; i < CfgA<N>::THREADS; i += 32) s += red[i];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+        if (t == 0) mupart[blockIdx.x] = s;
     }
 }
 
@@ -947,17 +950,17 @@ cudaError_t launch_adj_n(const esdc_ctx* c, const double* q, const double* lam, 
     if (c->setup.volume_flux == ESDC_FLUX_KG) {
         adj_main<N, kAdjKG><<<grid, C::THREADS, smem, s>>>(q, lam, c->d_geom, c->d_nbr, grad, c->d_adj_g, c->d_adj_t,
                                                            c->d_adj_mu, c->K, c->ops, c->phys, c->d_nsurf, c->d_qext,
-                                                           c->d_fnorm, nullptr);
+                                                           c->d_fnorm, nullptr, c->d_jinv);
     } else if (c->setup.volume_flux == ESDC_FLUX_DC) {
         adj_main<N, kAdjDC><<<grid, C::THREADS, smem, s>>>(q, lam, c->d_geom, c->d_nbr, grad, c->d_adj_g, c->d_adj_t,
                                                            c->d_adj_mu, c->K, c->ops, c->phys, c->d_nsurf, c->d_qext,
-                                                           c->d_fnorm, nullptr);
+                                                           c->d_fnorm, nullptr, c->d_jinv);
     } else {
         const cudaError_t e = launch_adj_pairs(c, q, lam, s);
         if (e != cudaSuccess) return e;
         adj_main<N, kAdjESC><<<grid, C::THREADS, smem, s>>>(q, lam, c->d_geom, c->d_nbr, grad, c->d_adj_g, c->d_adj_t,
                                                             c->d_adj_mu, c->K, c->ops, c->phys, c->d_nsurf, c->d_qext,
-                                                            c->d_fnorm, c->d_adj_pb);
+                                                            c->d_fnorm, c->d_adj_pb, c->d_jinv);
     }
     adj_face<N><<<grid, C::THREADS, 0, s>>>(q, c->d_nbr, c->d_adj_g, c->d_adj_t, grad, c->K, c->ops, c->phys);
     if (mu_acc) {

@@ -52,7 +52,7 @@ struct OpsL {
 struct Phys {
     double gamma, R, mu, kappa;
     double inv_gm1;            // 1/(gamma-1)
-    double gm1, kappa_R;       // gamma - 1, kappa/R
+    double gm1, inv_gamma, kappa_R;       // gamma - 1, 1/gamma, kappa/R
     double ip_coef;            // interior-penalty coefficient (0: off)
     int dissipation;           // 0 none, 1 local Lax-Friedrichs, 2 matrix
     int viscous;               // mu > 0

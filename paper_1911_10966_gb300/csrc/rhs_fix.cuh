@@ -118,12 +118,7 @@ struct LogMeanF64 {
 };
 
 // Primitives as in to_prim, with the float64 operations that can go to the integer pipe there: halving
-// is an exponent decrement (zeros, infinities and NaNs end up out of the fixed-point range), and the
-// reciprocals take r (1 + e + e^2), e = 1 - x r, from the 2^-23 approximation r.
-__device__ __forceinline__ double rcp_cubic(double x) {
-    const double r = rcp_approx(x), e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
+// is an exponent decrement (zeros, infinities and NaNs end up out of the fixed-point range).
 __device__ __forceinline__ double half_of(double x) { return __hiloint2double(__double2hiint(x) - (1 << 20), __double2loint(x)); }
 __device__ __forceinline__ void to_prim_fx(const double* q, const Phys& ph, Prim& s, double& RT) {
     const double ri = rcp_cubic(q[0]), rh = half_of(ri);

@@ -286,7 +286,7 @@ lg_viscous(const double* __restrict__ q, const double* __restrict__ geom, const 
 #pragma unroll
             for (int m = 0; m < 3; ++m) du[k][m] = RT * (g[m][k] + u[k] * g[m][3]);
         const double div = du[0][0] + du[1][1] + du[2][2];
-        const double hc = ph.kappa / ph.R * RT * RT;
+        const double hc = ph.kappa_R * RT * RT;
         double FV[3][4];
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
