@@ -53,8 +53,10 @@ struct CfgA {
     // | neighbour face w 24 N2
     static constexpr int TSZ = 12 * N3 > 30 * N2 ? 12 * N3 : 30 * N2;
     static constexpr int SM = 36 * N3 + TSZ + 24 * N2;
-    // resident CTAs the register allocation is sized for (3 at N = 4, 5 measured faster than 2)
-    static constexpr int MINB = (N == 4 || N == 5) ? 3 : 1;
+    // resident CTAs the register allocation is sized for: four at N = 4, 5 hold 512 elements in one wave (VJP at
+    // p = 4, three against four: 8^3 elements 231 -> 218 us, 16^3 1.379 -> 1.375 ms), two at N = 6 (14^3 1.89 ->
+    // 1.84 ms; two at N = 7 lose, 1.87 -> 1.88 ms on 12^3)
+    static constexpr int MINB = (N == 4 || N == 5) ? 4 : (N == 6 ? 2 : 1);
 };
 
 struct Prim {
