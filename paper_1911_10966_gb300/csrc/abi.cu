@@ -524,7 +524,6 @@ void free_ctx(esdc_ctx* c) {
     cudaFree(c->d_fnorm);
     cudaFree(c->d_nsurf);
     cudaFree(c->d_lr);
-    cudaFree(c->d_lwf);
     cudaFree(c->d_lft);
     cudaFree(c->d_geomf);
     cudaFree(c->d_nsurff);
@@ -786,6 +785,20 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
         c->ops.LF = esdc::fx_split(esdc::fx_from_double(0.5 * c->ops.winv[0], c->ops.kD));
     }
     c->ops.CG = esdc::fx_split(esdc::fx_from_double(std::frexp(1.0 / (s.gamma - 1.0), &c->ops.kg), 0));
+    c->opsl.CG = c->ops.CG;
+    c->opsl.kg = c->ops.kg;
+    if (hs.N == esdc::kLargeN) {
+        double dmax = 0.0;
+        for (double d : hs.D) dmax = std::fmax(dmax, std::fabs(d));
+        std::frexp(dmax, &c->opsl.kD);
+        for (int i = 0; i < hs.N; ++i) {
+            for (int k = 1; k <= hs.N / 2; ++k)
+                c->opsl.SF[k - 1][i] = esdc::fx_split(esdc::fx_from_double(c->opsl.S[i][(i + k) % hs.N], 0));
+            for (int j = 0; j < hs.N; ++j)
+                c->opsl.DF[i][j] = esdc::fx_split(esdc::fx_from_double(c->opsl.D[i][j], c->opsl.kD));
+        }
+        c->opsl.LF = esdc::fx_split(esdc::fx_from_double(0.5 * c->opsl.winv[0], c->opsl.kD));
+    }
     const double R = 1.0 / (s.gamma * s.Ma * s.Ma);
     const double mu = s.Re > 0.0 ? 1.0 / s.Re : 0.0;
     const double cp = s.gamma * R / (s.gamma - 1.0);
@@ -845,7 +858,6 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
     }
     if (e == cudaSuccess && hs.N == esdc::kLargeN) {
         e = cudaMalloc(&c->d_lr, (size_t)3 * c->n_nodes * 5 * sizeof(double));
-        if (e == cudaSuccess) e = cudaMalloc(&c->d_lwf, (size_t)c->K * 6 * 4 * N2 * sizeof(double));
         if (e == cudaSuccess) e = cudaMalloc(&c->d_lft, (size_t)c->K * 3 * 4 * c->N3 * sizeof(double));
     }
     if (e == cudaSuccess) {

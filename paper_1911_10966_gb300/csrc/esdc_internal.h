@@ -47,6 +47,11 @@ struct OpsL {
     double S[kLargeN][kLargeN];
     double w[kLargeN];
     double winv[kLargeN];
+    FxPair SF[kLargeN / 2][kLargeN];      // as in Ops
+    FxPair CG;
+    FxPair DF[kLargeN][kLargeN];
+    FxPair LF;
+    int kg, kD;
 };
 
 struct Phys {
@@ -128,8 +133,7 @@ struct esdc_ctx {
     double* d_nsurf = nullptr;       // [K][6][3][N2] surface metrics of the optimized metrics (else null)
     // p = 15 residual passes (N = kLargeN only)
     double* d_lr = nullptr;          // [3][K][5][N3] per-direction residual parts
-    double* d_lwf = nullptr;         // [K][6][4][N2] neighbour entropy variables at the faces
-    double* d_lft = nullptr;         // [K][3][4][N3] contravariant viscous fluxes
+    double* d_lft = nullptr;         // [K][3][4][N3] theta, then the contravariant viscous fluxes
     const double* d_qext = nullptr;  // caller-owned exterior (Dirichlet) state, [K][5][N3] (bounded boxes)
     const double* d_src = nullptr;   // caller-owned source term added to dq/dt, [K][5][N3]
     float* d_geomf = nullptr;        // [K][10][N3] float32 copy (mixed precision)

@@ -288,8 +288,8 @@ ESDC_HD FixScale fix_scale_kg(int Er, int Eu, int Eb, int En, int Ey, int Ez, in
     s.sB = fx_clamp(s.km - kb);
     const int kC = s.k0 + s.kq, kM = s.kp + s.ku + s.kn - 1;
     s.k5 = fx_max(kC, kM) + 1;
-    s.sC = fx_clamp(s.k5 - kC);
-    s.sD = fx_clamp(s.k5 - kM);
+    s.sC = fx_clamp(s.k5 - 1 - kC);              // the sum's last bit is rounded off once (kg_flux_fx)
+    s.sD = fx_clamp(s.k5 - 1 - kM);
     s.hC = (1ll << s.sC) >> 1;
     s.hD = (1ll << s.sD) >> 1;
     s.ky = Ey - 1021;
@@ -497,7 +497,7 @@ ESDC_HD void kg_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, c
     f[1] = fx_mul2<3>(fa, v0, pa, n0);
     f[2] = fx_mul2<3>(fa, v1, pa, n1);
     f[3] = fx_mul2<3>(fa, v2, pa, n2);
-    f[4] = ((fx_mul<2>(fx_split(f1), fx_add(a.q, b.q)) + s.hC) >> s.sC) + ((fx_mul<2>(pt, un) + s.hD) >> s.sD);
+    f[4] = (((fx_mul<2>(fx_split(f1), fx_add(a.q, b.q)) + s.hC) >> s.sC) + ((fx_mul<2>(pt, un) + s.hD) >> s.sD) + 1) >> 1;
 }
 
 // The Euler flux of one node contracted with n (euler_flux_prim), units as above

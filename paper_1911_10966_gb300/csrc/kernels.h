@@ -35,7 +35,6 @@ ESDC_FIX_DECL(dc_xf)
 cudaError_t prepare_adj_pairs(const esdc_ctx* c);
 cudaError_t launch_adj_pairs(const esdc_ctx* c, const double* q, const double* lam, cudaStream_t s);
 // the p = 15 float64 residual (N = kLargeN), called by the two above
-cudaError_t prepare_rhs_large(const esdc_ctx* c);
 cudaError_t launch_rhs_large(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s, cudaEvent_t* ev);
 
 // out = q0 + sum_j coef[j] * k[j]   (n doubles; k pointers may alias nothing but each other)

@@ -165,8 +165,8 @@ __device__ __forceinline__ void pair_exponents(const double (&pi)[NP], int (&E)[
 }
 // the element's scales from its maxima
 template <int VF, int NE>
-__device__ __forceinline__ FixScale element_scale(const int (&E)[NE], const Ops& ops) {
-    if constexpr (VF == kFluxESC) return fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], ops.kg);
+__device__ __forceinline__ FixScale element_scale(const int (&E)[NE], int kg) {
+    if constexpr (VF == kFluxESC) return fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], kg);
     else if constexpr (VF == kFluxKG) return fix_scale_kg(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
     else return fix_scale_dc(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
 }
@@ -340,7 +340,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         return;
     }
     if (active) {
-        const FixScale s = element_scale<VF>(sE[el_loc], ops);
+        const FixScale s = element_scale<VF>(sE[el_loc], ops.kg);
         if (node == 0) sScale[el_loc] = s;
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
@@ -357,7 +357,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     for (int id = t; id < n_el * 6 * N2; id += C::THREADS) {
         const int e = id / (6 * N2), fn = id - e * 6 * N2;
         double* f = smem + (size_t)e * C::SM + C::F + fn;
-        scale_inputs<VF>(f, reinterpret_cast<Fx*>(f), 6 * N2, element_scale<VF>(sE[e], ops));
+        scale_inputs<VF>(f, reinterpret_cast<Fx*>(f), 6 * N2, element_scale<VF>(sE[e], ops.kg));
     }
     __syncthreads();
 

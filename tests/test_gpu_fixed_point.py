@@ -7,7 +7,7 @@ import pytest
 import torch
 
 from oracle import esdc_oracle as O
-from tests.gpu_common import assert_parity, make_pair
+from tests.gpu_common import assert_parity, geometry_rounding, make_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -79,3 +79,11 @@ def test_nonphysical_state_stays_in_its_neighbourhood(p):
     assert clean
     assert torch.isnan(rb[0]).any()
     assert torch.equal(rb[clean], r[clean])
+
+
+@pytest.mark.parametrize("kind", ["far", "log", "range"])
+@pytest.mark.parametrize("flux", ["esc", "kg"])
+def test_p15_parity_across_the_rules(flux, kind):
+    """p = 15 decides the range plane by plane."""
+    solver, q, mesh, gas, qo = _case(15, kind, (2, 2, 1), flux)
+    assert_parity(solver.rhs(q), O.rhs(qo, mesh, gas, scheme=flux), qo, mesh, gas, geo_rel=geometry_rounding(15))
