@@ -512,6 +512,30 @@ ESDC_HD void euler_flux_fx(const PrimFx& a, Fx n0, Fx n1, Fx n2, const FixScale&
     f[4] = fx_mul(fx_split(f1), a.q);
 }
 
+// ln x in Q58 for 2^-44 <= x < 2^45 by table reduction (Tang's method, ACM TOMS 15, 1989): x = m 2^e, m in
+// [1, 2), T the table's approximate 1/m for the leading 7 bits of m's fraction (T = 1/(1 + (k + 1/2)/128), exact
+// in Q60), lnT = -ln T in Q60.  With r = m T - 1, |r| <= 2^-8,
+//   ln x = e ln 2 + lnT + r - r^2 (1/2 - r (1/3 - r (1/4 - r (1/5 - r (1/6 - r/7))))),
+// the first omitted term r^8/8 below 2^-67; terms from 1/4 on in 32 bits.  Error: the shift to Q58 (one unit),
+// ln 2's rounding |e|/8, the products and lnT less than two together.
+constexpr int kLnRange = 44;
+ESDC_HD int ln_exponent(double x) { return (double_hi(x) >> 20) - 1023; }
+ESDC_HD int ln_index(double x) { return (double_hi(x) >> 13) & 127; }
+ESDC_HD long long ln_fx(double x, Fx T, long long lnT) {
+    const long long m = ((double_bits(x) & 0xfffffffffffffll) | 0x10000000000000ll) << 8;      // Q60
+    const long long r = fx_mul(fx_split(m), T) - (1ll << 60);
+    const Fx rf = fx_split(r);
+    const int rs = (int)(r >> 22);                                                             // units of 2^-38
+    int a = 715827883 - (int)(mul_wide(rs, 613566757) >> 38);                                  // units of 2^-32
+    a = 858993459 - (int)(mul_wide(rs, a) >> 38);
+    a = 1073741824 - (int)(mul_wide(rs, a) >> 38);
+    const long long a3 = 384307168202282325ll - (mul_wide(rs, a) >> 10);
+    const long long C = (1ll << 59) - fx_mul(rf, fx_split(a3));
+    const long long lm = r + lnT - fx_mul(rf, fx_split(fx_mul(rf, fx_split(C))));
+    const int e = ln_exponent(x);
+    return (lm >> 2) + (mul_wide(e, 744261117) << 28) + (mul_wide(e, 1025308571) >> 2);
+}
+
 // ---- reverse of the Chandrashekar flux
 
 // Exponents and alignment shifts of an element's pair reverse.  Cotangents mu (differences of the nodes'

@@ -6,7 +6,9 @@
 #include <cstring>
 
 #include "esdc_internal.h"
+#include "fix_f64.cuh"
 #include "kernels.h"
+#include "rcp_f64.cuh"
 
 namespace esdc {
 namespace {
@@ -121,9 +123,9 @@ __device__ __forceinline__ double rcp_nr(double x) {
 //   ln x = e ln 2 - ln T_k + ln(1 + r),  ln(1 + r) = r - r^2/2 + r^3/3 - ... + r^7/7,
 // the first omitted term r^8/8 being below 2^-67.  The error is about one unit in the last place of
 // the larger of e ln 2 and ln c_k; near x = 1 from below the two nearly cancel, so the error there is
-// absolute (~1e-16), which is what the entropy sums need.  tab: shared-memory copy of the table
-// (T_k, head, tail of -ln T_k).
-__device__ __forceinline__ double ln_pos(double x, const double* __restrict__ tab, double ln2_hi, double ln2_lo) {
+// absolute (~1e-16), which is what the entropy sums need.  tab: the table (T_k, head, tail of -ln T_k).
+// Called for what ln_fx does not cover.
+__device__ __noinline__ double ln_pos(double x, const double* __restrict__ tab, double ln2_hi, double ln2_lo) {
     long long b = __double_as_longlong(x);
     int e = 0;
     if (b < 0x0010000000000000LL) {            // subnormal: scale by 2^54 first
@@ -152,7 +154,18 @@ struct Ln2 {
 // true when x is neither infinite nor NaN (exponent field not all ones), tested on the integer pipe
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
 
+// A float32 as a double, by its bits: the conversion instruction goes to the float64 pipe.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (double)x;          // zero, subnormal, infinite, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+}
+
 // Per block: sums of P J S, P J KE, P J w.dq, P J dKE.dq and the count of non-physical nodes.
+// Bound by the float64 pipe (64 clocks per instruction and scheduler): with both logarithms in fixed point, the
+// tests and conversions on bits and w.dq = (gamma - s)/(gamma - 1) dq_0 + rho/p (dKE.dq - dq_4), about 32
+// instructions a node instead of 71: 109 -> 52 us for 12^3 elements at p = 7 with a float32 dq.
 template <typename TD>
 __global__ void __launch_bounds__(kRedThreads) budgets_kernel(const double* __restrict__ q, const TD* __restrict__ dq,
                                                               const double* __restrict__ geom, int64_t K, int N,
@@ -160,16 +173,22 @@ __global__ void __launch_bounds__(kRedThreads) budgets_kernel(const double* __re
                                                               const double* __restrict__ lntab, double* __restrict__ part) {
     __shared__ double sh[kRedThreads];
     __shared__ double sw[kMaxN * kMaxN * kMaxN];     // tensor-product LGL weights w_i1 w_i2 w_i3
-    __shared__ double stab[3 * kLnTab];
+    __shared__ Fx sT[kLnTab];
+    __shared__ long long sLnT[kLnTab];
     const int N3 = N * N * N;
     const bool table = N3 <= kMaxN * kMaxN * kMaxN;   // p = 15: weights formed per node below
     if (table)
         for (int node = threadIdx.x; node < N3; node += blockDim.x)
             sw[node] = ops.w[node % N] * ops.w[(node / N) % N] * ops.w[node / (N * N)];
-    for (int i = threadIdx.x; i < 3 * kLnTab; i += blockDim.x) stab[i] = lntab[i];
+    for (int i = threadIdx.x; i < kLnTab; i += blockDim.x) {
+        sT[i] = fx_split(fx_from_double(lntab[3 * i], 0));
+        sLnT[i] = fx_from_double(lntab[3 * i + 1], 0) + fx_from_double(lntab[3 * i + 2], 0);
+    }
     __syncthreads();
     const int64_t n = K * N3;
-    double aS = 0.0, aK = 0.0, aW = 0.0, aE = 0.0, bad = 0.0;
+    const double g1 = ph.gamma * ph.inv_gm1;
+    double aS = 0.0, aK = 0.0, aW = 0.0, aE = 0.0;
+    int bad = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += stride) {
         const int64_t e = (int64_t)div_n3((unsigned long long)g);
@@ -177,37 +196,50 @@ __global__ void __launch_bounds__(kRedThreads) budgets_kernel(const double* __re
         const double wn = table ? sw[node] : ops.w[node % N] * ops.w[(node / N) % N] * ops.w[node / (N * N)];
         const double PJ = wn * geom[e * 10 * N3 + node];
         double qv[5];
+        TD d[5];
+#pragma unroll
         for (int v = 0; v < 5; ++v) qv[v] = q[(e * 5 + v) * N3 + node];
+        if (dq)
+#pragma unroll
+            for (int v = 0; v < 5; ++v) d[v] = dq[(e * 5 + v) * N3 + node];
         const double rho = qv[0];
-        const bool pos = rho > 0.0 && finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) &&
+        const bool pos = double_bits(rho) > 0 && finite_bits(qv[0]) && finite_bits(qv[1]) && finite_bits(qv[2]) &&
                          finite_bits(qv[3]) && finite_bits(qv[4]);
-        const double ri = rcp_nr(pos ? rho : 1.0);
+        const double ri = rcp_cubic(pos ? rho : 1.0);
         const double u0 = qv[1] * ri, u1 = qv[2] * ri, u2 = qv[3] * ri;
-        const double usq = u0 * u0 + u1 * u1 + u2 * u2;
-        const double p = (ph.gamma - 1.0) * (qv[4] - 0.5 * rho * usq);
-        if (!(pos && p > 0.0)) {
-            bad += 1.0;
+        const double h = 0.5 * fma(u2, u2, fma(u1, u1, u0 * u0));
+        const double p = ph.gm1 * fma(-rho, h, qv[4]);
+        if (!(pos && double_bits(p) > 0 && double_bits(p) <= 0x7ff0000000000000ll)) {
+            ++bad;
             continue;
         }
-        const double s = ln_pos(p, stab, ln2.hi, ln2.lo) - ph.gamma * ln_pos(rho, stab, ln2.hi, ln2.lo);
-        aS += PJ * (-rho * s * ph.inv_gm1);
-        aK += PJ * 0.5 * rho * usq;
+        double s;
+        if (abs(ln_exponent(p)) <= kLnRange && abs(ln_exponent(rho)) <= kLnRange) {
+            const int kp = ln_index(p), kr = ln_index(rho);
+            s = fma(-ph.gamma, fx_to_double(ln_fx(rho, sT[kr], sLnT[kr]), 2), fx_to_double(ln_fx(p, sT[kp], sLnT[kp]), 2));
+        } else {
+            s = ln_pos(p, lntab, ln2.hi, ln2.lo) - ph.gamma * ln_pos(rho, lntab, ln2.hi, ln2.lo);
+        }
+        const double Pr = PJ * rho;
+        aS = fma(Pr, s, aS);
+        aK = fma(Pr, h, aK);
         if (dq) {
-            double d[5];
+            double x[5];
             bool fin = true;
+#pragma unroll
             for (int v = 0; v < 5; ++v) {
-                d[v] = (double)dq[(e * 5 + v) * N3 + node];
-                fin = fin && finite_bits(d[v]);
+                x[v] = widen(d[v]);
+                fin = fin && finite_bits(x[v]);
             }
-            const double rp = rho * rcp_nr(p);
-            const double w1 = (ph.gamma - s) * ph.inv_gm1 - 0.5 * rp * usq;
-            aW += PJ * (w1 * d[0] + rp * (u0 * d[1] + u1 * d[2] + u2 * d[3]) - rp * d[4]);
-            aE += PJ * (-0.5 * usq * d[0] + u0 * d[1] + u1 * d[2] + u2 * d[3]);
-            if (!fin) bad += 1.0;
+            const double dE = fma(-h, x[0], fma(u2, x[3], fma(u1, x[2], u0 * x[1])));
+            aW = fma(PJ, fma(fma(-s, ph.inv_gm1, g1), x[0], rho * rcp_cubic(p) * (dE - x[4])), aW);
+            aE = fma(PJ, dE, aE);
+            if (!fin) ++bad;
         }
     }
+    aS *= -ph.inv_gm1;
     const double r0 = block_sum(aS, sh), r1 = block_sum(aK, sh), r2 = block_sum(aW, sh), r3 = block_sum(aE, sh),
-                 r4 = block_sum(bad, sh);
+                 r4 = block_sum((double)bad, sh);
     if (threadIdx.x == 0) {
         double* o = part + blockIdx.x * 5;
         o[0] = r0; o[1] = r1; o[2] = r2; o[3] = r3; o[4] = r4;

@@ -20,6 +20,12 @@ struct LM {
     long long rho() const { return fx_from_double((double)(2 * ((long double)a[0] - b[0]) / lg(a, b)), s.kr); }
     long long inv_beta() const { return fx_from_double((double)(0.5L * g1 * lg(a + 4, b + 4) / ((long double)a[4] - b[4])), s.kA); }
 };
+extern "C" double ln_of(double x) {
+    const double T = 1.0 / (1.0 + (ln_index(x) + 0.5) / 128);
+    const long double L = -std::log((long double)T);
+    const double hi = (double)L;
+    return fx_to_double(ln_fx(x, fx_split(fx_from_double(T, 0)), fx_from_double(hi, 0) + fx_from_double((double)(L - hi), 0)), 2);
+}
 extern "C" double roundtrip(double x, int k) { return fx_to_double(fx_from_double(x, k), k); }
 // prim [n][6], metric [n][3] of one element: f_EC of every pair with the summed metric, as float64; 1 if out of range
 extern "C" int fluxes(int n, const double* P, const double* M, double gamma, double* out) {
@@ -123,6 +129,8 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(str(so))
     L.roundtrip.restype = ctypes.c_double
     L.roundtrip.argtypes = [ctypes.c_double, ctypes.c_int]
+    L.ln_of.restype = ctypes.c_double
+    L.ln_of.argtypes = [ctypes.c_double]
     L.reverses.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 3 + [ctypes.c_double, ctypes.c_void_p]
     L.fluxes.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_double, ctypes.c_void_p]
     return L
@@ -245,3 +253,15 @@ def test_out_of_range_is_refused(lib):
         Q = P.copy()
         Q[3, col] = val
         assert lib.fluxes(8, Q.ctypes.data, M.ctypes.data, 1.4, out.ctypes.data) == 1
+
+
+@pytest.mark.parametrize("lo,hi", [(-1e-9, 1e-9), (-0.01, 0.01), (-3.0, 3.0), (-30.0, 30.0)])
+def test_logarithm(lib, lo, hi):
+    """ln_fx over its range against extended precision: |e|/8 + 3 units of 2^-58 (its own bound) and the
+    rounding of the returned double."""
+    x = np.exp(np.random.default_rng(4).uniform(lo, hi, 20000))
+    x = np.concatenate([x, 2.0 ** np.arange(-44, 45), np.nextafter(2.0 ** np.arange(-43, 46), 0), 1.0 + np.arange(128) / 128.0])
+    y = np.array([lib.ln_of(float(v)) for v in x])
+    ref = np.log(x.astype(np.longdouble))
+    bound = (np.abs(np.frexp(x)[1] - 1) / 8.0 + 3.0) * 2.0 ** -58 + np.abs(ref) * 2.0 ** -53
+    assert (np.abs(y - ref) <= bound).all(), float((np.abs(y - ref) / bound).max())
