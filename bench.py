@@ -595,7 +595,7 @@ def run_ours(args):
         if dist is not None:
             dist.destroy_process_group()
         return
-    src = _src("rhs_f64.cu")
+    src = _src("rhs_fix.cuh")
     fl = element_kernel_flops_per_node(p) * n
     achieved = fl / (kernel_ms * 1e-3) / 1e12
     peak = peak_f64 / 1e12
@@ -608,10 +608,11 @@ def run_ours(args):
         "n_gpus": ws, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
         "data": "synthetic", "config": _config(args),
-        "roofline": {"bound": "alu", "kernel": "rhs_main_f64<8>", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "alu", "kernel": "rhs_fix_f64<8>", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak,
-                     "traffic": _ncu_traffic("rhs_main_f64_tgv_p7.md", src, n),
-                     "peak_source": "of measured: float64 FMA throughput (esdc_probe_fma) in this run",
+                     "traffic": _ncu_traffic("rhs_fix_f64_tgv_p7.md", src, n),
+                     "peak_source": "of measured: float64 FMA throughput (esdc_probe_fma) in this run; the kernel does "
+                                    "most of its work in fixed point on the integer pipes, so the fraction exceeds 1",
                      "peak_nominal": FP64_NOMINAL_TFLOPS, "frac_nominal": achieved / FP64_NOMINAL_TFLOPS,
                      "flops_per_launch": fl, "kernel_ms": kernel_ms,
                      "hbm_frac": element_kernel_bytes_per_node(p) * n / (kernel_ms * 1e-3) / (hbm * 1e9),

@@ -483,15 +483,16 @@ int ensure_adjoint(esdc_ctx* c) {
         return fail(ESDC_ERR_UNSUPPORTED, "the adjoint is built for float64 contexts with p <= 7");
     if (c->setup.bounded != 0 && !c->d_qext)
         return fail(ESDC_ERR_ARG, "a bounded box needs an exterior state (esdc_set_exterior)");
-    if (c->d_adj_g) return ESDC_OK;
+    if (c->d_adj_acc) return ESDC_OK;              // the last of them: all are there
     const size_t N2 = (size_t)c->N * c->N;
-    CUDA_TRY(cudaMalloc(&c->d_adj_g, (size_t)c->K * 6 * 5 * N2 * sizeof(double)));
-    CUDA_TRY(cudaMalloc(&c->d_adj_t, (size_t)c->K * 6 * 4 * N2 * sizeof(double)));
-    if (c->setup.volume_flux == ESDC_FLUX_ESC)
-        CUDA_TRY(cudaMalloc(&c->d_adj_pb, (size_t)c->K * 5 * c->N3 * sizeof(double)));
-    CUDA_TRY(cudaMalloc(&c->d_adj_mu, esdc::adjoint_mu_blocks(c) * sizeof(double)));
-    CUDA_TRY(cudaMalloc(&c->d_adj_acc, 8 * sizeof(double)));
+    // a call after a failed one takes up where that stopped
+    auto need = [](double*& p, size_t n) { return p ? cudaSuccess : cudaMalloc(&p, n * sizeof(double)); };
     CUDA_TRY(esdc::prepare_adjoint(c));
+    CUDA_TRY(need(c->d_adj_g, (size_t)c->K * 6 * 5 * N2));
+    CUDA_TRY(need(c->d_adj_t, (size_t)c->K * 6 * 4 * N2));
+    if (c->setup.volume_flux == ESDC_FLUX_ESC) CUDA_TRY(need(c->d_adj_pb, (size_t)c->K * 5 * c->N3));
+    CUDA_TRY(need(c->d_adj_mu, esdc::adjoint_mu_blocks(c)));
+    CUDA_TRY(need(c->d_adj_acc, 8));
     return ESDC_OK;
 }
 

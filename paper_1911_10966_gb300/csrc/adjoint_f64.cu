@@ -1,5 +1,5 @@
 // Vector-Jacobian product of the float64 residual: grad = (dR/dq)^T lambda and
-// grad_mu = lambda . dR/dmu, for R = dq/dt of rhs_f64.cu (same discretization, same readings).
+// grad_mu = lambda . dR/dmu, for R = dq/dt of rhs_fix.cuh (same discretization, same readings).
 //
 // The forward residual is a sum of terms, each local to one element except the face couplings:
 //   volume   r_i -= 2 S_ij f(q_i,q_j)/w_i, r_j += 2 S_ij f(q_i,q_j)/w_j     (pairs on xi_l lines)

@@ -1,9 +1,8 @@
 // Float64 residual of the elements of one CTA: flux differencing, interface SAT, BR1 gradients, viscous
-// fluxes and their divergence, every operation in float64.  rhs_f64.cu runs it for the volume fluxes
-// without a fixed-point form; rhs_fix_f64.cu for elements outside the fixed-point range.
+// fluxes and their divergence, every operation in float64.  rhs_fix.cuh runs it for elements outside the fixed-point range.
 //
-// One element per group of N^3 threads (EPB elements per CTA, which has at least EPB N^3 threads).  The element's state is loaded once,
-// converted to primitive and entropy variables in shared memory, and then:
+// One element per group of N^3 threads (EPB elements per CTA, which has at least EPB N^3 threads).  The
+// element's state is loaded once, converted to primitive and entropy variables in shared memory, and then:
 //   1. volume: one thread per xi_l line of each direction evaluates the N(N-1)/2 distinct node pairs of
 //      its line once each, using the skew part S of Q = S + E/2: r_i -= 2 S_ij f_ij / w_i,
 //      r_j += 2 S_ij f_ij / w_j.  The E/2 boundary part of the volume term, -E_ii f(q_i).n_J / w_i,
@@ -28,12 +27,9 @@ template <int N>
 struct Cfg {
     static constexpr int N2 = N * N, N3 = N * N * N;
     static constexpr int EPB = N3 >= 96 ? 1 : (N3 >= 48 ? 2 : (N3 >= 24 ? 4 : 16));
-    static constexpr int THREADS = (EPB * N3 + 31) / 32 * 32;
     // shared doubles per element: prim/w/Ftilde 12 x N3 | r 3 x 5 x N3 (one per line direction) |
     // geometry 10 x N3 | face w 24 x N2
     static constexpr int SM = 37 * N3 + 24 * N2;
-    // resident CTAs per SM the register allocation is sized for (the float64 pipe needs few warps)
-    static constexpr int MINB = N >= 7 ? 1 : (N == 6 ? 2 : (N >= 4 ? 3 : 4));
 };
 
 // XF: the kernel also handles the matrix dissipation, the interior penalty, boundary faces with an

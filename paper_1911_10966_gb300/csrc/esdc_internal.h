@@ -10,7 +10,7 @@
 
 namespace esdc {
 
-constexpr int kMaxN = 8;     // p <= 7: one element per CTA (rhs_f64.cu, rhs_f32.cu, the adjoint)
+constexpr int kMaxN = 8;     // p <= 7: one element per CTA (rhs_fix.cuh, rhs_f32.cu, the adjoint)
 constexpr int kLargeN = 16;  // p = 15: the multi-pass float64 residual (rhs_large_f64.cu)
 
 // The two limbs of a fixed-point number (h 2^30 + l) 2^-60.

@@ -1,4 +1,4 @@
-// Float64 device functions shared by the residual kernels (rhs_f64.cu for p <= 7, rhs_large_f64.cu
+// Float64 device functions shared by the residual kernels (rhs_fix.cuh for p <= 7, rhs_large_f64.cu
 // for p = 15): primitive variables, reciprocals, the Chandrashekar, Kennedy-Gruber and Euler fluxes
 // contracted with a direction (Sec. 4), the face jump/average quantities and the matrix dissipation,
 // and the line indexing of an element's tensor-product nodes.

@@ -1,4 +1,4 @@
-// FP32 residual kernels of the mixed-precision form: the same ES-C residual as rhs_f64.cu with all
+// FP32 residual kernels of the mixed-precision form: the same ES-C residual as rhs_fix.cuh with all
 // flux differencing, interface and viscous arithmetic in float32, evaluated on a perturbation
 // state so that float32 rounding acts on O(1) quantities rather than on the O(1/(gamma Ma^2))
 // pressure and enthalpy.
