@@ -87,3 +87,23 @@ def test_p15_parity_across_the_rules(flux, kind):
     """p = 15 decides the range plane by plane."""
     solver, q, mesh, gas, qo = _case(15, kind, (2, 2, 1), flux)
     assert_parity(solver.rhs(q), O.rhs(qo, mesh, gas, scheme=flux), qo, mesh, gas, geo_rel=geometry_rounding(15))
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -60, 2.0 ** -43, 1.0, 2.0 ** 44, 2.0 ** 60])
+def test_budget_logarithms(scale):
+    """Entropy budgets with densities and pressures inside and beyond the exponents of the fixed-point
+    logarithm.  Bound: 1e-13 of the terms' magnitudes, as in the other budget tests (the two sides build J
+    independently), those of s = ln p - gamma ln rho taken before they cancel."""
+    solver, q, mesh, gas, qo = make_pair(3, (3, 2, 2), warp=0.1, seed=3, Re=100.0)
+    x = qo * scale
+    d = torch.tensor(np.random.default_rng(1).uniform(-1, 1, tuple(x.shape))) * scale
+    b, bo = solver.budgets(solver.to_device(x.numpy()), solver.to_device(d.numpy())), O.budgets(x, d, mesh, gas)
+    PJ, g = O.quadrature_weights(mesh), gas.gamma
+    rho, p = x[:, 0], (g - 1) * (x[:, 4] - 0.5 * (x[:, 1:4] ** 2).sum(1) / x[:, 0])
+    logs = (p.log().abs() + g * rho.log().abs() + g) / (g - 1)
+    wd = logs * d[:, 0].abs() + rho / p * ((x[:, 1:4] * d[:, 1:4]).abs().sum(1) / rho + d[:, 4].abs()
+                                          + 0.5 * (x[:, 1:4] ** 2).sum(1) / rho ** 2 * d[:, 0].abs())
+    eps = 1e-13
+    assert abs(b[0] - bo[0]) <= eps * float((PJ * rho * logs).sum())
+    assert abs(b[1] - bo[1]) <= eps * abs(bo[1])
+    assert abs(b[2] - bo[2]) <= eps * float((PJ * wd).sum())
