@@ -234,10 +234,11 @@ ESDC_HD int fx_clamp(int a) { return a > 62 ? 62 : a; }
 
 // Er, Eu, Eb, En: largest biased exponents of the half density, half velocity, beta and metric terms;
 // Er0, Eb0: smallest of half density and beta.  kg: exponent of inv_gm1 = c 2^kg, 1/2 <= c < 1.
-// Bounds in Q60: densities and betas < 1/2, velocities and metrics < 1/4 (so that the twelve limb
-// products of a three-term dot product stay inside 64 bits), |u|^2/4 < 3/8, ubar.n < 3/4 and kept doubled,
-// mass flux < 3/2, p_t <= 1, momentum flux < 5/4 (7/8 if the pressure part sets its exponent), energy
-// coefficient < 1.01, energy flux < 2.2.  All but p_t and the coefficient carry a factor S_ij (or 1 on a
+// Bounds in Q60: densities and betas < 1/2, velocities and metrics < 1/4 (the limb products of
+// ubar.n then sum to at most 3 (2 1/2 + 1/2) = 4.5 2^60, a sum of two having a low limb of up to 2^31),
+// |u|^2/4 < 3/8, ubar.n < 3/4 and kept doubled, mass flux < 3/2, p_t <= 1, momentum flux < 5/4 (7/8 if
+// the pressure part sets its exponent; three products with it would reach 3 (2 5/4 + 1/2) = 9 2^60, so
+// the energy flux sums them in two parts), energy coefficient < 1.01, energy flux < 2.2.  All but p_t and the coefficient carry a factor S_ij (or 1 on a
 // face), |S_ij| with row sums below 3.41, so their sums over a line stay inside 63 bits.
 // Ey, Ez: largest exponents of mu RT/J and kappa/R RT^2/J.
 ESDC_HD FixScale fix_scale(int Er, int Er0, int Eu, int Eb, int Eb0, int En, int Ey, int Ez, int kg) {
@@ -483,7 +484,8 @@ ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, F
     f[3] = fx_mul2<3>(fa, v2, pa, n2);
     const Fx c5 = fx_split((A >> s.sc) - (fx_join(fx_add(a.q, b.q)) >> s.sq));
     const Fx m0 = fx_split(f[1]), m1 = fx_split(f[2]), m2 = fx_split(f[3]);
-    f[4] = ((fx_mul(fx_split(f1), c5) + s.hC) >> s.sC) + ((fx_dot<6>(v0, m0, v1, m1, v2, m2) + s.hD) >> s.sD);
+    const long long vm = fx_mul2<4>(v0, m0, v1, m1) + fx_mul<2>(v2, m2);
+    f[4] = ((fx_mul(fx_split(f1), c5) + s.hC) >> s.sC) + ((vm + s.hD) >> s.sD);
 }
 
 // The Kennedy-Gruber flux of flux_f64.cuh (kg_flux), units as above
