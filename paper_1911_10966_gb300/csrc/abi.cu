@@ -523,6 +523,7 @@ void free_ctx(esdc_ctx* c) {
     cudaFree(c->d_jinv);
     cudaFree(c->d_xyz);
     cudaFree(c->d_fnorm);
+    cudaFree(c->d_kn);
     cudaFree(c->d_nsurf);
     cudaFree(c->d_lr);
     cudaFree(c->d_lft);
@@ -852,6 +853,10 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
     }
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_nbr, hs.nbr.data(), hs.nbr.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_kn, hs.kn.size() * sizeof(int32_t));
+    if (e == cudaSuccess)
+        e = cudaMemcpy(c->d_kn, hs.kn.data(), hs.kn.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    c->float64_form = esdc::float64_form(c, hs.kn.data());
     if (e == cudaSuccess) {
         const size_t xyz_bytes = (size_t)c->K * 3 * c->N3 * sizeof(double);
         e = cudaMalloc(&c->d_xyz, xyz_bytes);

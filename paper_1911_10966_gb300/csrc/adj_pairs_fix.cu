@@ -111,7 +111,7 @@ template <int N>
 __global__ void __launch_bounds__(AdjCfg<N>::THREADS, AdjCfg<N>::MINB)
 adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, const double* __restrict__ geom,
               const double* __restrict__ jinv, double* __restrict__ pbar, int64_t K, const __grid_constant__ Ops ops,
-              const __grid_constant__ Phys ph) {
+              const __grid_constant__ Phys ph, const int32_t* __restrict__ kn) {
     using C = AdjCfg<N>;
     constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NE = 11;
     extern __shared__ double smem[];
@@ -127,7 +127,8 @@ adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, cons
     double* sm = smem + (size_t)el_loc * C::SM;
     Fx* X = reinterpret_cast<Fx*>(sm);
     const int own = slot<N>(node % N, (node / N) % N, node / N2);
-    for (int i = t; i < EPB * NE; i += C::THREADS) sE[i / NE][i % NE] = 0;
+    for (int i = t; i < EPB * NE; i += C::THREADS)
+        sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? metric_exponent(kn[(int64_t)blockIdx.x * EPB + i / NE], kAdjStretch) : 0;
     for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
     for (int i = t; i < N; i += C::THREADS) sW[i] = ops.WB[i];
     __syncthreads();
@@ -139,11 +140,7 @@ adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, cons
         int E[NE];
         E[5] = 0;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) {
-            const double g = geom[(el * 10 + 1 + c) * N3 + node];
-            sm[C::XN + c * SL + own] = g;
-            E[5] = max(E[5], biased_exp(g));
-        }
+        for (int c = 0; c < 9; ++c) sm[C::XN + c * SL + own] = geom[(el * 10 + 1 + c) * N3 + node];
         double lt[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
@@ -295,7 +292,7 @@ template <int N>
 cudaError_t launch_n_adj(const esdc_ctx* c, const double* q, const double* lam, cudaStream_t s) {
     using C = AdjCfg<N>;
     adj_pairs_fix<N><<<(unsigned)((c->K + C::EPB - 1) / C::EPB), C::THREADS, C::EPB * C::SM * sizeof(double), s>>>(
-        q, lam, c->d_geom, c->d_jinv, c->d_adj_pb, c->K, c->ops, c->phys);
+        q, lam, c->d_geom, c->d_jinv, c->d_adj_pb, c->K, c->ops, c->phys, c->d_kn);
     return cudaGetLastError();
 }
 

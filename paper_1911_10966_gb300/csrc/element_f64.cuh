@@ -30,6 +30,9 @@ struct Cfg {
     // shared doubles per element: prim/w/Ftilde 12 x N3 | r 3 x 5 x N3 (one per line direction) |
     // geometry 10 x N3 | face w 24 x N2
     static constexpr int SM = 37 * N3 + 24 * N2;
+    // the float64 kernel's threads, and resident CTAs per SM its registers are sized for (its pipe needs few warps)
+    static constexpr int THREADS = EPB * N3;
+    static constexpr int MINB = N >= 7 ? 1 : (N == 6 ? 2 : (N >= 4 ? 3 : 4));
 };
 
 // XF: the kernel also handles the matrix dissipation, the interior penalty, boundary faces with an

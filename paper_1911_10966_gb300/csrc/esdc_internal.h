@@ -94,8 +94,23 @@ struct HostSetup {
     std::vector<double> geom;            // [K][10][N^3]: J, Ja_lm (l-major)
     std::vector<double> nsurf;           // [K][6][3][N^2] surface metrics (optimized metrics only)
     std::vector<int32_t> nbr;            // [K][6]
+    std::vector<int32_t> kn;             // [K] exponent of the largest metric entry and stretch (metric_code)
     double h_min = 0.0;
 };
+
+// Stretch of an element: the ratio between the largest metric entries of the three coordinates, max over
+// directions and nodes of |Ja_lm|, m = 1..3; beyond kRhsStretch an element's residual, beyond kAdjStretch its
+// adjoint is evaluated in float64.  One exponent serves all nine entries of an element, so the fluxes' errors are
+// relative to the largest, where float64's follow each coordinate's own.
+// Errors against extended precision, fixed point over float64, axis-aligned elements, worst variable and flow of
+// p = 3, 4 and 7: 1.0 to 1.1 at ratio 2, 1.7 at 4, 3.5 at 8, 200 at 1000, more in the viscous terms.
+// The reverse pairs keep exponents of their own: 0.1 at ratio 1, 0.2 at 4, 0.7 to 1.1 at 16, 15 at 1000 (p = 3).
+constexpr int kRhsStretch = 1, kAdjStretch = 3;
+// An element's code: the biased exponent E of its largest metric entry, and the smallest s >= 0 with that ratio at
+// most 1.025 2^s (a little slack for 2 : 1 boxes).
+constexpr int metric_code(int E, int s) { return E + (s << 12); }
+// the exponent again, or one out of range (fix_range_ok) where the stretch is above `most`
+constexpr int metric_exponent(int code, int most) { return (code >> 12) > most ? 2047 : code & 4095; }
 
 int lgl(int p, double* xi, double* w);
 int build_operators(int p, HostSetup& hs);
@@ -139,6 +154,8 @@ struct esdc_ctx {
     float* d_geomf = nullptr;        // [K][10][N3] float32 copy (mixed precision)
     float* d_nsurff = nullptr;       // [K][6][3][N2] float32 copy of the surface metrics (mixed precision)
     int32_t* d_nbr = nullptr;        // [K][6]
+    int32_t* d_kn = nullptr;         // [K] HostSetup::kn
+    bool float64_form = false;       // the fixed-point kernels would pass on nearly every CTA
     void* d_trace = nullptr;         // [K][6][4][N2] viscous normal-flux traces (f64 or f32)
     float* d_shadow = nullptr;       // [K][5][N3] float32 perturbation state (mixed precision)
     double* d_red = nullptr;         // reduction partials

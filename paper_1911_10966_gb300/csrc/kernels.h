@@ -20,6 +20,8 @@ struct DivU64 {
 cudaError_t prepare_rhs_f64(const esdc_ctx* c);
 // ev: NULL, or four events recorded around the element kernel and the face kernel
 cudaError_t launch_rhs_f64(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s, cudaEvent_t* ev);
+// whether so many elements are stretched (kn) that the float64 kernels alone are faster
+bool float64_form(const esdc_ctx* c, const int32_t* kn);
 // the element kernel in block fixed point (rhs_fix.cuh) by volume flux; _xf: with the optional interface terms
 #define ESDC_FIX_DECL(name)                          \
     cudaError_t prepare_fix_##name(const esdc_ctx* c); \

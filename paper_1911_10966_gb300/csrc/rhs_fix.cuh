@@ -244,7 +244,8 @@ __global__ void __launch_bounds__(FixCfg<N, VF, WIDE>::THREADS, FixCfg<N, VF, WI
 rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
             const double* __restrict__ jinv, const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K,
             const __grid_constant__ Ops ops, const __grid_constant__ Phys ph, const double* __restrict__ qext,
-            const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
+            const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm,
+            const int32_t* __restrict__ kn) {
     using C = FixCfg<N, VF, WIDE>;
     constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxESC ? 8 : 10;
     extern __shared__ double smem[];
@@ -264,7 +265,8 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     Fx* X = reinterpret_cast<Fx*>(sm);
     const int own_slot = slot<N>(i1, i2, i3);
     const int64_t eoff = el * 5 * N3;
-    for (int i = t; i < EPB * NE; i += C::THREADS) sE[i / NE][i % NE] = 0;
+    for (int i = t; i < EPB * NE; i += C::THREADS)
+        sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? metric_exponent(kn[(int64_t)blockIdx.x * EPB + i / NE], kRhsStretch) : 0;
     if (t < EPB) sMag[t][0] = sMag[t][1] = 0;
     for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
     for (int i = t; i < N; i += C::THREADS) sW[i] = ops.winv[i];
@@ -280,11 +282,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         int E[NE];
         E[5] = 0;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) {
-            const double g = geom[(el * 10 + 1 + c) * N3 + node];
-            sm[C::XN + c * SL + own_slot] = g;
-            E[5] = max(E[5], biased_exp(g));
-        }
+        for (int c = 0; c < 9; ++c) sm[C::XN + c * SL + own_slot] = geom[(el * 10 + 1 + c) * N3 + node];
         pair_inputs<VF>(qv, ph, pi, RT);
 #pragma unroll
         for (int i = 0; i < NP; ++i) sm[C::XP + i * SL + own_slot] = pi[i];
@@ -312,10 +310,6 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         // a boundary face (neighbour -1, bounded boxes only) sees the exterior state at its own nodes
         if constexpr (XF) {
             if (nb < 0) qn = qext + ee * 5 * N3 + base + (side ? (N - 1) * st : 0);
-            if (nsurf) {
-                const double* ns = nsurf + (ee * 6 + 2 * l + side) * 3 * N2 + fi;
-                E[5] = max(biased_exp(ns[0]), max(biased_exp(ns[N2]), biased_exp(ns[2 * N2])));
-            }
         }
         double qv[5], RT, pi[NP];
 #pragma unroll
@@ -705,7 +699,28 @@ cudaError_t launch_w(const esdc_ctx* c, const double* q, double* dqdt, cudaStrea
     const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
     rhs_fix_f64<N, VF, XF, WIDE><<<grid, C::THREADS, fix_smem<N, VF, WIDE>(), s>>>(
         q, dqdt, c->d_geom, c->d_jinv, c->d_nbr, (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext, c->d_src,
-        c->d_nsurf, c->d_fnorm);
+        c->d_nsurf, c->d_fnorm, c->d_kn);
+    return cudaGetLastError();
+}
+
+// the float64 form as a kernel of its own, for meshes of stretched elements
+template <int N, int VF, bool XF>
+__global__ void __launch_bounds__(Cfg<N>::THREADS, Cfg<N>::MINB)
+rhs_f64(const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
+        const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K, const __grid_constant__ Ops ops,
+        const __grid_constant__ Phys ph, const double* __restrict__ qext, const double* __restrict__ src,
+        const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
+    extern __shared__ double smem[];
+    element_f64<N, VF, XF>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+}
+
+template <int N, int VF, bool XF>
+cudaError_t launch_f64(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    using C = Cfg<N>;
+    const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
+    rhs_f64<N, VF, XF><<<grid, C::THREADS, C::EPB * C::SM * sizeof(double), s>>>(
+        q, dqdt, c->d_geom, c->d_nbr, (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext, c->d_src, c->d_nsurf,
+        c->d_fnorm);
     return cudaGetLastError();
 }
 
@@ -717,14 +732,16 @@ constexpr int wide_upto(int n) { return n == 2 ? 6 : (n == 3 ? 4 : (n == 4 ? 2 :
 
 template <int N, int VF, bool XF>
 cudaError_t launch_n(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
+    if (c->float64_form) return launch_f64<N, VF, XF>(c, q, dqdt, s);
     if constexpr (wide_upto(N) > 0)
         if (c->K <= (int64_t)wide_upto(N) * sm_count()) return launch_w<N, VF, XF, true>(c, q, dqdt, s);
     return launch_w<N, VF, XF, false>(c, q, dqdt, s);
 }
 
 template <int N, int VF, bool XF>
-cudaError_t prepare_n() {
+cudaError_t prepare_n(const esdc_ctx* c) {
     constexpr cudaFuncAttribute kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (c->float64_form) return cudaFuncSetAttribute(rhs_f64<N, VF, XF>, kAttr, (int)(Cfg<N>::EPB * Cfg<N>::SM * sizeof(double)));
     const cudaError_t e = cudaFuncSetAttribute(rhs_fix_f64<N, VF, XF, false>, kAttr, (int)fix_smem<N, VF, false>());
     if constexpr (wide_upto(N) > 0)
         if (e == cudaSuccess) return cudaFuncSetAttribute(rhs_fix_f64<N, VF, XF, true>, kAttr, (int)fix_smem<N, VF, true>());
@@ -734,13 +751,13 @@ cudaError_t prepare_n() {
 template <int VF, bool XF>
 cudaError_t prepare_vf(const esdc_ctx* c) {
     switch (c->N) {
-        case 2: return prepare_n<2, VF, XF>();
-        case 3: return prepare_n<3, VF, XF>();
-        case 4: return prepare_n<4, VF, XF>();
-        case 5: return prepare_n<5, VF, XF>();
-        case 6: return prepare_n<6, VF, XF>();
-        case 7: return prepare_n<7, VF, XF>();
-        case 8: return prepare_n<8, VF, XF>();
+        case 2: return prepare_n<2, VF, XF>(c);
+        case 3: return prepare_n<3, VF, XF>(c);
+        case 4: return prepare_n<4, VF, XF>(c);
+        case 5: return prepare_n<5, VF, XF>(c);
+        case 6: return prepare_n<6, VF, XF>(c);
+        case 7: return prepare_n<7, VF, XF>(c);
+        case 8: return prepare_n<8, VF, XF>(c);
         default: return cudaErrorInvalidValue;
     }
 }

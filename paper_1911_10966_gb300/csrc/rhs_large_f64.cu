@@ -310,7 +310,7 @@ template <int VF>
 __global__ void __launch_bounds__(LTHREADS, 6)
 lg_volume_fix(const double* __restrict__ q, const double* __restrict__ geom, const int32_t* __restrict__ nbr,
               const double* __restrict__ fnorm, double* __restrict__ rl, double* __restrict__ th, int64_t K,
-              const __grid_constant__ OpsL ops, const __grid_constant__ Phys ph) {
+              const __grid_constant__ OpsL ops, const __grid_constant__ Phys ph, const int32_t* __restrict__ kn) {
     constexpr int NP = fix_inputs<VF>(), NE = VF == kFluxESC ? 8 : 10, NF = 2 * LN;
     extern __shared__ double sm[];
     __shared__ int sE[NE], sNext;
@@ -378,7 +378,7 @@ lg_volume_fix(const double* __restrict__ q, const double* __restrict__ geom, con
     }
     block_max<true>(sE, 0, E, lane);
     __syncthreads();
-    if (!fix_range_ok(sE[0], 4096 - sE[1], sE[2], sE[3], 4096 - sE[4], sE[5])) {
+    if (metric_exponent(kn[el], kRhsStretch) == 2047 || !fix_range_ok(sE[0], 4096 - sE[1], sE[2], sE[3], 4096 - sE[4], sE[5])) {
         __syncthreads();
         plane_out_of_range<VF>(sm, q, geom, nbr, fnorm, rl, th, K, ops, ph);
         return;
@@ -689,12 +689,14 @@ lg_finish(const double* __restrict__ rl, const double* __restrict__ jinv, double
 template <int VF>
 cudaError_t launch_volume(const esdc_ctx* c, const double* q, cudaStream_t s) {
     const unsigned grid = (unsigned)(c->K * 3 * LN);
-    if constexpr (VF == kFluxDC)
+    if (VF == kFluxDC || c->float64_form) {
         lg_volume<VF><<<grid, LTHREADS, plane_smem_doubles<VF>() * sizeof(double), s>>>(
             q, c->d_geom, c->d_nbr, c->d_fnorm, c->d_lr, c->d_lft, c->K, c->opsl, c->phys);
-    else
+        return cudaGetLastError();
+    }
+    if constexpr (VF != kFluxDC)
         lg_volume_fix<VF><<<grid, LTHREADS, fix_smem_doubles<VF>() * sizeof(double), s>>>(
-            q, c->d_geom, c->d_nbr, c->d_fnorm, c->d_lr, c->d_lft, c->K, c->opsl, c->phys);
+            q, c->d_geom, c->d_nbr, c->d_fnorm, c->d_lr, c->d_lft, c->K, c->opsl, c->phys, c->d_kn);
     return cudaGetLastError();
 }
 

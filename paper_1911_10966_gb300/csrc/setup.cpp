@@ -417,6 +417,23 @@ double element_min_edge(int N, const double* xyz) {
 
 }  // namespace
 
+// HostSetup::kn of one element: g its metric rows [9][N3], ns its surface metrics [6][3][N2] or null
+static int32_t element_metric_code(int N, const double* g, const double* ns) {
+    const int N2 = N * N, N3 = N2 * N;
+    double c[3] = {0.0, 0.0, 0.0};
+    for (int m = 0; m < 3; ++m) {
+        for (int l = 0; l < 3; ++l)
+            for (int i = 0; i < N3; ++i) c[m] = std::max(c[m], std::fabs(g[(3 * l + m) * N3 + i]));
+        for (int f = 0; ns && f < 6; ++f)
+            for (int i = 0; i < N2; ++i) c[m] = std::max(c[m], std::fabs(ns[(3 * f + m) * N2 + i]));
+    }
+    const double hi = std::max(c[0], std::max(c[1], c[2])), lo = std::min(c[0], std::min(c[1], c[2]));
+    int e, s = 0;
+    std::frexp(hi, &e);
+    for (double r = 1.025 * lo; s < 1000 && !(hi <= r); r *= 2.0) ++s;
+    return metric_code(std::max(e + 1022, 0), s);
+}
+
 int build_geometry(const esdc_setup_t& s, const double* xyz, HostSetup& hs, std::string& err) {
     const int N = hs.N, N3 = N * N * N, N2 = N * N;
     const int64_t K = (int64_t)s.kx * s.ky * s.kz;
@@ -429,6 +446,7 @@ int build_geometry(const esdc_setup_t& s, const double* xyz, HostSetup& hs, std:
     } else {
         hs.nsurf.clear();
     }
+    hs.kn.assign((size_t)K, 0);
     unsigned nt = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
     if (K < 64) nt = 1;
     std::vector<int> bad(nt, 0);
@@ -442,6 +460,7 @@ int build_geometry(const esdc_setup_t& s, const double* xyz, HostSetup& hs, std:
                                                                    &hs.nsurf[(size_t)e * 6 * 3 * N2])
                                       : element_geometry(hs.D, N, x, &hs.geom[(size_t)e * 10 * N3]);
                 if (!good) bad[t] = 1;
+                hs.kn[e] = element_metric_code(N, &hs.geom[((size_t)e * 10 + 1) * N3], opt ? &hs.nsurf[(size_t)e * 18 * N2] : nullptr);
                 hmin[t] = std::min(hmin[t], element_min_edge(N, x));
             }
         });
