@@ -55,54 +55,50 @@ struct AdjMeansF64 {
     }
 };
 
-// The pair loop in float64 for a CTA with an element out of range: inputs still float64 in shared memory.
+// The pair loop in float64 for a CTA with an element out of range: inputs still float64 in shared memory.  One
+// thread per line, the lines numbered consecutively over the threads: a float64 instruction costs its pipe 64
+// clocks whatever its active lanes, and the half-filled last round of the cyclic distances would be a seventh
+// (N = 8) to a third (N = 4) more of them.
 template <int N>
 __device__ __noinline__ void pairs_f64(double* smem, int n_el, const Ops& ops, const Phys& ph) {
     using C = AdjCfg<N>;
     constexpr int N2 = C::N2, SL = C::SL;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int lw = lane / N, i = lane - lw * N;
 #pragma unroll 1
-    for (int task = warp; task < 3 * C::TPD; task += C::WARPS) {
-        const int l = task / C::TPD;
-        int line = (task - l * C::TPD) * C::LPW + lw;
-        const bool go = lw < C::LPW && line < n_el * N2;
-        line = go ? line : 0;
-        const int e = line / N2, li = line - e * N2;
+    for (int g = threadIdx.x; g < n_el * 3 * N2; g += C::THREADS) {
+        const int e = g / (3 * N2), r = g - e * 3 * N2;
+        const int l = r / N2, li = r - l * N2;
+        const int c1 = li % N, c2 = li / N;
         double* se = smem + (size_t)e * C::SM;
         const double *X = se + C::XP, *n = se + C::XN + 3 * l * SL, *lt = se + C::LT;
-        const int ii = line_slot<N>(l, i < N ? i : 0, li % N, li / N);
-        const PrimH a = {2.0 * X[ii], X[SL + ii], X[2 * SL + ii], X[3 * SL + ii], X[4 * SL + ii], X[5 * SL + ii]};
-        PRaw acc{0, 0, 0, 0, 0, 0};
+        double* B = se + C::B + 6 * l * SL;
+        auto prim = [&](int k) { return PrimH{2.0 * X[k], X[SL + k], X[2 * SL + k], X[3 * SL + k], X[4 * SL + k], X[5 * SL + k]}; };
+        auto sums = [&](int k) { return PRaw{B[k], B[SL + k], B[2 * SL + k], B[3 * SL + k], B[4 * SL + k], B[5 * SL + k]}; };
+        auto store = [&](int k, const PRaw& p) {
+            B[k] = p.rho;
+            B[SL + k] = p.u0;
+            B[2 * SL + k] = p.u1;
+            B[3 * SL + k] = p.u2;
+            B[4 * SL + k] = p.beta;
+            B[5 * SL + k] = p.c;
+        };
+        for (int i = 0; i < N; ++i) store(line_slot<N>(l, i, c1, c2), PRaw{0, 0, 0, 0, 0, 0});
 #pragma unroll 1
-        for (int k = 1; k <= N / 2; ++k) {
-            const int j = i + k < N ? i + k : i + k - N;
-            PRaw o{0, 0, 0, 0, 0, 0};
-            if (go && (2 * k < N || i < k)) {
-                const int jj = line_slot<N>(l, j, li % N, li / N);
-                const PrimH b = {2.0 * X[jj], X[SL + jj], X[2 * SL + jj], X[3 * SL + jj], X[4 * SL + jj], X[5 * SL + jj]};
+        for (int i = 0; i < N - 1; ++i) {
+            const int ii = line_slot<N>(l, i, c1, c2);
+            const PrimH a = prim(ii);
+            PRaw acc = sums(ii);
+#pragma unroll 1
+            for (int j = i + 1; j < N; ++j) {
+                const int jj = line_slot<N>(l, j, c1, c2);
+                PRaw o = sums(jj);
                 double mu[5];
 #pragma unroll
                 for (int v = 0; v < 5; ++v)
                     mu[v] = ops.S[i][j] * (lt[v * SL + jj] * ops.winv[j] - lt[v * SL + ii] * ops.winv[i]);
-                ec_pair_vjp(a, b, n[ii] + n[jj], n[SL + ii] + n[SL + jj], n[2 * SL + ii] + n[2 * SL + jj], mu, ph, acc, o);
+                ec_pair_vjp(a, prim(jj), n[ii] + n[jj], n[SL + ii] + n[SL + jj], n[2 * SL + ii] + n[2 * SL + jj], mu, ph, acc, o);
+                store(jj, o);
             }
-            const int from = (lw * N + (i >= k ? i - k : i - k + N)) & 31;
-            acc.rho += __shfl_sync(0xffffffffu, o.rho, from);
-            acc.u0 += __shfl_sync(0xffffffffu, o.u0, from);
-            acc.u1 += __shfl_sync(0xffffffffu, o.u1, from);
-            acc.u2 += __shfl_sync(0xffffffffu, o.u2, from);
-            acc.beta += __shfl_sync(0xffffffffu, o.beta, from);
-            acc.c += __shfl_sync(0xffffffffu, o.c, from);
-        }
-        if (go) {
-            double* B = se + C::B + 6 * l * SL + ii;
-            B[0] = acc.rho;
-            B[SL] = acc.u0;
-            B[2 * SL] = acc.u1;
-            B[3 * SL] = acc.u2;
-            B[4 * SL] = acc.beta;
-            B[5 * SL] = acc.c;
+            store(ii, acc);
         }
     }
 }
