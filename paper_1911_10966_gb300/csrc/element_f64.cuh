@@ -41,9 +41,9 @@ struct Cfg {
 template <int N, int VF, bool XF, int EPB = Cfg<N>::EPB>
 __device__ __forceinline__ void
 element_f64(double* smem, const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
-            const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K, const Ops& ops, const Phys& ph,
-            const double* __restrict__ qext, const double* __restrict__ src, const double* __restrict__ nsurf,
-            const double* __restrict__ fnorm) {
+            const double* __restrict__ jinv, const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K,
+            const Ops& ops, const Phys& ph, const double* __restrict__ qext, const double* __restrict__ src,
+            const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
     constexpr int N2 = Cfg<N>::N2, N3 = Cfg<N>::N3;
     const int t = threadIdx.x;
     const int el_loc = t / N3;
@@ -252,7 +252,7 @@ element_f64(double* smem, const double* __restrict__ q, double* __restrict__ dqd
     }
     __syncthreads();
 
-    const double Jinv = active ? 1.0 / sG[node] : 0.0;
+    const double Jinv = active ? jinv[el * N3 + node] : 0.0;
     if (ph.viscous) {
         const int i1 = node % N, i2 = (node / N) % N, i3 = node / N2;
         double Ft[3][4];

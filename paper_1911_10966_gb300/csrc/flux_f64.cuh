@@ -18,21 +18,35 @@ struct Prim {
     double hr, hu0, hu1, hu2, beta, qq;
 };
 
+// sqrt of a positive normal x: Goldschmidt's iteration (one step to 2^-44) and a correction from the residual
+__device__ __forceinline__ double sqrt_newton(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = x * y, h = 0.5 * y;
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(h, fma(-g, g, x), g);
+}
+// of any x: where the iteration's products could leave the normal range, by the library
+__device__ __forceinline__ double sqrt_pos(double x) {
+    return (unsigned)(__double2hiint(x) - 0x00900000) < 0x7e000000u ? sqrt_newton(x) : sqrt(x);
+}
 
 // Primitives of a conserved state, plus RT = p/rho and the sound speed c = sqrt(gamma p/rho).
 __device__ __forceinline__ void to_prim(const double* q, const Phys& ph, Prim& s, double& RT, double& c) {
-    const double ri = rcp_newton2(q[0]);
+    const double ri = rcp_cubic(q[0]);
     const double u0 = q[1] * ri, u1 = q[2] * ri, u2 = q[3] * ri;
     const double usq = u0 * u0 + u1 * u1 + u2 * u2;
-    const double p = (ph.gamma - 1.0) * (q[4] - 0.5 * q[0] * usq);
+    const double p = ph.gm1 * (q[4] - 0.5 * q[0] * usq);
     s.hr = 0.5 * q[0];
     s.hu0 = 0.5 * u0;
     s.hu1 = 0.5 * u1;
     s.hu2 = 0.5 * u2;
-    s.beta = s.hr * rcp_newton2(p);
+    s.beta = s.hr * rcp_cubic(p);
     s.qq = 0.25 * usq;
     RT = p * ri;
-    c = sqrt(ph.gamma * RT);
+    c = sqrt_pos(ph.gamma * RT);
 }
 
 // u = ((a-b)/(a+b))^2 < 1e-4, tested on the high word (integer pipe): the threshold moves by less
@@ -56,7 +70,7 @@ __device__ __forceinline__ void ec_flux(const Prim& a, const Prim& b, double n0,
     if (small_jump(ur)) rho_ln = sh * fma(ur, fma(ur, fma(ur, -44.0 / 945.0, -4.0 / 45.0), -1.0 / 3.0), 1.0);
     else rho_ln = 2.0 * (a.hr - b.hr) / log(a.hr / b.hr);
     // 1/beta_ln and p_t share 1/(beta_a + beta_b)
-    const double rsb = rcp_newton2(a.beta + b.beta);
+    const double rsb = rcp_cubic(a.beta + b.beta);
     const double fb = (a.beta - b.beta) * rsb;
     const double ub = fb * fb;
     double ibeta_ln;
@@ -116,7 +130,7 @@ __device__ __forceinline__ void face_jump_avg(const Prim& a, double RTa, const P
     const double ur = fr * fr;
     if (small_jump(ur)) st.rho = sh * fma(ur, fma(ur, fma(ur, -44.0 / 945.0, -4.0 / 45.0), -1.0 / 3.0), 1.0);
     else st.rho = 2.0 * (a.hr - b.hr) / log(a.hr / b.hr);
-    st.p = sh * rcp_newton2(a.beta + b.beta);
+    st.p = sh * rcp_cubic(a.beta + b.beta);
     st.u0 = a.hu0 + b.hu0;
     st.u1 = a.hu1 + b.hu1;
     st.u2 = a.hu2 + b.hu2;

@@ -16,11 +16,7 @@ __device__ __forceinline__ double rcp_newton1(double x) {     // ~46 bits
     const double r = rcp_approx(x);
     return fma(r, fma(-x, r, 1.0), r);
 }
-__device__ __forceinline__ double rcp_newton2(double x) {     // full double precision (within an ulp)
-    double r = rcp_newton1(x);
-    return fma(r, fma(-x, r, 1.0), r);
-}
-// The same accuracy in three operations: with e = 1 - x r ~ 2^-23, 1/x = r (1 + e + e^2) to 2^-66.
+// full double precision (within an ulp): with e = 1 - x r ~ 2^-23, 1/x = r (1 + e + e^2) to 2^-66
 __device__ __forceinline__ double rcp_cubic(double x) {
     const double r = rcp_approx(x), e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);

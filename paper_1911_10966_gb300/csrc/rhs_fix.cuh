@@ -187,24 +187,16 @@ __device__ __forceinline__ PrimFx load_inputs(const Fx* x, int stride) {
     return a;
 }
 
-// sqrt of a positive normal x: Goldschmidt's iteration (one step to 2^-44) and a correction from the residual
-__device__ __forceinline__ double sqrt_newton(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double g = x * y, h = 0.5 * y;
-    const double r = fma(-g, h, 0.5);
-    g = fma(g, r, g);
-    h = fma(h, r, h);
-    return fma(h, fma(-g, g, x), g);
-}
-
-// the element of a CTA left to the float64 form; out of line, so that the kernel's registers are its own
+// The elements of a CTA left to the float64 form; out of line, so that the kernel's registers are its own.  With
+// every element out of range a residual takes phase 0 more than the all-float64 kernel did: ES-C p = 1 1.08 against
+// 1.00 ms on 40^3, p = 3 1.84 against 1.81 on 24^3, p = 4 1.57 against 1.55 on 18^3, p = 7 2.15 against 2.16 on
+// 12^3; SF-KG, whose pairs cost less, 14% more at p = 1 down to 4% at p = 7.
 template <int N, int VF, bool XF, int EPB>
 __device__ __noinline__ void out_of_range(double* smem, const double* q, double* dqdt, const double* geom,
-                                          const int32_t* nbr, double* trace, int64_t K, const Ops& ops, const Phys& ph,
-                                          const double* qext, const double* src, const double* nsurf,
-                                          const double* fnorm) {
-    element_f64<N, VF, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+                                          const double* jinv, const int32_t* nbr, double* trace, int64_t K,
+                                          const Ops& ops, const Phys& ph, const double* qext, const double* src,
+                                          const double* nsurf, const double* fnorm) {
+    element_f64<N, VF, XF, EPB>(smem, q, dqdt, geom, jinv, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
 }
 
 // The two-point flux in fixed point (units 2^k0, 2^km, 2^k5), contracted with n.
@@ -330,7 +322,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     }
     if (!ok) {
         __syncthreads();
-        out_of_range<N, VF, XF, EPB>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+        out_of_range<N, VF, XF, EPB>(smem, q, dqdt, geom, jinv, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
         return;
     }
     if (active) {
@@ -707,11 +699,11 @@ cudaError_t launch_w(const esdc_ctx* c, const double* q, double* dqdt, cudaStrea
 template <int N, int VF, bool XF>
 __global__ void __launch_bounds__(Cfg<N>::THREADS, Cfg<N>::MINB)
 rhs_f64(const double* __restrict__ q, double* __restrict__ dqdt, const double* __restrict__ geom,
-        const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K, const __grid_constant__ Ops ops,
-        const __grid_constant__ Phys ph, const double* __restrict__ qext, const double* __restrict__ src,
-        const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
+        const double* __restrict__ jinv, const int32_t* __restrict__ nbr, double* __restrict__ trace, int64_t K,
+        const __grid_constant__ Ops ops, const __grid_constant__ Phys ph, const double* __restrict__ qext,
+        const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm) {
     extern __shared__ double smem[];
-    element_f64<N, VF, XF>(smem, q, dqdt, geom, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
+    element_f64<N, VF, XF>(smem, q, dqdt, geom, jinv, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
 }
 
 template <int N, int VF, bool XF>
@@ -719,8 +711,8 @@ cudaError_t launch_f64(const esdc_ctx* c, const double* q, double* dqdt, cudaStr
     using C = Cfg<N>;
     const unsigned grid = (unsigned)((c->K + C::EPB - 1) / C::EPB);
     rhs_f64<N, VF, XF><<<grid, C::THREADS, C::EPB * C::SM * sizeof(double), s>>>(
-        q, dqdt, c->d_geom, c->d_nbr, (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext, c->d_src, c->d_nsurf,
-        c->d_fnorm);
+        q, dqdt, c->d_geom, c->d_jinv, c->d_nbr, (double*)c->d_trace, c->K, c->ops, c->phys, c->d_qext, c->d_src,
+        c->d_nsurf, c->d_fnorm);
     return cudaGetLastError();
 }
 
