@@ -33,6 +33,11 @@ using Fx = FxPair;
 ESDC_HD Fx fx_split(long long v) { return {(int)(v >> 30), (int)v & 0x3fffffff}; }
 
 ESDC_HD Fx fx_add(Fx a, Fx b) { return {a.h + b.h, a.l + b.l}; }
+// a sum of two with its low limb below 2^30 again
+ESDC_HD Fx fx_sum(Fx a, Fx b) {
+    const int l = a.l + b.l;
+    return {a.h + b.h + (l >> 30), l & 0x3fffffff};
+}
 ESDC_HD Fx fx_sub(Fx a, Fx b) { return {a.h - b.h, a.l - b.l}; }
 
 // 32 x 32 -> 64 signed products as single instructions: a limb is known not to be negative, and a
@@ -86,6 +91,13 @@ ESDC_HD long long fx_mul2(Fx a, Fx b, Fx c, Fx d) {
     t = mad_wide(c.l, d.h, mad_wide(c.h, d.l, t));
     return mad_wide(a.h, b.h, mad_wide(c.h, d.h, t >> 30));
 }
+// the same times 2^SH
+template <int LL, int SH>
+ESDC_HD long long fx_mul2_shl(Fx a, Fx b, Fx c, Fx d) {
+    long long t = mad_wide(a.l, b.h, mad_wide(a.h, b.l, (kFxHalf >> SH) + LL * kFxLow));
+    t = mad_wide(c.l, d.h, mad_wide(c.h, d.l, t));
+    return (mad_wide(a.h, b.h, mul_wide(c.h, d.h)) << SH) + (t >> (30 - SH));
+}
 // one more product added to the limb sums (hi, mid) of a dot product; fx_dot_end closes it
 ESDC_HD void fx_mac(long long& hi, long long& mid, Fx a, Fx b) {
     hi = mad_wide(a.h, b.h, hi);
@@ -105,6 +117,17 @@ ESDC_HD long long fx_dot(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f) {
 template <int LL, int SH>
 ESDC_HD long long fx_dot_shl(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f) {
     long long mid = mad_wide(a.l, b.h, mad_wide(a.h, b.l, (kFxHalf >> SH) + LL * kFxLow));
+    mid = mad_wide(c.l, d.h, mad_wide(c.h, d.l, mid));
+    mid = mad_wide(e.l, f.h, mad_wide(e.h, f.l, mid));
+    const long long hh = mad_wide(a.h, b.h, mad_wide(c.h, d.h, mul_wide(e.h, f.h)));
+    return (hh << SH) + (mid >> (30 - SH));
+}
+
+// the same with the low limbs' products, normalised operands: rounded once, and 0 for products of zeros
+template <int SH>
+ESDC_HD long long fx_dot_exact_shl(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f) {
+    const long long low = mad_wide(a.l, b.l, mad_wide(c.l, d.l, mul_wide(e.l, f.l)));
+    long long mid = mad_wide(a.l, b.h, mad_wide(a.h, b.l, (low >> 30) + (kFxHalf >> SH)));
     mid = mad_wide(c.l, d.h, mad_wide(c.h, d.l, mid));
     mid = mad_wide(e.l, f.h, mad_wide(e.h, f.l, mid));
     const long long hh = mad_wide(a.h, b.h, mad_wide(c.h, d.h, mul_wide(e.h, f.h)));
@@ -234,12 +257,15 @@ ESDC_HD int fx_clamp(int a) { return a > 62 ? 62 : a; }
 
 // Er, Eu, Eb, En: largest biased exponents of the half density, half velocity, beta and metric terms;
 // Er0, Eb0: smallest of half density and beta.  kg: exponent of inv_gm1 = c 2^kg, 1/2 <= c < 1.
-// Bounds in Q60: densities and betas < 1/2, velocities and metrics < 1/4 (the limb products of
-// ubar.n then sum to at most 3 (2 1/2 + 1/2) = 4.5 2^60, a sum of two having a low limb of up to 2^31),
-// |u|^2/4 < 3/8, ubar.n < 3/4 and kept doubled, mass flux < 3/2, p_t <= 1, momentum flux < 5/4 (7/8 if
-// the pressure part sets its exponent; three products with it would reach 3 (2 5/4 + 1/2) = 9 2^60, so
-// the energy flux sums them in two parts), energy coefficient < 1.01, energy flux < 2.2.  All but p_t and the coefficient carry a factor S_ij (or 1 on a
-// face), |S_ij| with row sums below 3.41, so their sums over a line stay inside 63 bits.
+// Bounds in Q60: densities and betas < 1/2, velocities and metrics < 1/4, |u|^2/4 < 3/8, ubar.n < 3/4 and
+// kept doubled, mass flux < 3/2, p_t <= 1, momentum flux < 5/4 (7/8 if the pressure part sets its exponent)
+// and kept doubled, energy coefficient < 1.01, energy flux < 2.2.  Velocity sums are normalised: three products
+// of a momentum flux with sums whose low limb goes up to 2^31 would reach 3 (2 5/4 + 1/2) = 9 2^60, with limbs
+// below 2^30 they stay below 3 (5/4 + 1/2) 2^60.  All but p_t and the coefficient carry a factor S_ij (or 1 on a
+// face), |S_ij| with row sums below 3.41 (p <= 7), 4.86 (p = 15).  For a given i a flux of bound F, a product of
+// arithmetic means of i and j times positive factors, stays within c +- 0.575 F with |c| < F/2, and the rows of S
+// sum to +-1/2 or 0, so the sum over a line is below F/4 + 0.575 F (row sum) = 2.2 F, 3.05 F: inside 63 bits for
+// the largest F, the doubled momentum flux's 5/2.  Partial sums may wrap, hence unsigned.
 // Ey, Ez: largest exponents of mu RT/J and kappa/R RT^2/J.
 ESDC_HD FixScale fix_scale(int Er, int Er0, int Eu, int Eb, int Eb0, int En, int Ey, int Ez, int kg) {
     FixScale s;
@@ -254,14 +280,15 @@ ESDC_HD FixScale fix_scale(int Er, int Er0, int Eu, int Eb, int Eb0, int En, int
     s.fb = pow2f(60 - s.ib);
     s.k0 = s.kr + s.ku + s.kn - 1;
     const int ka = s.k0 + s.ku, kb = s.kr + s.ib - s.kb + s.kn;
-    s.km = fx_max(ka, kb);
-    s.sA = fx_clamp(s.km - ka);
-    s.sB = fx_clamp(s.km - kb);
+    const int k1 = fx_max(ka, kb);
+    s.km = k1 - 1;
+    s.sA = fx_clamp(k1 - ka);
+    s.sB = fx_clamp(k1 - kb);
     s.kA = kg + s.ib - s.kb;
     const int kc = fx_max(s.kA, s.kq);
     s.sc = fx_clamp(kc - s.kA);
     s.sq = fx_clamp(kc - s.kq);
-    const int kC = s.k0 + kc, kM = s.ku + s.km;
+    const int kC = s.k0 + kc, kM = s.ku + k1;
     s.k5 = kC - kM >= (kb > ka ? 1 : 2) ? kC : fx_max(kC, kM) + 1;
     s.sC = fx_clamp(s.k5 - kC);
     s.sD = fx_clamp(s.k5 - kM);
@@ -273,7 +300,7 @@ ESDC_HD FixScale fix_scale(int Er, int Er0, int Eu, int Eb, int Eb0, int En, int
 }
 
 // The same for the Kennedy-Gruber flux; Eq, Ep: largest exponents of PrimFx::q and p.  Bounds: q and p < 1/2,
-// mass flux < 3/2, momentum flux < 5/4, energy flux < 3/2 (each with its factor S_ij).
+// mass flux < 3/2, momentum flux < 5/4 (kept doubled), energy flux < 9/4 (each with its factor S_ij).
 ESDC_HD FixScale fix_scale_kg(int Er, int Eu, int Eb, int En, int Ey, int Ez, int Eq, int Ep) {
     FixScale s = {};
     s.kr = Er - 1021;
@@ -283,14 +310,14 @@ ESDC_HD FixScale fix_scale_kg(int Er, int Eu, int Eb, int En, int Ey, int Ez, in
     s.kq = Eq - 1021;
     s.kp = Ep - 1021;
     s.k0 = s.kr + s.ku + s.kn - 1;
-    const int ka = s.k0 + s.ku, kb = s.kp + s.kn;
-    s.km = fx_max(ka, kb);
-    s.sA = fx_clamp(s.km - ka);
-    s.sB = fx_clamp(s.km - kb);
+    const int ka = s.k0 + s.ku, kb = s.kp + s.kn, k1 = fx_max(ka, kb);
+    s.km = k1 - 1;
+    s.sA = fx_clamp(k1 - ka);
+    s.sB = fx_clamp(k1 - kb);
     const int kC = s.k0 + s.kq, kM = s.kp + s.ku + s.kn - 1;
-    s.k5 = fx_max(kC, kM) + 1;
-    s.sC = fx_clamp(s.k5 - 1 - kC);              // the sum's last bit is rounded off once (kg_flux_fx)
-    s.sD = fx_clamp(s.k5 - 1 - kM);
+    s.k5 = kC == kM ? kC + 1 : fx_max(kC, kM);
+    s.sC = fx_clamp(s.k5 - kC);
+    s.sD = fx_clamp(s.k5 - kM);
     s.hC = (1ll << s.sC) >> 1;
     s.hD = (1ll << s.sD) >> 1;
     s.ky = Ey - 1021;
@@ -473,33 +500,32 @@ ESDC_HD void ec_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, F
     if ((unsigned)(ir + kFxNear) >= 2u * kFxNear || (unsigned)(ib + kFxNear) >= 2u * kFxNear)
         log_means_far(sh, dh, db, rs, g, s, lm, rl, A);
     const Fx rlf = fx_split(rl);
-    const Fx v0 = fx_add(a.u0, b.u0), v1 = fx_add(a.u1, b.u1), v2 = fx_add(a.u2, b.u2);
-    const Fx un = fx_split(fx_dot_shl<6, 1>(v0, n0, v1, n1, v2, n2));
+    const Fx v0 = fx_sum(a.u0, b.u0), v1 = fx_sum(a.u1, b.u1), v2 = fx_sum(a.u2, b.u2);
+    const Fx un = fx_split(fx_dot_shl<3, 1>(v0, n0, v1, n1, v2, n2));
     const long long f1 = fx_mul(rlf, un);
     const long long pt = fx_mul<2>(sh, rs);
     const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(pt >> s.sB);
     f[0] = f1;
-    f[1] = fx_mul2<3>(fa, v0, pa, n0);
-    f[2] = fx_mul2<3>(fa, v1, pa, n1);
-    f[3] = fx_mul2<3>(fa, v2, pa, n2);
+    f[1] = fx_mul2_shl<2, 1>(fa, v0, pa, n0);
+    f[2] = fx_mul2_shl<2, 1>(fa, v1, pa, n1);
+    f[3] = fx_mul2_shl<2, 1>(fa, v2, pa, n2);
     const Fx c5 = fx_split((A >> s.sc) - (fx_join(fx_add(a.q, b.q)) >> s.sq));
-    const Fx m0 = fx_split(f[1]), m1 = fx_split(f[2]), m2 = fx_split(f[3]);
-    const long long vm = fx_mul2<4>(v0, m0, v1, m1) + fx_mul<2>(v2, m2);
-    f[4] = ((fx_mul(fx_split(f1), c5) + s.hC) >> s.sC) + ((vm + s.hD) >> s.sD);
+    const Fx m0 = fx_split(f[1] >> 1), m1 = fx_split(f[2] >> 1), m2 = fx_split(f[3] >> 1);
+    f[4] = ((fx_mul(fx_split(f1), c5) + s.hC) >> s.sC) + ((fx_dot(v0, m0, v1, m1, v2, m2) + s.hD) >> s.sD);
 }
 
 // The Kennedy-Gruber flux of flux_f64.cuh (kg_flux), units as above
 ESDC_HD void kg_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, const FixScale& s, long long f[5]) {
-    const Fx sh = fx_add(a.r, b.r), pt = fx_add(a.p, b.p);
-    const Fx v0 = fx_add(a.u0, b.u0), v1 = fx_add(a.u1, b.u1), v2 = fx_add(a.u2, b.u2);
-    const Fx un = fx_split(fx_dot_shl<6, 1>(v0, n0, v1, n1, v2, n2));
-    const long long f1 = fx_mul<2>(sh, un);
+    const Fx sh = fx_sum(a.r, b.r), pt = fx_sum(a.p, b.p);
+    const Fx v0 = fx_sum(a.u0, b.u0), v1 = fx_sum(a.u1, b.u1), v2 = fx_sum(a.u2, b.u2);
+    const Fx un = fx_split(fx_dot_exact_shl<1>(v0, n0, v1, n1, v2, n2));
+    const long long f1 = fx_mul(sh, un);
     const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(fx_join(pt) >> s.sB);
     f[0] = f1;
-    f[1] = fx_mul2<3>(fa, v0, pa, n0);
-    f[2] = fx_mul2<3>(fa, v1, pa, n1);
-    f[3] = fx_mul2<3>(fa, v2, pa, n2);
-    f[4] = (((fx_mul<2>(fx_split(f1), fx_add(a.q, b.q)) + s.hC) >> s.sC) + ((fx_mul<2>(pt, un) + s.hD) >> s.sD) + 1) >> 1;
+    f[1] = fx_mul2_shl<2, 1>(fa, v0, pa, n0);
+    f[2] = fx_mul2_shl<2, 1>(fa, v1, pa, n1);
+    f[3] = fx_mul2_shl<2, 1>(fa, v2, pa, n2);
+    f[4] = ((fx_mul<2>(fx_split(f1), fx_add(a.q, b.q)) + s.hC) >> s.sC) + ((fx_mul(pt, un) + s.hD) >> s.sD);
 }
 
 // The Euler flux of one node contracted with n (euler_flux_prim), units as above

@@ -398,7 +398,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             const int ii = line_slot<N>(l, i < N ? i : 0, c1, c2);
             const PrimFx a = load_inputs<VF>(XP + ii, SL);
             const Fx na0 = XN[ii], na1 = XN[SL + ii], na2 = XN[2 * SL + ii];
-            long long acc[5] = {0, 0, 0, 0, 0};
+            unsigned long long acc[5] = {0, 0, 0, 0, 0};
 #pragma unroll 1
             for (int k = 1; k <= N / 2; ++k) {
                 const int j = i + k < N ? i + k : i + k - N;
@@ -413,18 +413,18 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                              n2 = fx_split(fx_mul<2>(S, fx_add(na2, XN[2 * SL + jj])));
                     two_point<VF>(a, b, n0, n1, n2, ops.CG, ph.inv_gm1, s, Pv);
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) acc[v] -= Pv[v];
+                    for (int v = 0; v < 5; ++v) acc[v] -= (unsigned long long)Pv[v];
                 }
                 const int from = (lw * N + (i >= k ? i - k : i - k + N)) & 31;
 #pragma unroll
-                for (int v = 0; v < 5; ++v) acc[v] += __shfl_sync(0xffffffffu, Pv[v], from);
+                for (int v = 0; v < 5; ++v) acc[v] += (unsigned long long)__shfl_sync(0xffffffffu, Pv[v], from);
             }
             if (go) {
                 double* R = se + C::R + l * 5 * SL + ii;
                 const double w = sW[i];
 #pragma unroll
                 for (int v = 0; v < 5; ++v)
-                    R[v * SL] = w * fx_to_double(acc[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km));
+                    R[v * SL] = w * fx_to_double((long long)acc[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km));
             }
         }
     }

@@ -296,11 +296,7 @@ constexpr int fix_smem_doubles() {
 // 1..N/2 the lane of node i evaluates the pair (i, i + k mod N), S_ij f is summed in registers on one side and
 // by a shuffle on the other.  One warp evaluates the 32 face terms while the others begin on the lines, which a
 // counter hands out; which warp, changes with the plane.
-// The rows of |S| sum to 4.86 here, which keeps the mass and momentum fluxes' sums (bounds 3/2, 5/4) inside 63 bits
-// by themselves.  ES-C's energy flux (bound F = 2.2) does too, although 4.86 F does not: f_ij is a product of
-// arithmetic means of i and j, u.n and n among them, times factors positive but for the kinetic u_i.u_j, so that
-// for a given i it spans at most 1.15 F, c +- 0.575 F with |c| < F/2, and the rows of S itself sum to +-1/2 or 0:
-// |sum_j S_ij f_ij| < 1/4 F + 4.86 0.575 F = 3.05 F < 8.  Partial sums may wrap, hence unsigned.
+// The sums over a line stay inside 63 bits by the bounds at fix_scale.
 // In float64 the pairs kept that pipe (64 clocks per instruction and scheduler) busy; bound now by the multiply
 // and shift pipes and their latency.  Viscous ES-C residual of the Taylor-Green flow on 6 x 5 x 7 elements, with
 // theta from here and the divergence's line products in fixed point too: 3.89 -> 1.00 ms, of which this kernel

@@ -116,6 +116,21 @@ int main() {
                     check("DC", f, ref, kd);
                 }
             }
+    // SF-KG mass flux through a face that the flow is parallel to, its velocity and normal along
+    // different axes: products of zeros, exactly zero in float64 whatever the density and pressure
+    for (int d = 0; d < 3; ++d)
+        for (int t = 0; t < 16; ++t) {
+            const double hr = kTop[t & 3], u = kTop[t >> 2], e = 2.0 + 0.1 * t, p = 0.7 + 0.01 * t;
+            const FixScale s = fix_scale_kg(biased_exp(hr), biased_exp(u), 1022, 1022, 1000, 1000, biased_exp(e), biased_exp(p));
+            Fx h[3] = {}, n[3] = {};
+            h[d] = fx_split(fx_from_double(u, s.ku));
+            n[(d + 1) % 3] = fx_split(fx_from_double(0.7, s.kn));
+            auto f = [](double x, int k) { return fx_split(fx_from_double(x, k)); };
+            const PrimFx a = {f(hr, s.kr), h[0], h[1], h[2], f(0.5, s.kb), f(e, s.kq), f(p, s.kp)};
+            long long F[5];
+            kg_flux_fx(a, a, n[0], n[1], n[2], s, F);
+            if (F[0] != 0) wrong++, std::printf("SF-KG mass flux of parallel flow: %lld units\\n", F[0]);
+        }
     return wrong != 0;
 }
 """
