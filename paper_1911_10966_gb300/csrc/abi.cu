@@ -769,9 +769,7 @@ int esdc_create(const esdc_setup_t* setup, const double* xyz, esdc_ctx** out) {
                 c->ops.SF[k - 1][i] = esdc::fx_split(esdc::fx_from_double(c->ops.S[i][(i + k) % hs.N], 0));
         }
         for (int i = 0; i < hs.N; ++i)
-            for (int j = 0; j < hs.N; ++j)       // the rows of S sum to -E_ii/2
-                c->ops.MF[i][j] = esdc::fx_split(esdc::fx_from_double(
-                    i != j ? c->ops.S[i][j] : (i == 0 ? 0.5 : (i == hs.N - 1 ? -0.5 : 0.0)), 1));
+            for (int j = 0; j < hs.N; ++j) c->ops.MF[i][j] = esdc::fx_split(esdc::fx_from_double(c->ops.S[i][j], 0));
         std::frexp(c->ops.winv[0], &c->ops.kW);          // the end weights are the smallest
         for (int i = 0; i < hs.N; ++i) {
             std::frexp(c->ops.winv[i], &c->ops.WE[i]);

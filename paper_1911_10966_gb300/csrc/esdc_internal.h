@@ -34,7 +34,7 @@ struct Ops {
     FxPair WB[kMaxN];          // 1/w_i 2^-kW < 1
     int WE[kMaxN];             // 1/w_i < 2^WE[i]
     int kW;
-    FxPair MF[kMaxN][kMaxN];   // S_ij / 2, on the diagonal half the row's sum 1/2, 0, .., -1/2 (DC)
+    FxPair MF[kMaxN][kMaxN];   // S_ij (DC's line products)
     FxPair DF[kMaxN][kMaxN];   // D_ij 2^-kD
     FxPair LF;                 // interface lift 1/(2 w_0) 2^-kD
     int kD;

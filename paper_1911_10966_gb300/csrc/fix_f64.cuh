@@ -325,20 +325,14 @@ ESDC_HD FixScale fix_scale_kg(int Er, int Eu, int Eb, int En, int Ey, int Ez, in
     return s;
 }
 
-// The same for nodal fluxes contracted with n < 1/4, whose densities and enthalpies are not summed: both < 1,
-// u.n < 3/16 and kept quadrupled, mass and energy flux < 3/4, momentum flux < 5/16.  Their products with half
-// of S: absolute row sums < 2.4 with the diagonal, at most seven limbs besides the head's, so the limb sums
-// stay below 7.6 2^60.
-ESDC_HD FixScale fix_scale_dc(int Er, int Eu, int Eb, int En, int Ey, int Ez, int Eq, int Ep) {
-    FixScale s = fix_scale_kg(Er, Eu, Eb, En, Ey, Ez, Eq, Ep);
-    --s.kr;
-    --s.kq;
-    s.k0 = s.kr + s.ku + s.kn;
-    const int ka = s.k0 + s.ku + 1, kb = s.kp + 1 + s.kn;
-    s.km = fx_max(ka, kb);
-    s.sA = fx_clamp(s.km - ka);
-    s.sB = fx_clamp(s.km - kb);
-    s.k5 = s.k0 + s.kq;
+// DC, whose fluxes are float64 (rhs_fix.cuh): the viscous chain's inputs only.
+ESDC_HD FixScale fix_scale_dc(int Eu, int Eb, int En, int Ey, int Ez) {
+    FixScale s = {};
+    s.ku = Eu - 1020;
+    s.kb = Eb - 1021;
+    s.kn = En - 1020;
+    s.ky = Ey - 1021;
+    s.kz = Ez - 1021;
     return s;
 }
 
@@ -382,8 +376,7 @@ ESDC_HD bool fix_range_ok(int Er, int Er0, int Eu, int Eb, int Eb0, int En) {
 }
 
 // Per-node inputs of the pair loop, Q60 limbs: half density, half velocity, beta, and
-//   ES-C: q = |u|^2/4;   SF-KG: q = RT/(2(gamma - 1)) + |u|^2/4, p = half the pressure;
-//   DC: q = the specific enthalpy, p = half the pressure.
+//   ES-C: q = |u|^2/4;   SF-KG: q = RT/(2(gamma - 1)) + |u|^2/4, p = half the pressure.
 struct PrimFx {
     Fx r, u0, u1, u2, b, q, p;
 };
@@ -526,18 +519,6 @@ ESDC_HD void kg_flux_fx(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, c
     f[2] = fx_mul2_shl<2, 1>(fa, v1, pa, n1);
     f[3] = fx_mul2_shl<2, 1>(fa, v2, pa, n2);
     f[4] = ((fx_mul<2>(fx_split(f1), fx_add(a.q, b.q)) + s.hC) >> s.sC) + ((fx_mul(pt, un) + s.hD) >> s.sD);
-}
-
-// The Euler flux of one node contracted with n (euler_flux_prim), units as above
-ESDC_HD void euler_flux_fx(const PrimFx& a, Fx n0, Fx n1, Fx n2, const FixScale& s, long long f[5]) {
-    const Fx un = fx_split(fx_dot_shl<3, 2>(a.u0, n0, a.u1, n1, a.u2, n2));
-    const long long f1 = fx_mul(a.r, un);
-    const Fx fa = fx_split(f1 >> s.sA), pa = fx_split(fx_join(a.p) >> s.sB);
-    f[0] = f1;
-    f[1] = fx_mul2(fa, a.u0, pa, n0);
-    f[2] = fx_mul2(fa, a.u1, pa, n1);
-    f[3] = fx_mul2(fa, a.u2, pa, n2);
-    f[4] = fx_mul(fx_split(f1), a.q);
 }
 
 // ln x in Q58 for 2^-44 <= x < 2^45 by table reduction (Tang's method, ACM TOMS 15, 1989): x = m 2^e, m in

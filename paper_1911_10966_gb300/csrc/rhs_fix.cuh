@@ -12,8 +12,9 @@
 //   1. volume: one thread per (node, direction), whole lines side by side in a warp.  At cyclic distance
 //      k = 1..N/2 the thread of node i evaluates the pair (i, i + k mod N), so that each pair is
 //      evaluated once; S_ij f is summed in registers on one side and by a shuffle on the other.  DC: the
-//      nodal contravariant fluxes per node, then one thread per line and variable.
-//   2. interface: one thread per face node; two-point flux in fixed point, dissipation in float64.
+//      nodal contravariant fluxes per node in float64, then one thread per line and variable, each line in
+//      fixed point under the largest exponent of its direction and variable in the element.
+//   2. interface: one thread per face node; two-point flux in fixed point (DC: float64), dissipation in float64.
 //   3. viscous: lines of w for theta_a = D_a w + lift (one thread per line and variable, the operator
 //      from the constant bank), one thread per node for the fluxes, lines again for the divergence.
 //
@@ -158,7 +159,7 @@ __device__ __forceinline__ void pair_exponents(const double (&pi)[NP], int (&E)[
     E[2] = max(biased_exp(pi[1]), max(biased_exp(pi[2]), biased_exp(pi[3])));
     E[3] = (unsigned)double_hi(pi[4]) >> 20;
     E[4] = 4096 - E[3];
-    if constexpr (NP == 7) {
+    if constexpr (NE == 10) {
         E[8] = biased_exp(pi[5]);
         E[9] = biased_exp(pi[6]);
     }
@@ -168,15 +169,17 @@ template <int VF, int NE>
 __device__ __forceinline__ FixScale element_scale(const int (&E)[NE], int kg) {
     if constexpr (VF == kFluxESC) return fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], kg);
     else if constexpr (VF == kFluxKG) return fix_scale_kg(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
-    else return fix_scale_dc(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
+    else return fix_scale_dc(E[2], E[3], E[5], E[6], E[7]);
 }
-// a node's (or neighbour's) pair inputs from float64 to limbs, arrays `stride` apart
+// a node's (or neighbour's) pair inputs from float64 to limbs, arrays `stride` apart; of DC's only those of the
+// viscous terms
 template <int VF>
 __device__ __forceinline__ void scale_inputs(const double* p, Fx* x, int stride, const FixScale& s) {
-    x[0] = fx_split(fx_from_double(p[0], s.kr));
 #pragma unroll
     for (int m = 1; m < 4; ++m) x[m * stride] = fx_split(fx_from_double(p[m * stride], s.ku));
     x[4 * stride] = fx_split(fx_from_double(p[4 * stride], s.kb));
+    if constexpr (VF == kFluxDC) return;
+    x[0] = fx_split(fx_from_double(p[0], s.kr));
     x[5 * stride] = fx_split(fx_from_double(p[5 * stride], s.kq));
     if constexpr (VF != kFluxESC) x[6 * stride] = fx_split(fx_from_double(p[6 * stride], s.kp));
 }
@@ -199,20 +202,24 @@ __device__ __noinline__ void out_of_range(double* smem, const double* q, double*
     element_f64<N, VF, XF, EPB>(smem, q, dqdt, geom, jinv, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);
 }
 
+// Euler flux contracted with n, from density, velocity, pressure and specific enthalpy
+__device__ __forceinline__ void euler_flux(double rho, double u0, double u1, double u2, double p, double H, double n0,
+                                           double n1, double n2, double (&f)[5]) {
+    f[0] = rho * fma(u2, n2, fma(u1, n1, u0 * n0));
+    f[1] = fma(f[0], u0, p * n0);
+    f[2] = fma(f[0], u1, p * n1);
+    f[3] = fma(f[0], u2, p * n2);
+    f[4] = f[0] * H;
+}
+
 // The two-point flux in fixed point (units 2^k0, 2^km, 2^k5), contracted with n.
 template <int VF>
 __device__ __forceinline__ void two_point(const PrimFx& a, const PrimFx& b, Fx n0, Fx n1, Fx n2, Fx cg, double inv_gm1,
                                           const FixScale& s, long long (&f)[5]) {
     if constexpr (VF == kFluxESC) {
         ec_flux_fx(a, b, n0, n1, n2, cg, s, LogMeanF64{a.r, b.r, a.b, b.b, s, inv_gm1}, f);
-    } else if constexpr (VF == kFluxKG) {
-        kg_flux_fx(a, b, n0, n1, n2, s, f);
     } else {
-        long long g[5];                          // the mean of the two nodal fluxes
-        euler_flux_fx(a, n0, n1, n2, s, f);
-        euler_flux_fx(b, n0, n1, n2, s, g);
-#pragma unroll
-        for (int v = 0; v < 5; ++v) f[v] = (f[v] + g[v] + 1) >> 1;
+        kg_flux_fx(a, b, n0, n1, n2, s, f);
     }
 }
 
@@ -239,9 +246,10 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm,
             const int32_t* __restrict__ kn) {
     using C = FixCfg<N, VF, WIDE>;
-    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxESC ? 8 : 10;
+    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxKG ? 10 : 8;
     extern __shared__ double smem[];
     __shared__ int sE[EPB][NE];                  // largest exponents (of 4096 - E for the smallest)
+    __shared__ int sF[VF == kFluxDC ? EPB : 1][15];       // DC: of the nodal fluxes, by direction and variable
     __shared__ FixScale sScale[EPB];
     __shared__ unsigned sMag[EPB][2];            // magnitude bits of theta: w2..w4, w5
     __shared__ Fx sS[(N / 2) * N];
@@ -259,6 +267,8 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     const int64_t eoff = el * 5 * N3;
     for (int i = t; i < EPB * NE; i += C::THREADS)
         sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? metric_exponent(kn[(int64_t)blockIdx.x * EPB + i / NE], kRhsStretch) : 0;
+    if constexpr (VF == kFluxDC)
+        for (int i = t; i < EPB * 15; i += C::THREADS) sF[i / 15][i % 15] = 0;
     if (t < EPB) sMag[t][0] = sMag[t][1] = 0;
     for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
     for (int i = t; i < N; i += C::THREADS) sW[i] = ops.winv[i];
@@ -328,6 +338,24 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     if (active) {
         const FixScale s = element_scale<VF>(sE[el_loc], ops.kg);
         if (node == 0) sScale[el_loc] = s;
+        if constexpr (VF == kFluxDC) {
+            // nodal contravariant fluxes Ftilde_l
+            const double* pi = sm + C::XP + own_slot;
+            int EF[15];
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const double* n = sm + C::XN + 3 * l * SL + own_slot;
+                double f[5];
+                euler_flux(2.0 * pi[0], 2.0 * pi[SL], 2.0 * pi[2 * SL], 2.0 * pi[3 * SL], 2.0 * pi[6 * SL], pi[5 * SL], n[0], n[SL],
+                           n[2 * SL], f);
+#pragma unroll
+                for (int v = 0; v < 5; ++v) {
+                    sm[C::R + (5 * l + v) * SL + own_slot] = f[v];
+                    EF[5 * l + v] = biased_exp(f[v]);
+                }
+            }
+            block_max<EPB == 1 || N3 % 32 == 0>(sF[el_loc], el_loc, EF, lane);
+        }
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
             const int i = C::XN + c * SL + own_slot;
@@ -349,34 +377,20 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
 
     // ---- 1. volume flux differencing
     if constexpr (VF == kFluxDC) {
-        // nodal contravariant fluxes Ftilde_l, then twice their central fluxes' differences along the lines,
-        // acc_i = sum_j S_ij (F_i + F_j) = sum_j M_ij F_j, in place
-        if (active) {
-            const FixScale& s = sScale[el_loc];
-            const PrimFx a = load_inputs<VF>(X + C::XP + own_slot, SL);
-#pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                const Fx* n = X + C::XN + 3 * l * SL + own_slot;
-                long long f[5];
-                euler_flux_fx(a, n[0], n[SL], n[2 * SL], s, f);
-#pragma unroll
-                for (int v = 0; v < 5; ++v) X[C::R + (5 * l + v) * SL + own_slot] = fx_split(f[v]);
-            }
-        }
-        __syncthreads();
+        // the nodal fluxes' differences along the lines, sum_j S_ij (F_i + F_j) with the own flux left out, which at
+        // the end nodes is half the interface flux's own part; in fixed point under the largest exponent of the
+        // direction's and variable's fluxes, in place
 #pragma unroll 1
         for (int id = t; id < n_el * 15 * N2; id += C::THREADS) {
             const int e = id / (15 * N2), r = id - e * 15 * N2;
             const int lv = r / N2, li = r - lv * N2;
-            const int l = lv / 5, v = lv - 5 * l;
-            const int c1 = li % N, c2 = li / N;
+            const int l = lv / 5, c1 = li % N, c2 = li / N;
             double* R = smem + (size_t)e * C::SM + C::R + lv * SL;
-            const FixScale& s = sScale[e];
-            const int k = (v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)) + 1;
+            const int k = sF[e][lv] - 1021;
             Fx x[N];
             long long out[N];
 #pragma unroll
-            for (int j = 0; j < N; ++j) x[j] = reinterpret_cast<const Fx*>(R)[line_slot<N>(l, j, c1, c2)];
+            for (int j = 0; j < N; ++j) x[j] = fx_split(fx_from_double(R[line_slot<N>(l, j, c1, c2)], k));
             line_product<N>(x, ops.MF, out);
 #pragma unroll
             for (int j = 0; j < N; ++j) R[line_slot<N>(l, j, c1, c2)] = -ops.winv[j] * fx_to_double(out[j], k);
@@ -472,8 +486,35 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                 n2 = fx_split(fx_from_double(nd[2], s.kn));
             }
         }
-        long long f[5];
-        two_point<VF>(a, b, n0, n1, n2, ops.CG, ph.inv_gm1, s, f);
+        [[maybe_unused]] long long f[5];
+        [[maybe_unused]] double fnb[5];          // DC: the neighbour's nodal flux
+        if constexpr (VF == kFluxDC) {
+            const double* gd = se + C::F + fn;
+            if constexpr (!XF) {
+                const double* ns = geom + (ee * 10 + 1 + 3 * l) * N3 + own;
+                nd[0] = ns[0];
+                nd[1] = ns[N3];
+                nd[2] = ns[2 * N3];
+            }
+            const double ri = rcp_cubic(qn[0]);
+            euler_flux(qn[0], qn[N3] * ri, qn[2 * N3] * ri, qn[3 * N3] * ri, 2.0 * gd[6 * 6 * N2], gd[5 * 6 * N2], nd[0], nd[1],
+                       nd[2], fnb);
+            if constexpr (XF) {
+                // optimized metrics: the own flux left out of the volume term was one with the volume metrics
+                if (nsurf) {
+                    const double *qo = q + ee * 5 * N3 + own, *nv = geom + (ee * 10 + 1 + 3 * l) * N3 + own;
+                    const double ro = rcp_cubic(qo[0]), RT = se[C::P + own];
+                    const double u0 = qo[N3] * ro, u1 = qo[2 * N3] * ro, u2 = qo[3 * N3] * ro;
+                    double fo[5];
+                    euler_flux(qo[0], u0, u1, u2, qo[0] * RT, fma(ph.gamma * ph.inv_gm1, RT, 0.5 * fma(u2, u2, fma(u1, u1, u0 * u0))),
+                               nd[0] - nv[0], nd[1] - nv[N3], nd[2] - nv[2 * N3], fo);
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) fnb[v] += fo[v];
+                }
+            }
+        } else {
+            two_point<VF>(a, b, n0, n1, n2, ops.CG, ph.inv_gm1, s, f);
+        }
         double lam = 0.0;
         double dm[5] = {0.0, 0.0, 0.0, 0.0, 0.0};      // 1/2 D (w_own - w_nbr) + interior penalty
         if (XF && (ph.dissipation == 2 || ph.ip_coef > 0.0)) {
@@ -514,7 +555,9 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         double* R = se + C::R + l * 5 * SL + os;
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            double r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * SL]);
+            double r;
+            if constexpr (VF == kFluxDC) r = fma(0.5 * wi, fnb[v], R[v * SL]);
+            else r = fma(wi, fx_to_double(f[v], v == 0 ? s.k0 : (v == 4 ? s.k5 : s.km)), R[v * SL]);
             if (ph.dissipation == 1) r = fma(-lam, q[ee * 5 * N3 + v * N3 + own] - qn[v * N3], r);
             if constexpr (XF) r = fma(-ops.winv[0], dm[v], r);
             R[v * SL] = r;

@@ -96,24 +96,15 @@ int main() {
                     }
                 }
                 {
-                    const double p = hr * (0.5 / b), e = 0.5 * g1 * (0.5 / b) + q, H = gamma * g1 * (0.5 / b) + 2 * q;
-                    FixScale s = fix_scale_kg(Er, Eu, Eb, En, 1000, 1000, biased_exp(e), biased_exp(p));
-                    PrimFx a = inputs(s, e, p);
+                    const double p = hr * (0.5 / b), e = 0.5 * g1 * (0.5 / b) + q;
+                    const FixScale s = fix_scale_kg(Er, Eu, Eb, En, 1000, 1000, biased_exp(e), biased_exp(p));
+                    const PrimFx a = inputs(s, e, p);
                     const int k[5] = {s.k0, s.km, s.km, s.km, s.k5};
                     metric(s.kn, nf);
                     kg_flux_fx(a, a, nf[0], nf[1], nf[2], s, f);
                     forward(2 * (Q)p, 0);
                     ref[4] = ref[0] * 2 * e + 2 * (Q)p * un;
                     check("SF-KG", f, ref, k);
-                    s = fix_scale_dc(Er, Eu, Eb, En, 1000, 1000, biased_exp(H), biased_exp(p));
-                    a = inputs(s, H, p);
-                    for (int d = 0; d < 3; ++d) nf[d] = fx_split(fx_from_double(n[d], s.kn)), nn[d] = n[d];
-                    un = 2 * ((Q)h[0] * nn[0] + (Q)h[1] * nn[1] + (Q)h[2] * nn[2]);
-                    euler_flux_fx(a, nf[0], nf[1], nf[2], s, f);
-                    forward(2 * (Q)p, 0);
-                    ref[4] = ref[0] * H;
-                    const int kd[5] = {s.k0, s.km, s.km, s.km, s.k5};
-                    check("DC", f, ref, kd);
                 }
             }
     // SF-KG mass flux through a face that the flow is parallel to, its velocity and normal along

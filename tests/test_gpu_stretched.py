@@ -18,9 +18,9 @@ from tests.gpu_common import EPS64, assert_parity, geometry_rounding, make_pair,
 pytestmark = pytest.mark.gpu
 
 
-def _pair(p, side, flow, flux="esc", Re=0.0, k=(2, 2, 2), warp=0.0):
+def _pair(p, side, flow, flux="esc", Re=0.0, k=(2, 2, 2), Ma=0.1):
     size = [1.0, 1.0, float(side)]
-    solver, q, mesh, gas, qo = make_pair(p, k, warp=warp, seed=2, Re=Re, box=([0.0] * 3, size), volume_flux=flux)
+    solver, q, mesh, gas, qo = make_pair(p, k, Ma=Ma, seed=2, Re=Re, box=([0.0] * 3, size), volume_flux=flux)
     x = torch.as_tensor(np.asarray(solver.coords)).reshape(qo.shape[0], 3, *qo.shape[2:])
     X = [2.0 * math.pi * x[:, d] / size[d] for d in range(3)]
     rho = 1.0 + 0.05 * torch.sin(X[0] + 0.3) + 0.05 * torch.cos(X[2]) + 0.03 * torch.sin(X[1])
