@@ -375,6 +375,19 @@ ESDC_HD bool fix_range_ok(int Er, int Er0, int Eu, int Eb, int Eb0, int En) {
            Eu < 1151 && En < 1151;
 }
 
+// Where the kinetic part sets the momentum fluxes' exponent, a velocity component much smaller than the others
+// leaves its own momentum flux, and the pressure's in it, few bits; and the energy flux is the difference of
+// larger parts.  u0, u1, u2: largest |u_m| of the element (speed_code), Eb0 as above; k is ka - kb of fix_scale.
+// Errors against extended precision, fixed point over float64, worst variable of p = 3, 4, 7 and 15 with the flow
+// along one axis: 0.88 at k = 1 (Mach 0.5), 0.9 to 1.5 at 2 (0.7, 0.85), 1.8 at 3 (1), 8 at 5 (2); in all three:
+// 0.8 at k = 3 (1), 1.0 at 5 (2), p = 15 1.3, 1.2 at 7 (4).  Hence `most`, 5, or 3 at p = 15.
+ESDC_HD int speed_code(double u) { return (double_hi(u) & 0x7fffffff) >> 8; }      // biased exponent, 12 bits below it
+ESDC_HD int speed_exponent(int u0, int u1, int u2) { return fx_max(u0, fx_max(u1, u2)) >> 12; }
+ESDC_HD bool fix_speed_ok(int u0, int u1, int u2, int Eb0, int most) {
+    const int k = 2 * speed_exponent(u0, u1, u2) + Eb0 - 3063;
+    return k <= 1 || (k <= most && fx_max(u0, fx_max(u1, u2)) + fx_max(-u0, fx_max(-u1, -u2)) <= 4096);
+}
+
 // Per-node inputs of the pair loop, Q60 limbs: half density, half velocity, beta, and
 //   ES-C: q = |u|^2/4;   SF-KG: q = RT/(2(gamma - 1)) + |u|^2/4, p = half the pressure.
 struct PrimFx {

@@ -159,17 +159,32 @@ __device__ __forceinline__ void pair_exponents(const double (&pi)[NP], int (&E)[
     E[2] = max(biased_exp(pi[1]), max(biased_exp(pi[2]), biased_exp(pi[3])));
     E[3] = (unsigned)double_hi(pi[4]) >> 20;
     E[4] = 4096 - E[3];
-    if constexpr (NE == 10) {
-        E[8] = biased_exp(pi[5]);
-        E[9] = biased_exp(pi[6]);
+}
+// The same for the residual kernels: the velocity components' speed codes apart (E[2], E[8], E[9]), and SF-KG's last
+// two inputs.
+template <int NP, int NE>
+__device__ __forceinline__ void rhs_exponents(const double (&pi)[NP], int (&E)[NE]) {
+    pair_exponents(pi, E);
+    E[2] = speed_code(pi[1]);
+    E[8] = speed_code(pi[2]);
+    E[9] = speed_code(pi[3]);
+    if constexpr (NE == 12) {
+        E[10] = biased_exp(pi[5]);
+        E[11] = biased_exp(pi[6]);
     }
+}
+template <int NE>
+__device__ __forceinline__ bool rhs_range_ok(const int (&E)[NE], int most_speed = 5) {
+    return fix_range_ok(E[0], 4096 - E[1], speed_exponent(E[2], E[8], E[9]), E[3], 4096 - E[4], E[5]) &&
+           fix_speed_ok(E[2], E[8], E[9], 4096 - E[4], most_speed) && E[6] < 1151 && E[7] < 1151;
 }
 // the element's scales from its maxima
 template <int VF, int NE>
 __device__ __forceinline__ FixScale element_scale(const int (&E)[NE], int kg) {
-    if constexpr (VF == kFluxESC) return fix_scale(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5], E[6], E[7], kg);
-    else if constexpr (VF == kFluxKG) return fix_scale_kg(E[0], E[2], E[3], E[5], E[6], E[7], E[8], E[9]);
-    else return fix_scale_dc(E[2], E[3], E[5], E[6], E[7]);
+    const int Eu = speed_exponent(E[2], E[8], E[9]);
+    if constexpr (VF == kFluxESC) return fix_scale(E[0], 4096 - E[1], Eu, E[3], 4096 - E[4], E[5], E[6], E[7], kg);
+    else if constexpr (VF == kFluxKG) return fix_scale_kg(E[0], Eu, E[3], E[5], E[6], E[7], E[10], E[11]);
+    else return fix_scale_dc(Eu, E[3], E[5], E[6], E[7]);
 }
 // a node's (or neighbour's) pair inputs from float64 to limbs, arrays `stride` apart; of DC's only those of the
 // viscous terms
@@ -246,7 +261,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
             const double* __restrict__ src, const double* __restrict__ nsurf, const double* __restrict__ fnorm,
             const int32_t* __restrict__ kn) {
     using C = FixCfg<N, VF, WIDE>;
-    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxKG ? 10 : 8;
+    constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxKG ? 12 : 10;
     extern __shared__ double smem[];
     __shared__ int sE[EPB][NE];                  // largest exponents (of 4096 - E for the smallest)
     __shared__ int sF[VF == kFluxDC ? EPB : 1][15];       // DC: of the nodal fluxes, by direction and variable
@@ -289,7 +304,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
 #pragma unroll
         for (int i = 0; i < NP; ++i) sm[C::XP + i * SL + own_slot] = pi[i];
         sm[C::P + node] = RT;
-        pair_exponents<NP>(pi, E);
+        rhs_exponents(pi, E);
         Y = ph.mu * RT * Jinv;                   // velocity gradient to stress
         Z = ph.kappa_R * RT * RT * Jinv;         // dw5 to heat flux
         E[6] = biased_exp(Y);
@@ -321,15 +336,13 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
 #pragma unroll
         for (int i = 0; i < NP; ++i) f[i * 6 * N2] = pi[i];
         f[NP * 6 * N2] = sqrt_newton(ph.gamma * RT);
-        pair_exponents<NP>(pi, E);
+        rhs_exponents(pi, E);
         block_max<EPB == 1 || (6 * N2) % 32 == 0>(sE[e], e, E, lane);
     }
     __syncthreads();
-    bool ok = true;
-    for (int e = 0; e < n_el; ++e) {
-        const int* E = sE[e];
-        ok = ok && fix_range_ok(E[0], 4096 - E[1], E[2], E[3], 4096 - E[4], E[5]) && E[6] < 1151 && E[7] < 1151;
-    }
+    bool ok;
+    if constexpr (EPB <= 2) ok = rhs_range_ok(sE[0]) && (n_el < 2 || rhs_range_ok(sE[EPB - 1]));
+    else ok = __syncthreads_and(t >= n_el || rhs_range_ok(sE[t]));
     if (!ok) {
         __syncthreads();
         out_of_range<N, VF, XF, EPB>(smem, q, dqdt, geom, jinv, nbr, trace, K, ops, ph, qext, src, nsurf, fnorm);

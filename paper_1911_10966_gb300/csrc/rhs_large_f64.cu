@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(LTHREADS, 6)
 lg_volume_fix(const double* __restrict__ q, const double* __restrict__ geom, const int32_t* __restrict__ nbr,
               const double* __restrict__ fnorm, double* __restrict__ rl, double* __restrict__ th, int64_t K,
               const __grid_constant__ OpsL ops, const __grid_constant__ Phys ph, const int32_t* __restrict__ kn) {
-    constexpr int NP = fix_inputs<VF>(), NE = VF == kFluxESC ? 8 : 10, NF = 2 * LN;
+    constexpr int NP = fix_inputs<VF>(), NE = VF == kFluxESC ? 10 : 12, NF = 2 * LN;
     extern __shared__ double sm[];
     __shared__ int sE[NE], sNext;
     __shared__ FixScale sScale;
@@ -355,7 +355,7 @@ lg_volume_fix(const double* __restrict__ q, const double* __restrict__ geom, con
         pair_inputs<VF>(qv, ph, pi, RT);
 #pragma unroll
         for (int m = 0; m < NP; ++m) sm[m * LN2 + si] = pi[m];
-        pair_exponents<NP>(pi, En);
+        rhs_exponents(pi, En);
 #pragma unroll
         for (int m = 0; m < NE; ++m) E[m] = max(E[m], En[m]);
     }
@@ -368,13 +368,13 @@ lg_volume_fix(const double* __restrict__ q, const double* __restrict__ geom, con
 #pragma unroll
         for (int m = 0; m < NP; ++m) sNb[m * NF + lane] = pi[m];
         sNb[NP * NF + lane] = sqrt_newton(ph.gamma * RT);
-        pair_exponents<NP>(pi, En);
+        rhs_exponents(pi, En);
 #pragma unroll
         for (int m = 0; m < NE; ++m) E[m] = max(E[m], En[m]);
     }
     block_max<true>(sE, 0, E, lane);
     __syncthreads();
-    if (metric_exponent(kn[el], kRhsStretch) == 2047 || !fix_range_ok(sE[0], 4096 - sE[1], sE[2], sE[3], 4096 - sE[4], sE[5])) {
+    if (metric_exponent(kn[el], kRhsStretch) == 2047 || !rhs_range_ok(sE, 3)) {
         __syncthreads();
         plane_out_of_range<VF>(sm, q, geom, nbr, fnorm, rl, th, K, ops, ph);
         return;

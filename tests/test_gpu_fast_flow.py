@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("flow", ["x", "z", "all"])
-@pytest.mark.parametrize("flux", ["dc"])
+@pytest.mark.parametrize("flux", ["esc", "kg", "dc"])
 @pytest.mark.parametrize("p,Ma,Re", [(5, 6.0, 0.0), (7, 2.0, 0.0), (7, 2.0, 500.0), (7, 4.0, 0.0)])
 def test_residual_parity(p, Ma, Re, flux, flow):
     solver, q, mesh, gas, qo = _pair(p, 1.0, flow, flux, Re=Re, Ma=Ma)
