@@ -237,7 +237,6 @@ __device__ __forceinline__ void load_prim(const double* sP, int N3, int idx, Pri
     s.usq = sP[5 * N3 + idx];
 }
 
-
 __device__ __forceinline__ double sgn(double x) { return x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0); }
 
 // Reverse of the interface terms built on the face-averaged state: the matrix dissipation
@@ -467,9 +466,10 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
     }
     __syncthreads();
 
-    // ---- volume term.  ES-C: the pair reverse of adj_pairs_fix.cu; else the 3 N^2 lines of all directions at once, one per thread; direction l
-    // assigns its primitive cotangents to its own array (sB for l = 0, the two halves of the
-    // theta-bar buffer sT for l = 1, 2, which is free until the viscous part).  With several
+    // ---- volume term.  ES-C: the pair reverse of adj_pairs_fix.cu; else the 3 N^2 lines of all
+    // directions at once, one per thread; direction l assigns its primitive cotangents to its own
+    // array (sB for l = 0, the two halves of the theta-bar buffer sT for l = 1, 2, which is free until
+    // the viscous part).  With several
     // elements per CTA their lines are numbered consecutively over the CTA's threads, so that the
     // lines fill whole warps (a warp instruction costs the float64 pipe its full time whatever its
     // active lanes).
@@ -500,47 +500,45 @@ adj_main(const double* __restrict__ q, const double* __restrict__ lam, const dou
             const double* n2p = n1p + N3;
             // pair cotangent mu = S_ij (lt_j/w_j - lt_i/w_i) = SW_ij lt_j + SW_ji lt_i, half of the pair
             // term's 2 S_ij (...): the flux is linear in n, so it takes the sum of the two metrics
-            {
-                PBar acc[N];
+            PBar acc[N];
 #pragma unroll
-                for (int i = 0; i < N; ++i) acc[i] = PBar{0, 0, 0, 0, 0, 0};
+            for (int i = 0; i < N; ++i) acc[i] = PBar{0, 0, 0, 0, 0, 0};
 #pragma unroll
-                for (int i = 0; i < N - 1; ++i) {
-                    const int ii = base + i * st;
-                    Prim si;
-                    load_prim(sP, N3, ii, si);
-                    const double a0 = n0p[ii], a1 = n1p[ii], a2 = n2p[ii];
-                    double li[5];
+            for (int i = 0; i < N - 1; ++i) {
+                const int ii = base + i * st;
+                Prim si;
+                load_prim(sP, N3, ii, si);
+                const double a0 = n0p[ii], a1 = n1p[ii], a2 = n2p[ii];
+                double li[5];
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) li[v] = sL[v * N3 + ii];
+                for (int v = 0; v < 5; ++v) li[v] = sL[v * N3 + ii];
 #pragma unroll
-                    for (int j = i + 1; j < N; ++j) {
-                        const int jj = base + j * st;
-                        Prim sj;
-                        load_prim(sP, N3, jj, sj);
-                        double mu[5];
+                for (int j = i + 1; j < N; ++j) {
+                    const int jj = base + j * st;
+                    Prim sj;
+                    load_prim(sP, N3, jj, sj);
+                    double mu[5];
 #pragma unroll
-                        for (int v = 0; v < 5; ++v) mu[v] = fma(ops.SW[i][j], sL[v * N3 + jj], ops.SW[j][i] * li[v]);
-                        if constexpr (VF == kAdjDC) {
-                            // the pair term is 2 S_ij times the central flux (F(q_i).Ja_l(i) + F(q_j).Ja_l(j))/2
-                            // of the nodal contravariant fluxes (D applied to nodal fluxes)
-                            euler_flux_vjp(si, a0, a1, a2, mu, ph, acc[i]);
-                            euler_flux_vjp(sj, n0p[jj], n1p[jj], n2p[jj], mu, ph, acc[j]);
-                        } else {
-                            kg_flux_vjp(si, sj, a0 + n0p[jj], a1 + n1p[jj], a2 + n2p[jj], mu, ph, acc[i], acc[j]);
-                        }
+                    for (int v = 0; v < 5; ++v) mu[v] = fma(ops.SW[i][j], sL[v * N3 + jj], ops.SW[j][i] * li[v]);
+                    if constexpr (VF == kAdjDC) {
+                        // the pair term is 2 S_ij times the central flux (F(q_i).Ja_l(i) + F(q_j).Ja_l(j))/2
+                        // of the nodal contravariant fluxes (D applied to nodal fluxes)
+                        euler_flux_vjp(si, a0, a1, a2, mu, ph, acc[i]);
+                        euler_flux_vjp(sj, n0p[jj], n1p[jj], n2p[jj], mu, ph, acc[j]);
+                    } else {
+                        kg_flux_vjp(si, sj, a0 + n0p[jj], a1 + n1p[jj], a2 + n2p[jj], mu, ph, acc[i], acc[j]);
                     }
                 }
+            }
 #pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    const int ii = base + i * st;
-                    Bl[ii] = acc[i].rho;
-                    Bl[N3 + ii] = acc[i].u0;
-                    Bl[2 * N3 + ii] = acc[i].u1;
-                    Bl[3 * N3 + ii] = acc[i].u2;
-                    Bl[4 * N3 + ii] = acc[i].beta;
-                    Bl[5 * N3 + ii] = acc[i].usq;
-                }
+            for (int i = 0; i < N; ++i) {
+                const int ii = base + i * st;
+                Bl[ii] = acc[i].rho;
+                Bl[N3 + ii] = acc[i].u0;
+                Bl[2 * N3 + ii] = acc[i].u1;
+                Bl[3 * N3 + ii] = acc[i].u2;
+                Bl[4 * N3 + ii] = acc[i].beta;
+                Bl[5 * N3 + ii] = acc[i].usq;
             }
         }
     }

@@ -337,10 +337,11 @@ ESDC_HD FixScale fix_scale_dc(int Eu, int Eb, int En, int Ey, int Ez) {
 }
 
 // The viscous chain's exponents, known once theta is: w2..w4 = 2 beta u < 1/2 in units 2^(kb + ku), w5 =
-// -2 beta as beta itself; operator entries D_ij 2^-kD with row sums below 1.7, so theta (with its lift)
-// < 1.25, or < 1 once shifted left by sw (w2..w4) and sb (w5).  Then the contraction with the metric
-// < 0.94, velocity gradients A < 1.2, a quarter of their symmetric combination < 1.2 in the stress,
-// stress < 0.6, energy flux < 0.92, contravariant fluxes < 0.7.
+// -2 beta as beta itself; operator entries D_ij 2^-kD with row sums below 2.35, below 1.7 without the diagonal,
+// which the lift cancels at the end nodes and which is zero elsewhere, so theta (with its lift) < 1.25, or < 1 once
+// shifted left by sw (w2..w4) and sb (w5).  Then the contraction with the metric < 0.94, velocity gradients
+// A < 1.2, a quarter of their symmetric combination < 1.2 in the stress, stress < 0.6, energy flux < 0.92,
+// contravariant fluxes < 0.7.
 struct ViscScale {
     int ky, kz;              // mu RT/J and (kappa/R) RT^2/J
     int sg, su;              // the two parts of the velocity gradients
@@ -579,7 +580,7 @@ struct AdjScale {
     int kc;                      // energy coefficient
     int kd;                      // d(inv_gm1/(2 beta_ln))/d beta in Q60
     int kA;                      // inv_gm1/(2 beta_ln)
-    long long hF, h4;            // half a unit of sF, s4
+    long long hF;                // half a unit of sF
 };
 // E0, E1, E4: biased exponents that bound lambda/(J w)'s components; pmin, pmax: high words of the smallest and
 // largest pressure, whose difference bounds the relative pressure jump by 2^-dp (a step of the high word is at
@@ -614,7 +615,6 @@ ESDC_HD AdjScale adj_scale(const FixScale& s, int E0, int E1, int E4, int pmin, 
     t.kb = t.kc + t.kd;
     t.kp = kp + ep;
     t.hF = (1ll << t.sF) >> 1;
-    t.h4 = (1ll << t.s4) >> 1;
     return t;
 }
 
