@@ -776,13 +776,19 @@ cudaError_t launch_f64(const esdc_ctx* c, const double* q, double* dqdt, cudaStr
 // against wide form: N = 2 512 elements 36.0 -> 20.7 us, N = 3 512 32.9 -> 24.7, N = 4 64 30 -> 20, 216
 // 30.9 -> 24.7, 343 37.0 -> 35.0, 512 37.1 -> 39.1, N = 5 125 35.0 -> 26.8, 216 41.1 -> 41.8, N = 7 125
 // 53.4 -> 47.3, 343 121.5 -> 125.1; N = 6 and 8 gain nothing (37.0 and 63.6 us for up to one element per SM).
-constexpr int wide_upto(int n) { return n == 2 ? 6 : (n == 3 ? 4 : (n == 4 ? 2 : (n == 5 || n == 7 ? 1 : 0))); }
+// The instances with the optional interface terms keep fewer CTAs resident, so their line lies lower (bounded box,
+// normal against wide: N = 2 576 elements ES-C 0.89 of the time, 720 1.10, 900 1.16, DC 0.84, 1.09, 1.14, SF-KG 900
+// 39.1 -> 32.9 us; N = 3 448 elements 0.7, 576 1.06 to 1.11; N = 4 294 DC 31.9 -> 39.1 us, the others 0.8).
+constexpr int wide_upto(int n, int vf, bool xf) {
+    return n == 2 ? (xf && vf != kFluxKG ? 4 : 6)
+                  : (n == 3 ? (xf ? 3 : 4) : (n == 4 ? (xf && vf == kFluxDC ? 1 : 2) : (n == 5 || n == 7 ? 1 : 0)));
+}
 
 template <int N, int VF, bool XF>
 cudaError_t launch_n(const esdc_ctx* c, const double* q, double* dqdt, cudaStream_t s) {
     if (c->float64_form) return launch_f64<N, VF, XF>(c, q, dqdt, s);
-    if constexpr (wide_upto(N) > 0)
-        if (c->K <= (int64_t)wide_upto(N) * sm_count()) return launch_w<N, VF, XF, true>(c, q, dqdt, s);
+    if constexpr (wide_upto(N, VF, XF) > 0)
+        if (c->K <= (int64_t)wide_upto(N, VF, XF) * sm_count()) return launch_w<N, VF, XF, true>(c, q, dqdt, s);
     return launch_w<N, VF, XF, false>(c, q, dqdt, s);
 }
 
@@ -791,7 +797,7 @@ cudaError_t prepare_n(const esdc_ctx* c) {
     constexpr cudaFuncAttribute kAttr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     if (c->float64_form) return cudaFuncSetAttribute(rhs_f64<N, VF, XF>, kAttr, (int)(Cfg<N>::EPB * Cfg<N>::SM * sizeof(double)));
     const cudaError_t e = cudaFuncSetAttribute(rhs_fix_f64<N, VF, XF, false>, kAttr, (int)fix_smem<N, VF, false>());
-    if constexpr (wide_upto(N) > 0)
+    if constexpr (wide_upto(N, VF, XF) > 0)
         if (e == cudaSuccess) return cudaFuncSetAttribute(rhs_fix_f64<N, VF, XF, true>, kAttr, (int)fix_smem<N, VF, true>());
     return e;
 }
