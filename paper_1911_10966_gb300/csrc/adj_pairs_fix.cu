@@ -7,8 +7,10 @@
 // about fifty 60-bit products of 17.  Same mapping as the residual's pair loop (rhs_fix.cuh): one thread per
 // (node, direction), whole lines side by side in a warp, pair (i, i + k mod N) at cyclic distance k; the
 // partner's lambda/(J w) and the results for it travel by shuffle.  The flux is linear in the metric, so
-// S_ij multiplies n_i + n_j and the cotangent is the plain difference of lambda/(J w).  Elements outside the
-// fixed-point range (primitives as in the residual, or lambda/J beyond it) take the float64 reverse.
+// S_ij multiplies n_i + n_j and the cotangent is the plain difference of lambda/(J w).  Results are linear in
+// lambda, which may vary by orders within an element (quadrature weights alone by (w_mid/w_end)^2, 130 at p = 7):
+// each line takes it under its own largest value and shifts its sums back.  Elements outside the fixed-point range
+// (primitives as in the residual, or lambda/J beyond it) take the float64 reverse.
 #include <cuda_runtime.h>
 
 #include "adj_pair_f64.cuh"
@@ -54,6 +56,11 @@ struct AdjMeansF64 {
         beta_mean_f64(fx_join(ba), fx_join(bb), s.kb, hig, s.kA, kd, m);
     }
 };
+
+// x 2^-d on the exponent's bits; 0 below the normal range
+__device__ __forceinline__ double shift_down(double x, int d) {
+    return biased_exp(x) <= d ? 0.0 : __hiloint2double(__double2hiint(x) - (d << 20), __double2loint(x));
+}
 
 // The pair loop in float64 for a CTA with an element out of range: inputs still float64 in shared memory.  One
 // thread per line, the lines numbered consecutively over the threads: a float64 instruction costs its pipe 64
@@ -185,11 +192,6 @@ adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, cons
                 X[i] = fx_split(fx_from_double(sm[i], s.kn));
             }
             scale_inputs<kFluxESC>(sm + C::XP + own, X + C::XP + own, SL, s);
-#pragma unroll
-            for (int v = 0; v < 5; ++v) {
-                const int i = C::LT + v * SL + own;
-                X[i] = fx_split(fx_from_double(sm[i], (v == 0 ? ta.l0 : (v == 4 ? ta.l4 : ta.l1)) - ops.kW));
-            }
         }
         __syncthreads();
         const int lw = lane / N, i = lane - lw * N;
@@ -203,15 +205,28 @@ adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, cons
             const int c1 = li % N, c2 = li / N;
             double* se = smem + (size_t)e * C::SM;
             const Fx* Xe = reinterpret_cast<const Fx*>(se);
-            const Fx *XP = Xe + C::XP, *XN = Xe + C::XN + 3 * l * SL, *LT = Xe + C::LT;
+            const Fx *XP = Xe + C::XP, *XN = Xe + C::XN + 3 * l * SL;
             const FixScale& s = sScale[e];
             const AdjScale& ta = sAdj[e];
             const int ic = i < N ? i : 0, ii = line_slot<N>(l, ic, c1, c2);
             const PrimFx a = load_inputs<kFluxESC>(XP + ii, SL);
             const Fx na0 = XN[ii], na1 = XN[SL + ii], na2 = XN[2 * SL + ii], w = sW[ic];
-            long long lo[5];                     // lambda/(J w)
+            // lambda/(J w) in fixed point, shifted up by what the line's largest leaves free of the element's bound
+            double lt[5];
+            int up = 60;
 #pragma unroll
-            for (int v = 0; v < 5; ++v) lo[v] = fx_mul(LT[v * SL + ii], w);
+            for (int v = 0; v < 5; ++v) {
+                lt[v] = se[C::LT + v * SL + ii];
+                const int b = biased_exp(lt[v]);
+                if (b) up = min(up, sE[e][v == 0 ? 6 : (v == 4 ? 8 : 7)] - b - ops.WE[ic]);
+            }
+            const int mine = up;
+#pragma unroll
+            for (int k = 1; k < N; ++k) up = min(up, __shfl_sync(0xffffffffu, mine, (lw * N + (ic + k < N ? ic + k : ic + k - N)) & 31));
+            long long lo[5];
+#pragma unroll
+            for (int v = 0; v < 5; ++v)
+                lo[v] = fx_mul(fx_split(fx_from_double(lt[v], (v == 0 ? ta.l0 : (v == 4 ? ta.l4 : ta.l1)) - ops.kW - up)), w);
             PairBarFx acc = {0.0, 0.0, 0.0, 0.0, {0.0, 0.0, 0.0}, 0.0};
 #pragma unroll 1
             for (int k = 1; k <= N / 2; ++k) {
@@ -244,11 +259,11 @@ adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, cons
             }
             if (go) {
                 double* B = se + C::B + 6 * l * SL + ii;
-                B[0] = acc.xa;
+                B[0] = shift_down(acc.xa, up);
 #pragma unroll
-                for (int d = 0; d < 3; ++d) B[(1 + d) * SL] = acc.u[d];
-                B[4 * SL] = acc.ba;
-                B[5 * SL] = acc.c;
+                for (int d = 0; d < 3; ++d) B[(1 + d) * SL] = shift_down(acc.u[d], up);
+                B[4 * SL] = shift_down(acc.ba, up);
+                B[5 * SL] = shift_down(acc.c, up);
             }
         }
     } else {

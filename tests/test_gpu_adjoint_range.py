@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import esdc_oracle as O
-from tests.gpu_common import normwise_errors
+from tests.gpu_common import EPS64, make_pair, normwise_errors
 from tests.test_gpu_fixed_point import _case
 
 pytestmark = pytest.mark.gpu
@@ -58,3 +58,21 @@ def test_nonfinite_cotangent_stays_in_its_neighbourhood(p, bad):
     assert not torch.isfinite(gb[0]).all()
     assert torch.isfinite(gb[same]).all()
     assert max(normwise_errors(gb[same], g[same].cpu())) <= 1e-10
+
+
+@pytest.mark.parametrize("p", [2, 3, 4, 5, 6, 7])
+def test_one_large_cotangent_leaves_other_lines_alone(p):
+    """Inviscid, without dissipation, the gradient at an element's interior nodes takes the cotangents of its three
+    lines only: one of 1e10 at a corner node, on none of them, must not cost it bits.  Bound: 64 N eps of the largest
+    interior value (3 N pair terms of about ten roundings), a hundred times that for density and energy (differences
+    of pressure terms)."""
+    solver, qg, mesh, gas, qo = make_pair(p, (3, 2, 2), warp=0.1, seed=3, Re=0.0, dissipation=False, noise=2e-2)
+    lam = _lam(qo).cuda()
+    g = solver.rhs_vjp(qg, lam)
+    big = lam.clone()
+    big[:, :, 0, 0, 0] = 1e10
+    inner = (slice(None), slice(None)) + (slice(1, -1),) * 3
+    e = normwise_errors(solver.rhs_vjp(qg, big)[inner], g[inner].cpu())
+    print("interior", ["%.1e" % x for x in e])
+    assert max(e[1:4]) <= 64 * (p + 1) * EPS64, e
+    assert max(e) <= 6400 * (p + 1) * EPS64, e
