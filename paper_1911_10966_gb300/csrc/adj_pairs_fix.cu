@@ -131,7 +131,7 @@ adj_pairs_fix(const double* __restrict__ q, const double* __restrict__ lam, cons
     Fx* X = reinterpret_cast<Fx*>(sm);
     const int own = slot<N>(node % N, (node / N) % N, node / N2);
     for (int i = t; i < EPB * NE; i += C::THREADS)
-        sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? metric_exponent(kn[(int64_t)blockIdx.x * EPB + i / NE], kAdjStretch) : 0;
+        sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? kn[(int64_t)blockIdx.x * EPB + i / NE] : 0;
     for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
     for (int i = t; i < N; i += C::THREADS) sW[i] = ops.WB[i];
     __syncthreads();

@@ -94,23 +94,18 @@ struct HostSetup {
     std::vector<double> geom;            // [K][10][N^3]: J, Ja_lm (l-major)
     std::vector<double> nsurf;           // [K][6][3][N^2] surface metrics (optimized metrics only)
     std::vector<int32_t> nbr;            // [K][6]
-    std::vector<int32_t> kn;             // [K] exponent of the largest metric entry and stretch (metric_code)
+    std::vector<int32_t> kn;             // [K] biased exponent of the largest metric entry, or kStretched
     double h_min = 0.0;
 };
 
-// Stretch of an element: the ratio between the largest metric entries of the three coordinates, max over
-// directions and nodes of |Ja_lm|, m = 1..3; beyond kRhsStretch an element's residual, beyond kAdjStretch its
-// adjoint is evaluated in float64.  One exponent serves all nine entries of an element, so the fluxes' errors are
-// relative to the largest, where float64's follow each coordinate's own.
-// Errors against extended precision, fixed point over float64, axis-aligned elements, worst variable and flow of
-// p = 3, 4 and 7: 1.0 to 1.1 at ratio 2, 1.7 at 4, 3.5 at 8, 200 at 1000, more in the viscous terms.
-// The reverse pairs keep exponents of their own: 0.1 at ratio 1, 0.2 at 4, 0.7 to 1.1 at 16, 15 at 1000 (p = 3).
-constexpr int kRhsStretch = 1, kAdjStretch = 3;
-// An element's code: the biased exponent E of its largest metric entry, and the smallest s >= 0 with that ratio at
-// most 1.025 2^s (a little slack for 2 : 1 boxes).
-constexpr int metric_code(int E, int s) { return E + (s << 12); }
-// the exponent again, or one out of range (fix_range_ok) where the stretch is above `most`
-constexpr int metric_exponent(int code, int most) { return (code >> 12) > most ? 2047 : code & 4095; }
+// Largest stretch of an element for which it is evaluated in fixed point: the ratio between the largest metric
+// entries of the three coordinates, max over directions and nodes of |Ja_lm|, m = 1..3 (2 : 1 boxes and a little
+// slack).  One exponent serves all nine entries of an element, so errors are relative to the largest, where float64's
+// follow each coordinate's own.  Errors against extended precision, fixed point over float64, axis-aligned elements,
+// worst variable and flow: residual of p = 3, 4 and 7 0.7 (ES-C) to 0.98 (SF-KG) at ratio 2, 1.7 at 4, 3.5 at 8, 200
+// at 1000, more in the viscous terms; gradient of the kinetic energy, p = 3, 1.1 at 1, 1.3 at 2, 2.5 at 4.
+constexpr double kMaxStretch = 2.05;
+constexpr int kStretched = 2047;         // beyond every exponent that fix_range_ok admits
 
 int lgl(int p, double* xi, double* w);
 int build_operators(int p, HostSetup& hs);

@@ -11,8 +11,9 @@
 // 30-bit limb, or the sum of two (so an addition needs no carry).  What a Q60 number stands for is
 // v 2^k with an exponent k that is the same for a whole element: the inputs are scaled by the largest
 // exponent of their kind in the element, and every intermediate's exponent follows from theirs.  An
-// element whose density or beta spans more than kMaxSpread binary exponents, or whose state is not
-// finite and positive, is evaluated in float64 instead (fix_range_ok).
+// element whose density or beta spans more than kMaxSpread binary exponents, whose state is not finite and
+// positive (fix_range_ok), whose metric terms are stretched (kMaxStretch) or whose flow is fast (fix_speed_ok)
+// is evaluated in float64 instead.
 #pragma once
 
 #include <cstdint>
@@ -379,9 +380,9 @@ ESDC_HD bool fix_range_ok(int Er, int Er0, int Eu, int Eb, int Eb0, int En) {
 // Where the kinetic part sets the momentum fluxes' exponent, a velocity component much smaller than the others
 // leaves its own momentum flux, and the pressure's in it, few bits; and the energy flux is the difference of
 // larger parts.  u0, u1, u2: largest |u_m| of the element (speed_code), Eb0 as above; k is ka - kb of fix_scale.
-// Errors against extended precision, fixed point over float64, worst variable of p = 3, 4, 7 and 15 with the flow
-// along one axis: 0.88 at k = 1 (Mach 0.5), 0.9 to 1.5 at 2 (0.7, 0.85), 1.8 at 3 (1), 8 at 5 (2); in all three:
-// 0.8 at k = 3 (1), 1.0 at 5 (2), p = 15 1.3, 1.2 at 7 (4).  Hence `most`, 5, or 3 at p = 15.
+// Errors against extended precision, fixed point over float64, worst variable of p = 3, 4, 7 and 15, ES-C and SF-KG,
+// with the flow along one axis: 0.7 to 1.04 at k = 1 (Mach 0.5), 0.9 to 1.5 at 2 (0.7, 0.85), 2.5 at 3 (1), 8 at 5
+// (2); in all three: 0.8 at k = 3 (1), 1.0 at 5 (2), p = 15 1.3, 1.2 at 7 (4).  Hence `most`, 5, or 3 at p = 15.
 ESDC_HD int speed_code(double u) { return (double_hi(u) & 0x7fffffff) >> 8; }      // biased exponent, 12 bits below it
 ESDC_HD int speed_exponent(int u0, int u1, int u2) { return fx_max(u0, fx_max(u1, u2)) >> 12; }
 ESDC_HD bool fix_speed_ok(int u0, int u1, int u2, int Eb0, int most) {

@@ -62,7 +62,7 @@ bool float64_form(const esdc_ctx* c, const int32_t* kn) {
     int64_t out = 0, blocks = (c->K + epb - 1) / epb;
     for (int64_t b = 0; b < blocks; ++b) {
         bool s = false;
-        for (int64_t e = b * epb; e < c->K && e < (b + 1) * epb; ++e) s = s || metric_exponent(kn[e], kRhsStretch) == 2047;
+        for (int64_t e = b * epb; e < c->K && e < (b + 1) * epb; ++e) s = s || kn[e] == kStretched;
         out += s;
     }
     return 8 * out > 7 * blocks;

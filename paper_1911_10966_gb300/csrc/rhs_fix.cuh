@@ -20,9 +20,10 @@
 //
 // Bound: multiply (8 lanes per clock and scheduler for a 32 x 32 -> 64 product) and shift/logic (16) pipes
 // in phases 1 and 3, the float64 pipe (half a lane) in 0 and 2.  Against the all-float64 kernel, which
-// kept the float64 pipe 87% busy, per viscous residual of the Taylor-Green flow: 8.59 -> 2.86 ms at p = 7
-// on 20^3 elements, 0.92 -> 0.31 ms at p = 4 on 16^3, 2.58 -> 1.02 ms at p = 2 on 41 x 37 x 39.  Its error
-// against extended precision is smaller in every variable and degree tried.
+// kept the float64 pipe 87% busy, per viscous residual of the Taylor-Green flow: 8.59 -> 2.92 ms at p = 7
+// on 20^3 elements, 0.92 -> 0.31 ms at p = 4 on 16^3, 2.58 -> 1.00 ms at p = 2 on 41 x 37 x 39.  Its error
+// against extended precision, worst variable over flows along one axis and all, is 0.6 to 1.04 of the float64
+// kernel's (kMaxStretch, fix_speed_ok; DC's energy at Mach 2 1.12).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -281,7 +282,7 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     const int own_slot = slot<N>(i1, i2, i3);
     const int64_t eoff = el * 5 * N3;
     for (int i = t; i < EPB * NE; i += C::THREADS)
-        sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? metric_exponent(kn[(int64_t)blockIdx.x * EPB + i / NE], kRhsStretch) : 0;
+        sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? kn[(int64_t)blockIdx.x * EPB + i / NE] : 0;
     if constexpr (VF == kFluxDC)
         for (int i = t; i < EPB * 15; i += C::THREADS) sF[i / 15][i % 15] = 0;
     if (t < EPB) sMag[t][0] = sMag[t][1] = 0;

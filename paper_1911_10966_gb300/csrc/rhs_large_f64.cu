@@ -374,7 +374,7 @@ lg_volume_fix(const double* __restrict__ q, const double* __restrict__ geom, con
     }
     block_max<true>(sE, 0, E, lane);
     __syncthreads();
-    if (metric_exponent(kn[el], kRhsStretch) == 2047 || !rhs_range_ok(sE, 3)) {
+    if (kn[el] == kStretched || !rhs_range_ok(sE, 3)) {
         __syncthreads();
         plane_out_of_range<VF>(sm, q, geom, nbr, fnorm, rl, th, K, ops, ph);
         return;

@@ -418,7 +418,7 @@ double element_min_edge(int N, const double* xyz) {
 }  // namespace
 
 // HostSetup::kn of one element: g its metric rows [9][N3], ns its surface metrics [6][3][N2] or null
-static int32_t element_metric_code(int N, const double* g, const double* ns) {
+static int32_t metric_exponent(int N, const double* g, const double* ns) {
     const int N2 = N * N, N3 = N2 * N;
     double c[3] = {0.0, 0.0, 0.0};
     for (int m = 0; m < 3; ++m) {
@@ -428,10 +428,9 @@ static int32_t element_metric_code(int N, const double* g, const double* ns) {
             for (int i = 0; i < N2; ++i) c[m] = std::max(c[m], std::fabs(ns[(3 * f + m) * N2 + i]));
     }
     const double hi = std::max(c[0], std::max(c[1], c[2])), lo = std::min(c[0], std::min(c[1], c[2]));
-    int e, s = 0;
+    int e;
     std::frexp(hi, &e);
-    for (double r = 1.025 * lo; s < 1000 && !(hi <= r); r *= 2.0) ++s;
-    return metric_code(std::max(e + 1022, 0), s);
+    return hi <= kMaxStretch * lo ? std::max(e + 1022, 0) : kStretched;
 }
 
 int build_geometry(const esdc_setup_t& s, const double* xyz, HostSetup& hs, std::string& err) {
@@ -460,7 +459,7 @@ int build_geometry(const esdc_setup_t& s, const double* xyz, HostSetup& hs, std:
                                                                    &hs.nsurf[(size_t)e * 6 * 3 * N2])
                                       : element_geometry(hs.D, N, x, &hs.geom[(size_t)e * 10 * N3]);
                 if (!good) bad[t] = 1;
-                hs.kn[e] = element_metric_code(N, &hs.geom[((size_t)e * 10 + 1) * N3], opt ? &hs.nsurf[(size_t)e * 18 * N2] : nullptr);
+                hs.kn[e] = metric_exponent(N, &hs.geom[((size_t)e * 10 + 1) * N3], opt ? &hs.nsurf[(size_t)e * 18 * N2] : nullptr);
                 hmin[t] = std::min(hmin[t], element_min_edge(N, x));
             }
         });
