@@ -55,7 +55,9 @@ struct CfgA {
     static constexpr int SM = 36 * N3 + TSZ + 24 * N2;
     // resident CTAs the register allocation is sized for: four at N = 4, 5 hold 512 elements in one wave (VJP at
     // p = 4, three against four: 8^3 elements 231 -> 218 us, 16^3 1.379 -> 1.375 ms), two at N = 6 (14^3 1.89 ->
-    // 1.84 ms; two at N = 7 lose, 1.87 -> 1.88 ms on 12^3)
+    // 1.84 ms; two at N = 7 lose, 1.87 -> 1.88 ms on 12^3).  SF-KG and DC, whose pair loop is in here, spill more
+    // (0.9 to 1.4 KB at p = 5) and gain as much: SF-KG p = 4 8^3 264 -> 249 us, p = 5 14^3 1.98 -> 1.94 ms, DC 258 ->
+    // 243 us, 1.92 -> 1.86 ms; within 1% on other sizes, SF-KG p = 5 on 5^3 128 -> 132 us
     static constexpr int MINB = (N == 4 || N == 5) ? 4 : (N == 6 ? 2 : 1);
 };
 
