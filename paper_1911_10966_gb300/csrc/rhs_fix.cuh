@@ -13,7 +13,7 @@
 //      k = 1..N/2 the thread of node i evaluates the pair (i, i + k mod N), so that each pair is
 //      evaluated once; S_ij f is summed in registers on one side and by a shuffle on the other.  DC: the
 //      nodal contravariant fluxes per node in float64, then one thread per line and variable, each line in
-//      fixed point under the largest exponent of its direction and variable in the element.
+//      fixed point under its own largest exponent.
 //   2. interface: one thread per face node; two-point flux in fixed point (DC: float64), dissipation in float64.
 //   3. viscous: lines of w for theta_a = D_a w + lift (one thread per line and variable, the operator
 //      from the constant bank), one thread per node for the fluxes, lines again for the divergence.
@@ -265,7 +265,6 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     constexpr int N2 = C::N2, N3 = C::N3, EPB = C::EPB, SL = C::SL, NP = C::NP, NE = VF == kFluxKG ? 12 : 10;
     extern __shared__ double smem[];
     __shared__ int sE[EPB][NE];                  // largest exponents (of 4096 - E for the smallest)
-    __shared__ int sF[VF == kFluxDC ? EPB : 1][15];       // DC: of the nodal fluxes, by direction and variable
     __shared__ FixScale sScale[EPB];
     __shared__ unsigned sMag[EPB][2];            // magnitude bits of theta: w2..w4, w5
     __shared__ Fx sS[(N / 2) * N];
@@ -283,8 +282,6 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     const int64_t eoff = el * 5 * N3;
     for (int i = t; i < EPB * NE; i += C::THREADS)
         sE[i / NE][i % NE] = i % NE == 5 && i / NE < n_el ? kn[(int64_t)blockIdx.x * EPB + i / NE] : 0;
-    if constexpr (VF == kFluxDC)
-        for (int i = t; i < EPB * 15; i += C::THREADS) sF[i / 15][i % 15] = 0;
     if (t < EPB) sMag[t][0] = sMag[t][1] = 0;
     for (int i = t; i < (N / 2) * N; i += C::THREADS) sS[i] = ops.SF[i / N][i % N];
     for (int i = t; i < N; i += C::THREADS) sW[i] = ops.winv[i];
@@ -355,7 +352,6 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
         if constexpr (VF == kFluxDC) {
             // nodal contravariant fluxes Ftilde_l
             const double* pi = sm + C::XP + own_slot;
-            int EF[15];
 #pragma unroll
             for (int l = 0; l < 3; ++l) {
                 const double* n = sm + C::XN + 3 * l * SL + own_slot;
@@ -363,12 +359,8 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
                 euler_flux(2.0 * pi[0], 2.0 * pi[SL], 2.0 * pi[2 * SL], 2.0 * pi[3 * SL], 2.0 * pi[6 * SL], pi[5 * SL], n[0], n[SL],
                            n[2 * SL], f);
 #pragma unroll
-                for (int v = 0; v < 5; ++v) {
-                    sm[C::R + (5 * l + v) * SL + own_slot] = f[v];
-                    EF[5 * l + v] = biased_exp(f[v]);
-                }
+                for (int v = 0; v < 5; ++v) sm[C::R + (5 * l + v) * SL + own_slot] = f[v];
             }
-            block_max<EPB == 1 || N3 % 32 == 0>(sF[el_loc], el_loc, EF, lane);
         }
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
@@ -392,19 +384,26 @@ rhs_fix_f64(const double* __restrict__ q, double* __restrict__ dqdt, const doubl
     // ---- 1. volume flux differencing
     if constexpr (VF == kFluxDC) {
         // the nodal fluxes' differences along the lines, sum_j S_ij (F_i + F_j) with the own flux left out, which at
-        // the end nodes is half the interface flux's own part; in fixed point under the largest exponent of the
-        // direction's and variable's fluxes, in place
+        // the end nodes is half the interface flux's own part; in fixed point under the line's largest exponent, in
+        // place
 #pragma unroll 1
         for (int id = t; id < n_el * 15 * N2; id += C::THREADS) {
             const int e = id / (15 * N2), r = id - e * 15 * N2;
             const int lv = r / N2, li = r - lv * N2;
             const int l = lv / 5, c1 = li % N, c2 = li / N;
             double* R = smem + (size_t)e * C::SM + C::R + lv * SL;
-            const int k = sF[e][lv] - 1021;
+            double f[N];
+            int k = 0;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                f[j] = R[line_slot<N>(l, j, c1, c2)];
+                k = max(k, biased_exp(f[j]));
+            }
+            k -= 1021;
             Fx x[N];
             long long out[N];
 #pragma unroll
-            for (int j = 0; j < N; ++j) x[j] = fx_split(fx_from_double(R[line_slot<N>(l, j, c1, c2)], k));
+            for (int j = 0; j < N; ++j) x[j] = fx_split(fx_from_double(f[j], k));
             line_product<N>(x, ops.MF, out);
 #pragma unroll
             for (int j = 0; j < N; ++j) R[line_slot<N>(l, j, c1, c2)] = -ops.winv[j] * fx_to_double(out[j], k);
